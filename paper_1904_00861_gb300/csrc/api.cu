@@ -609,8 +609,9 @@ int allocate(dtsph_ctx *c, const int64_t *nf)
     A(B.cell_start, (size_t)B.ncell + 1) A(B.scan_tmp, (size_t)B.ncell / 4096 + 2)
     A(B.vk[0], nd) A(B.vk[1], nd)
     A(B.pcount, n) A(B.pj, npair) A(B.pjt, (size_t)n * list_stride(B.K))
+    A(B.off, n)
     if (B.fp32c) {
-        A(B.off, n) A(B.nb32[0], n) A(B.nb32[1], n) A(B.pc32, npair)
+        A(B.nb32[0], n) A(B.nb32[1], n) A(B.pc32, npair)
     } else {
         A(B.nb64[0], n) A(B.nb64[1], n) A(B.pc64, npair)
     }

@@ -275,10 +275,11 @@ __global__ void __launch_bounds__(kBlock) k_permute_a_to_b(Buffers B)
     }
     const double p = B.pn_a[o];
     B.pn_b[s] = p;
+    // (the FP64 path reads the offsets in the list builders only)
+    const int inst = B.inst_of[s];
+    B.off[s] = SAME ? cell_offset_near(B.geo[inst], cell - B.inst[inst].cell_off, B.x_b, n, s, g >= (uint32_t)B.nf)
+                    : cell_offset(B.geo[inst], cell - B.inst[inst].cell_off, B.x_b, n, s, g >= (uint32_t)B.nf);
     if (B.fp32c) {
-        const int inst = B.inst_of[s];
-        B.off[s] = SAME ? cell_offset_near(B.geo[inst], cell - B.inst[inst].cell_off, B.x_b, n, s, g >= (uint32_t)B.nf)
-                        : cell_offset(B.geo[inst], cell - B.inst[inst].cell_off, B.x_b, n, s, g >= (uint32_t)B.nf);
         B.nb32[1][s] = make_float4((float)v[0], (float)v[1], (float)v[2], (float)p);
     } else {
         B.nb64[1][s] = make_double4_32a(v[0], v[1], v[2], p);
@@ -318,9 +319,9 @@ __global__ void __launch_bounds__(kBlock) k_permute_b_to_a(Buffers B)
     }
     if (wall) store_wall_velocity(B, s, u);
     const double ph = B.ph0_b[o];
+    const int inst = B.inst_of[s];
+    B.off[s] = cell_offset(B.geo[inst], cell - B.inst[inst].cell_off, B.xp_a, n, s, g >= (uint32_t)B.nf);
     if (B.fp32c) {
-        const int inst = B.inst_of[s];
-        B.off[s] = cell_offset(B.geo[inst], cell - B.inst[inst].cell_off, B.xp_a, n, s, g >= (uint32_t)B.nf);
         B.nb32[0][s] = make_float4((float)v[0], (float)v[1], (float)v[2], (float)ph);
     } else {
         B.nb64[0][s] = make_double4_32a(v[0], v[1], v[2], ph);

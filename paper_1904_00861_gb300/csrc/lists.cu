@@ -2,26 +2,28 @@
 // particles with neighbour updates, 3h + list_skin for lists reused at the next
 // r^n) of every slot, from the cell binning.
 //
-// One warp per home cell, the candidates in the lanes. The warp stages the
-// particles of the 3^D surrounding cells in shared memory, in the order rows
-// (dz, dy), then dx, then slot, each tagged with its list entry (slot, cell
-// shift code, wall flag); then, for every chunk of 32 staged candidates (one per
-// lane) and every home particle in turn, each lane tests its candidate against
-// that home particle. A ballot ranks the hits, which join the home particle's
-// list as one contiguous run, so a store of the warp touches one or two sectors
-// instead of one per lane. The lists are written per slot (slot s at s Ks + k,
-// Ks = K rounded up to 8); the state-n, pair-cache and uncached-loop passes read
-// them there, and only the pass of particles moving in pseudo-time gets a copy
-// sliced by warp (k_list_slice: entry k of slot s at ((s/32) K + k) 32 + s%32).
-// Large 2D problems on the FP32C path take the row-segment builder
-// (k_nlist_rows2_f32), 3D ones k_nlist_cells3_f32; every builder gives the same
-// lists in the same order.
+// Two builders, same lists in the same order:
+//  - k_nlist_home: the home particles in the lanes (a row segment of three cells
+//    in 2D, a cell in 3D), the candidates broadcast from shared memory;
+//  - k_nlist_cells2, small 2D problems: one warp per home cell, the candidates in
+//    the lanes. The warp stages the particles of the 9 surrounding cells in shared
+//    memory, in the order rows (dy), then dx, then slot, each tagged with its list
+//    entry (slot, cell shift code, wall flag); then, for every chunk of 32 staged
+//    candidates (one per lane) and every home particle in turn, each lane tests its
+//    candidate against that home particle. A ballot ranks the hits, which join the
+//    home particle's list as one contiguous run.
+// The lists are written per slot (slot s at s Ks + k, Ks = K rounded up to 8), each
+// row filled up to a multiple of four with entries of the slot itself; the
+// state-n, pair-cache and uncached-loop passes read them there, and only the pass
+// of particles moving in pseudo-time gets a copy sliced by warp (k_list_slice:
+// entry k of slot s at ((s/32) K + k) 32 + s%32).
 //
 // The tests are those of the neighbour definition: FP64 positions, squares
-// summed in axis order without FMA, minimum image on periodic axes; the FP32C
-// path tests the FP32 separation from cell offsets, (o_i - shift s) - o_j as the
-// pair kernels form it, and takes the FP64 test only inside a thin band around
-// the cutoff, so both paths give the same sets, in the same order.
+// summed in axis order without FMA, minimum image on periodic axes. Both
+// precisions first test the FP32 separation from cell offsets and take the FP64
+// test only inside a thin band around the cutoff, so both give the same sets, in
+// the same order.
+#include "f32x2.cuh"
 #include "geometry.cuh"
 
 namespace dtsph {
@@ -54,23 +56,16 @@ __device__ __forceinline__ int cell_instance(const Buffers &B, int c)
     return lo;
 }
 
-// A staged candidate: FP32C its cell offset (.w = list entry bits), FP64 its
-// position (.w = list entry bits).
-template <bool F32> struct Staged;
-template <> struct Staged<true> { using type = float4; };
-template <> struct Staged<false> { using type = double4_32a; };
-
-template <int D, bool F32>
-__global__ void __launch_bounds__(kBlock) k_nlist_cells(Buffers B, const double *__restrict__ xpos,
-                                                        const uint32_t *__restrict__ gid, uint32_t *__restrict__ lists,
-                                                        int Ks)
+// 2D lists of small problems, one warp per cell with the candidates in the lanes
+// (see the top of the file).
+__global__ void __launch_bounds__(kBlock) k_nlist_cells2(Buffers B, const double *__restrict__ xpos,
+                                                         uint32_t *__restrict__ lists, int Ks)
 {
     if (skip_relist(B)) return;   // (the step graph: relisting or not)
-    constexpr int NC = D == 3 ? 27 : 9;                 // surrounding cells
-    constexpr int CH = F32 ? 256 : 128;                 // staged candidates per round
-    using S = typename Staged<F32>::type;
-    __shared__ S cand[kWarpsPerBlock][CH];
-    __shared__ S home[kWarpsPerBlock][kWarp];
+    constexpr int NC = 9;                               // surrounding cells
+    constexpr int CH = 256;                             // staged candidates per round
+    __shared__ float4 cand[kWarpsPerBlock][CH];         // cell offsets, .w = list entry bits
+    __shared__ float4 home[kWarpsPerBlock][kWarp];
     __shared__ int tpre[kWarpsPerBlock][NC + 1];        // candidates before surrounding cell t
     __shared__ int tbeg[kWarpsPerBlock][NC];            // first slot of surrounding cell t
     constexpr unsigned full = 0xffffffffu;
@@ -81,33 +76,32 @@ __global__ void __launch_bounds__(kBlock) k_nlist_cells(Buffers B, const double 
     const int inst = cell_instance(B, c);
     const int cell_off = B.inst[inst].cell_off;
     const Geom &G = B.geo[inst];
-    const int nx = G.nc[0], ny = G.nc[1], nz = G.nc[2];
+    const int nx = G.nc[0], ny = G.nc[1];
     const int lc = c - cell_off;
-    if (lc >= nx * ny * nz) return;                     // the instance's empty sentinel cell
+    if (lc >= nx * ny) return;                          // the instance's empty sentinel cell
     const int *start = B.cell_start + cell_off;
     const int hb = start[lc], he = start[lc + 1];
     if (hb == he) return;
-    const int cx = lc % nx, cy = (lc / nx) % ny, cz = lc / (nx * ny);
-    const float sf[3] = {G.s_f[0], G.s_f[1], G.s_f[2]};
+    const int cx = lc % nx, cy = lc / nx;
+    const float sf[3] = {G.s_f[0], G.s_f[1], 0.f};
     const float rc2_lo = G.rc2_lo, rc2_hi = G.rc2_hi;
     const double rc2 = G.rc2;
-    // FP32C: squared distance from the home cell beyond which no home particle
-    // can reach a candidate (the band's top, with a margin far above the
-    // rounding of FP32 offsets, which lie in [0, s])
+    // squared distance from the home cell beyond which no home particle can reach
+    // a candidate (the band's top, with a margin far above the rounding of FP32
+    // offsets, which lie in [0, s])
     const float box_cut2 = rc2_hi * 1.001f;
     const int n = B.n, K = B.K;
-    // the surrounding cells side by side: lane t takes shift code
-    // (dx + 1) + 3 (dy + 1) + 9 (dz + 1), dz = 0 in 2D (empty when off a closed edge)
+    // the surrounding cells side by side: lane t takes shift code (dx + 1) +
+    // 3 (dy + 1) (+ 9: dz = 0); empty when off a closed edge
     int m = 0;
     if (lane < NC) {
-        const int dx = lane % 3 - 1, dy = (lane / 3) % 3 - 1, dz = D == 3 ? lane / 9 - 1 : 0;
-        int x = cx + dx, y = cy + dy, z = cz + dz;
+        const int dx = lane % 3 - 1, dy = lane / 3 - 1;
+        int x = cx + dx, y = cy + dy;
         bool ok = true;
         if (x < 0 || x >= nx) { if (G.periodic[0]) x = x < 0 ? x + nx : x - nx; else ok = false; }
         if (y < 0 || y >= ny) { if (G.periodic[1]) y = y < 0 ? y + ny : y - ny; else ok = false; }
-        if (D == 3 && (z < 0 || z >= nz)) { if (G.periodic[2]) z = z < 0 ? z + nz : z - nz; else ok = false; }
         if (ok) {
-            const int nc = (z * ny + y) * nx + x;
+            const int nc = y * nx + x;
             const int jb = start[nc];
             m = start[nc + 1] - jb;
             tbeg[w][lane] = jb;
@@ -128,58 +122,33 @@ __global__ void __launch_bounds__(kBlock) k_nlist_cells(Buffers B, const double 
     for (int h0 = hb; h0 < he; h0 += kWarp) {
         const int nh = min(kWarp, he - h0);
         // the home particles of this round, one per lane, into shared memory
-        if (lane < nh) {
-            const int s = h0 + lane;
-            if constexpr (F32) {
-                home[w][lane] = B.off[s];
-            } else {
-                S q;
-                q.x = xpos[s];
-                q.y = xpos[(size_t)n + s];
-                q.z = D == 3 ? xpos[2 * (size_t)n + s] : 0.0;
-                q.w = 0.0;
-                home[w][lane] = q;
-            }
-        }
+        if (lane < nh) home[w][lane] = B.off[h0 + lane];
         int cnt = 0;                                    // list length of home particle h0 + lane
         int t = 0;                                      // surrounding cell of the next fill position
         for (int c0 = 0; c0 < total; c0 += CH) {
             const int span = min(total - c0, CH);
             // fill: stream position p is candidate p - tpre[t] of surrounding
-            // cell t. FP32C drops, for the whole warp, a candidate farther than
-            // the cutoff from every point of the home cell (the outer parts of
-            // the edge and corner cells); the others keep their order
+            // cell t; a candidate farther than the cutoff from every point of the
+            // home cell (the outer parts of the edge and corner cells) is dropped
+            // for the whole warp; the others keep their order
             int take = 0;
             for (int q0 = 0; q0 < span; q0 += kWarp) {
                 const int q = q0 + lane;
                 bool keep = false;
-                S e;
+                float4 e;
                 if (q < span) {
                     const int p = c0 + q;
                     while (tpre[w][t + 1] <= p) ++t;
                     const int j = tbeg[w][t] + (p - tpre[w][t]);
-                    const int code = D == 3 ? t : t + 9;
-                    const int dx = t % 3 - 1, dy = (t / 3) % 3 - 1, dz = D == 3 ? t / 9 - 1 : 0;
-                    if constexpr (F32) {
-                        const float4 oj = B.off[j];
-                        e = oj;
-                        e.w = __uint_as_float(list_entry((uint32_t)j, code, oj.w != 0.f));
-                        const float ex = __fadd_rn(oj.x, (float)dx * sf[0]);
-                        const float ey = __fadd_rn(oj.y, (float)dy * sf[1]);
-                        const float ez = D == 3 ? __fadd_rn(oj.z, (float)dz * sf[2]) : 0.f;
-                        const float bx = fmaxf(fmaxf(-ex, ex - sf[0]), 0.f);
-                        const float by = fmaxf(fmaxf(-ey, ey - sf[1]), 0.f);
-                        const float bz = D == 3 ? fmaxf(fmaxf(-ez, ez - sf[2]), 0.f) : 0.f;
-                        keep = bx * bx + by * by + bz * bz < box_cut2;
-                    } else {
-                        e.x = xpos[j];
-                        e.y = xpos[(size_t)n + j];
-                        e.z = D == 3 ? xpos[2 * (size_t)n + j] : 0.0;
-                        // entry bits in .w, the wall flag from the caller index
-                        e.w = __longlong_as_double(
-                            (long long)list_entry((uint32_t)j, code, gid[j] >= (uint32_t)B.nf));
-                        keep = true;
-                    }
+                    const int dx = t % 3 - 1, dy = t / 3 - 1;
+                    const float4 oj = B.off[j];
+                    e = oj;
+                    e.w = __uint_as_float(list_entry((uint32_t)j, t + 9, oj.w != 0.f));
+                    const float ex = __fadd_rn(oj.x, (float)dx * sf[0]);
+                    const float ey = __fadd_rn(oj.y, (float)dy * sf[1]);
+                    const float bx = fmaxf(fmaxf(-ex, ex - sf[0]), 0.f);
+                    const float by = fmaxf(fmaxf(-ey, ey - sf[1]), 0.f);
+                    keep = bx * bx + by * by < box_cut2;
                 }
                 const unsigned bal = __ballot_sync(full, keep);
                 if (keep) cand[w][take + __popc(bal & lt)] = e;
@@ -188,48 +157,27 @@ __global__ void __launch_bounds__(kBlock) k_nlist_cells(Buffers B, const double 
             __syncwarp();
             for (int q0 = 0; q0 < take; q0 += kWarp) {
                 const bool valid = q0 + lane < take;
-                S e;
-                if (valid) e = cand[w][q0 + lane];
+                float4 e;
                 uint32_t ej = kNoParticle;
-                if constexpr (F32) {
-                    if (valid) ej = __float_as_uint(e.w);
-                } else {
-                    if (valid) ej = (uint32_t)__double_as_longlong(e.w);
+                if (valid) {
+                    e = cand[w][q0 + lane];
+                    ej = __float_as_uint(e.w);
                 }
                 const int j = entry_slot(ej);
                 int dx, dy, dz;
                 decode_shift(entry_code(ej), dx, dy, dz);
                 for (int h = 0; h < nh; ++h) {
                     const int s = h0 + h;
-                    bool in;
-                    if constexpr (F32) {
-                        const float4 oi = home[w][h];
-                        float f0, f1, f2;
-                        const float q2 = sep32<D>(shifted_offset<D>(oi, dx, dy, dz, sf), e, f0, f1, f2);
-                        const bool cand_ok = valid && j != s;
-                        in = cand_ok && q2 < rc2_lo;
-                        const bool band = cand_ok && q2 >= rc2_lo && q2 < rc2_hi;
-                        // the FP64 decision inside the band (rare)
-                        if (__any_sync(full, band) && band) {
-                            double d64[3];
-                            in = sep64<D>(G, xpos, n, s, j, d64) < rc2;
-                        }
-                    } else {
-                        const S xi = home[w][h];
-                        const double xiv[3] = {xi.x, xi.y, xi.z}, xjv[3] = {e.x, e.y, e.z};
-                        double d[3];
-#pragma unroll
-                        for (int a = 0; a < D; ++a) {
-                            double v = __dsub_rn(xiv[a], xjv[a]);
-                            if (G.periodic[a]) {
-                                if (v > G.halfL[a]) v = __dsub_rn(v, G.L[a]);
-                                else if (v < -G.halfL[a]) v = __dadd_rn(v, G.L[a]);
-                            }
-                            d[a] = v;
-                        }
-                        double r2 = __dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1]));
-                        if (D == 3) r2 = __dadd_rn(r2, __dmul_rn(d[2], d[2]));
-                        in = valid && j != s && r2 < rc2;
+                    const float4 oi = home[w][h];
+                    float f0, f1, f2;
+                    const float q2 = sep32<2>(shifted_offset<2>(oi, dx, dy, dz, sf), e, f0, f1, f2);
+                    const bool cand_ok = valid && j != s;
+                    bool in = cand_ok && q2 < rc2_lo;
+                    const bool band = cand_ok && q2 >= rc2_lo && q2 < rc2_hi;
+                    // the FP64 decision inside the band (rare)
+                    if (__any_sync(full, band) && band) {
+                        double d64[3];
+                        in = sep64<2>(G, xpos, n, s, j, d64) < rc2;
                     }
                     const unsigned bal = __ballot_sync(full, in);
                     if (bal) {
@@ -245,249 +193,149 @@ __global__ void __launch_bounds__(kBlock) k_nlist_cells(Buffers B, const double 
             __syncwarp();
         }
         if (lane < nh) {
+            const int s = h0 + lane;
             if (cnt > K) {
                 atomicOr(B.err, kErrCapacity);
                 cnt = K;
             }
-            B.pcount[h0 + lane] = cnt;
-        }
-        __syncwarp();
-    }
-}
-
-// 3D lists on the FP32C path, one warp per home cell with the home particles in
-// the lanes (a 3D cell holds about 28, so the lanes stay busy): the staged
-// candidates are moved into the home cell's frame (offset + shift s, tagged with
-// the list entry), every lane tests them four at a time with broadcast reads,
-// and appends its hits to an eight-entry buffer of its own in shared memory,
-// which it writes out as one aligned 32-byte sector of its list (slot s at
-// s Ks + k, Ks = K rounded up to 8) each time it fills. The FP32 separation here
-// is o_i - (o_j + shift s); it decides outside the band around the cutoff
-// exactly as the canonical form does, and the FP64 test decides inside it, so
-// the sets and their order are those of k_nlist_cells.
-constexpr int kBufEntries = 8;
-
-__global__ void __launch_bounds__(kBlock) k_nlist_cells3_f32(Buffers B, const double *__restrict__ xpos,
-                                                             uint32_t *__restrict__ lists, int Ks)
-{
-    if (skip_relist(B)) return;   // (the step graph: relisting or not)
-    constexpr int NC = 27;
-    constexpr int CH = 256;
-    __shared__ float4 cand[kWarpsPerBlock][CH];
-    __shared__ __align__(16) uint32_t buf[kWarpsPerBlock][kWarp][kBufEntries];
-    __shared__ int tpre[kWarpsPerBlock][NC + 1];
-    __shared__ int tbeg[kWarpsPerBlock][NC];
-    constexpr unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & (kWarp - 1), w = threadIdx.x >> 5;
-    const unsigned lt = (1u << lane) - 1u;
-    const int c = blockIdx.x * kWarpsPerBlock + w;
-    if (c >= B.ncell) return;
-    const int inst = cell_instance(B, c);
-    const int cell_off = B.inst[inst].cell_off;
-    const Geom &G = B.geo[inst];
-    const int nx = G.nc[0], ny = G.nc[1], nz = G.nc[2];
-    const int lc = c - cell_off;
-    if (lc >= nx * ny * nz) return;
-    const int *start = B.cell_start + cell_off;
-    const int hb = start[lc], he = start[lc + 1];
-    if (hb == he) return;
-    const int cx = lc % nx, cy = (lc / nx) % ny, cz = lc / (nx * ny);
-    const float sf[3] = {G.s_f[0], G.s_f[1], G.s_f[2]};
-    const float rc2_lo = G.rc2_lo, rc2_hi = G.rc2_hi;
-    const double rc2 = G.rc2;
-    const float box_cut2 = rc2_hi * 1.001f;
-    const int n = B.n, K = B.K;
-    int m = 0;
-    if (lane < NC) {
-        const int dx = lane % 3 - 1, dy = (lane / 3) % 3 - 1, dz = lane / 9 - 1;
-        int x = cx + dx, y = cy + dy, z = cz + dz;
-        bool ok = true;
-        if (x < 0 || x >= nx) { if (G.periodic[0]) x = x < 0 ? x + nx : x - nx; else ok = false; }
-        if (y < 0 || y >= ny) { if (G.periodic[1]) y = y < 0 ? y + ny : y - ny; else ok = false; }
-        if (z < 0 || z >= nz) { if (G.periodic[2]) z = z < 0 ? z + nz : z - nz; else ok = false; }
-        if (ok) {
-            const int nc = (z * ny + y) * nx + x;
-            const int jb = start[nc];
-            m = start[nc + 1] - jb;
-            tbeg[w][lane] = jb;
-        } else {
-            tbeg[w][lane] = 0;
-        }
-    }
-    int incl = m;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(full, incl, o);
-        if (lane >= o) incl += v;
-    }
-    if (lane < NC) tpre[w][lane] = incl - m;
-    const int total = __shfl_sync(full, incl, NC - 1);
-    if (lane == NC) tpre[w][NC] = total;
-    __syncwarp();
-    uint32_t *my = buf[w][lane];
-    for (int h0 = hb; h0 < he; h0 += kWarp) {
-        const int s = h0 + lane;
-        const bool act = s < he;
-        // an idle lane tests from far away: it fails every distance test
-        const float4 oi = act ? B.off[s] : make_float4(3e18f, 3e18f, 3e18f, 0.f);
-        uint32_t *out = lists + (size_t)s * Ks;
-        int cnt = 0;
-        int t = 0;
-        for (int c0 = 0; c0 < total; c0 += CH) {
-            const int span = min(total - c0, CH);
-            int take = 0;
-            for (int q0 = 0; q0 < span; q0 += kWarp) {
-                const int q = q0 + lane;
-                bool keep = false;
-                float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (q < span) {
-                    const int p = c0 + q;
-                    while (tpre[w][t + 1] <= p) ++t;
-                    const int j = tbeg[w][t] + (p - tpre[w][t]);
-                    const float4 oj = B.off[j];
-                    const int dx = t % 3 - 1, dy = (t / 3) % 3 - 1, dz = t / 9 - 1;
-                    e.x = __fadd_rn(oj.x, (float)dx * sf[0]);
-                    e.y = __fadd_rn(oj.y, (float)dy * sf[1]);
-                    e.z = __fadd_rn(oj.z, (float)dz * sf[2]);
-                    e.w = __uint_as_float(list_entry((uint32_t)j, t, oj.w != 0.f));
-                    const float bx = fmaxf(fmaxf(-e.x, e.x - sf[0]), 0.f);
-                    const float by = fmaxf(fmaxf(-e.y, e.y - sf[1]), 0.f);
-                    const float bz = fmaxf(fmaxf(-e.z, e.z - sf[2]), 0.f);
-                    keep = bx * bx + by * by + bz * bz < box_cut2;
-                }
-                const unsigned bal = __ballot_sync(full, keep);
-                if (keep) cand[w][take + __popc(bal & lt)] = e;
-                take += __popc(bal);
-            }
-            // pad to a multiple of four with entries that fail every test
-            const int take4 = (take + 3) & ~3;
-            if (take + lane < take4)
-                cand[w][take + lane] = make_float4(-3e18f, -3e18f, -3e18f, __uint_as_float(kNoParticle));
-            __syncwarp();
-            for (int q = 0; q < take4; q += 4) {
-                bool in[4], band[4];
-                uint32_t ew[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float4 e = cand[w][q + u];
-                    const float d0 = __fsub_rn(oi.x, e.x), d1 = __fsub_rn(oi.y, e.y), d2 = __fsub_rn(oi.z, e.z);
-                    const float q2 = __fmaf_rn(d2, d2, __fmaf_rn(d1, d1, __fmul_rn(d0, d0)));
-                    ew[u] = __float_as_uint(e.w);
-                    const bool other = (ew[u] & kSlotMask) != (uint32_t)s;
-                    in[u] = q2 < rc2_lo && other;
-                    band[u] = q2 >= rc2_lo && q2 < rc2_hi && other;
-                }
-                // the FP64 decision inside the band (rare)
-                if (__any_sync(full, band[0] || band[1] || band[2] || band[3])) {
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        if (band[u]) {
-                            double d64[3];
-                            in[u] = sep64<3>(G, xpos, n, s, entry_slot(ew[u]), d64) < rc2;
-                        }
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    if (in[u]) {
-                        my[cnt & (kBufEntries - 1)] = ew[u];
-                        ++cnt;
-                        // a full buffer goes out as one aligned sector of the list
-                        if ((cnt & (kBufEntries - 1)) == 0 && cnt <= K) {
-                            const uint4 a = *reinterpret_cast<const uint4 *>(my);
-                            const uint4 b = *reinterpret_cast<const uint4 *>(my + 4);
-                            uint4 *dst = reinterpret_cast<uint4 *>(out + (cnt - kBufEntries));
-                            dst[0] = a;
-                            dst[1] = b;
-                        }
-                    }
-                }
-            }
-            __syncwarp();
-        }
-        if (act) {
-            // the entries since the last full buffer
-            const int tail = cnt & (kBufEntries - 1);
-            for (int k = 0; k < tail; ++k)
-                if (cnt - tail + k < K) out[cnt - tail + k] = my[k];
-            if (cnt > K) {
-                atomicOr(B.err, kErrCapacity);
-                cnt = K;
-            }
+            // the row up to a multiple of four (Ks is one): the particle itself
+            for (int k = cnt; k & 3; ++k) lists[(size_t)s * Ks + k] = list_entry((uint32_t)s, 13, false);
             B.pcount[s] = cnt;
         }
         __syncwarp();
     }
 }
 
-// 2D lists on the FP32C path, one warp per row segment of up to kSeg2 cells along
-// x (a 2D cell holds about 9 particles, so three cells fill most of the lanes) with
-// the segment's particles in the lanes, as the 3D builder does for one cell. The
-// warp stages the candidates of the 3 x (segment + 2) surrounding cells in the
-// order rows (dy), then column, then slot, moved into the frame of the segment's
-// first cell; each lane tests them four at a time against its particle, keeps
-// those of the three columns around its own cell, and appends its hits through an
-// eight-entry buffer as whole sectors of its list. For every particle the
-// candidates of its own 3 x 3 cells come in the order rows, dx, slot, so its list
-// holds the entries of k_nlist_cells in the same order; outside the band around
-// the cutoff this FP32 separation decides as the canonical one does, and the FP64
-// test decides inside it.
+// 2D problems with fewer row segments than this take k_nlist_cells2: a warp per
+// cell instead of one per three keeps more warps busy (200 x 200, 1,452 segments:
+// a step of ten 0.311 ms, 0.320 ms with k_nlist_home).
 constexpr int kRowsMinSegments = 16384;
 
-__global__ void __launch_bounds__(kBlock) k_nlist_rows2_f32(Buffers B, const double *__restrict__ xpos,
-                                                            uint32_t *__restrict__ lists, int Ks)
+// Lists with the home particles in the lanes: one warp per row segment of kSeg2
+// cells along x in 2D (a 2D cell holds about 9 particles, so three fill most of the
+// lanes), per cell in 3D (about 28 particles). Bound by instruction issue.
+//  - Staging. The candidates of the surrounding cells pass in the order rows (dz,
+//    dy), column, slot; one farther than the cutoff from the whole segment is
+//    dropped; the others are moved into the frame of the segment's first cell
+//    and packed into shared memory, coordinates by component, entries apart.
+//  - Tests. Each lane tests a chunk of 32 candidates against its particle without
+//    a branch: t = |r|^2 - lo, two candidates per packed instruction and four per
+//    16-byte broadcast read; the sign bit is shifted into the lane's mask word,
+//    and the smallest t >= 0 kept as an integer (below the band's width: a
+//    candidate inside the band around the cutoff; then the chunk's band
+//    candidates take the FP64 test).
+//  - Emission. The roles turn round: a lane per candidate, one home particle
+//    after the other. The particle's mask word says which lanes write, the bits
+//    before a lane's own where, so every hit costs the warp nothing beyond its
+//    particle's word and the hits of a chunk leave as one contiguous run. (Each
+//    lane walking the bits of its own words: 1.5 ms against 1.1 ms a build at
+//    128^3, the lanes out of step.)
+// For every particle the candidates of its own 3^D cells come in the order of
+// k_nlist_cells2; the FP32 separation o_i - (o_j + shift s) decides outside the
+// band as the canonical form does, so sets and order are the same on every path.
+// The FP64 path takes the same pre-test (its offsets are kept for it): FP64 tests
+// of every candidate run at 1/64 of the rate (45^3: 3.7 ms a build, now 0.1 ms).
+// Against the builders with a per-hit append by the home particle's lane: 128^3
+// 2.04 ms a build, now 1.1 ms; the 64-vortex batch 0.37 ms, now 0.24 ms.
+constexpr int kListWarps = 4;                 // warps per block
+constexpr int kStage = 256;                   // staged candidates per warp
+
+// |o_i - c|^2 - lo of a home particle and a staged candidate in the same frame.
+template <int D>
+__device__ __forceinline__ float near_test(float4 oi, float x, float y, float z, float neg_lo)
+{
+    const float d0 = __fsub_rn(x, oi.x), d1 = __fsub_rn(y, oi.y);
+    float t = __fmaf_rn(d1, d1, __fmaf_rn(d0, d0, neg_lo));
+    if (D == 3) {
+        const float d2 = __fsub_rn(z, oi.z);
+        t = __fmaf_rn(d2, d2, t);
+    }
+    return t;
+}
+
+// near_test of two candidates.
+template <int D>
+__device__ __forceinline__ void near_test2(const F2 *oi, F2 x, F2 y, F2 z, F2 neg_lo, uint32_t &a, uint32_t &b)
+{
+    const F2 d0 = sub2(x, oi[0]), d1 = sub2(y, oi[1]);
+    F2 t = fma2(d1, d1, fma2(d0, d0, neg_lo));
+    if (D == 3) {
+        const F2 d2 = sub2(z, oi[2]);
+        t = fma2(d2, d2, t);
+    }
+    float ta, tb;
+    unpack2(t, ta, tb);
+    a = __float_as_uint(ta);
+    b = __float_as_uint(tb);
+}
+
+template <int D>
+__global__ void __launch_bounds__(kListWarps * kWarp) k_nlist_home(Buffers B, const double *__restrict__ xpos,
+                                                                   uint32_t *__restrict__ lists, int Ks)
 {
     if (skip_relist(B)) return;   // (the step graph: relisting or not)
-    constexpr int NCOL = kSeg2 + 2;                     // candidate columns
-    constexpr int NT = 3 * NCOL;                        // candidate cells
-    constexpr int CH = 256;
-    __shared__ float4 cand[kWarpsPerBlock][CH];
-    __shared__ __align__(16) uint32_t buf[kWarpsPerBlock][kWarp][kBufEntries];
-    __shared__ int tpre[kWarpsPerBlock][NT + 1];
-    __shared__ int tbeg[kWarpsPerBlock][NT];
+    constexpr int SEG = D == 2 ? kSeg2 : 1;
+    constexpr int NCOL = SEG + 2;                       // candidate columns
+    constexpr int NT = (D == 3 ? 9 : 3) * NCOL;         // candidate cells
+    constexpr int kHomeRow = D == 3 ? 4 : 1;            // the row dy = dz = 0
+    __shared__ __align__(16) float cx[kListWarps][D][kStage];
+    __shared__ uint32_t ent[kListWarps][kStage];
+    // per home particle of the round: its mask word of the chunk, and where its
+    // next entry goes from the round's first row (2D: and its cell, bits 30-31)
+    __shared__ __align__(16) uint2 word[kListWarps][kWarp];
+    __shared__ int own[kListWarps][kWarp];              // staged place of each home particle, -1
+    __shared__ int tpre[kListWarps][NT + 1];            // candidates before cell t
+    __shared__ int tbeg[kListWarps][NT];                // first slot of cell t
     constexpr unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & (kWarp - 1), w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    const int g = blockIdx.x * kWarpsPerBlock + w;     // global row segment of this warp
-    if (g >= B.nseg2) return;
-    const int inst = segment_instance(B, g);
-    const int cell_off = B.inst[inst].cell_off;
+    const int g = blockIdx.x * kListWarps + w;          // global segment (2D), cell (3D) of this warp
+    if (g >= (D == 2 ? B.nseg2 : B.ncell)) return;      // whole warp
+    const int inst = D == 2 ? segment_instance(B, g) : cell_instance(B, g);
     const Geom &G = B.geo[inst];
-    const int nx = G.nc[0], ny = G.nc[1];
-    const int nsx = (nx + kSeg2 - 1) / kSeg2;           // segments per row
-    const int ls = g - B.inst[inst].seg_off;
-    const int cx = (ls % nsx) * kSeg2, cy = ls / nsx;
-    const int lc = cy * nx + cx;
-    const int ns = min(kSeg2, nx - cx);                 // cells of this segment
-    const int *start = B.cell_start + cell_off;
+    const int nx = G.nc[0], ny = G.nc[1], nz = G.nc[2];
+    int cx0, cy0, cz0, lc, ns = 1;                      // first cell of the segment, its cells
+    if (D == 2) {
+        const int nsx = (nx + SEG - 1) / SEG;
+        const int ls = g - B.inst[inst].seg_off;
+        cx0 = (ls % nsx) * SEG;
+        cy0 = ls / nsx;
+        cz0 = 0;
+        lc = cy0 * nx + cx0;
+        ns = min(SEG, nx - cx0);
+    } else {
+        lc = g - B.inst[inst].cell_off;
+        if (lc >= nx * ny * nz) return;                 // the instance's empty sentinel cell
+        cx0 = lc % nx;
+        cy0 = (lc / nx) % ny;
+        cz0 = lc / (nx * ny);
+    }
+    const int *start = B.cell_start + B.inst[inst].cell_off;
     const int hb = start[lc], he = start[lc + ns];
     if (hb == he) return;
-    // first slots of the segment's second and third cells
-    const int b1 = ns > 1 ? start[lc + 1] : he, b2 = ns > 2 ? start[lc + 2] : he;
-    const float sf[2] = {G.s_f[0], G.s_f[1]};
-    const float rc2_lo = G.rc2_lo, rc2_hi = G.rc2_hi;
-    const double rc2 = G.rc2;
-    const float box_cut2 = rc2_hi * 1.001f;
-    const float seg_w = (float)ns * sf[0];
-    const int n = B.n, K = B.K;
-    // the candidate cells side by side: lane t takes row t / NCOL (dy + 1) and
-    // column t % NCOL (x = cx - 1 + column); empty when off a closed edge or past
-    // the segment's last column
-    int m = 0;
+    // first slots of a 2D segment's second and third cells
+    const int b1 = D == 2 && ns > 1 ? start[lc + 1] : he, b2 = D == 2 && ns > 2 ? start[lc + 2] : he;
+    const float sx = G.s_f[0], sy = G.s_f[1], sz = G.s_f[2];
+    const float neg_lo = -G.rc2_lo, box_cut2 = G.rc2_hi * 1.001f, seg_w = (float)ns * sx;
+    const uint32_t band = __float_as_uint(G.rc2_hi - G.rc2_lo);
+    const int K = B.K, n = B.n;
+    // the candidate cells side by side: lane t takes row t / NCOL = (dy + 1) +
+    // 3 (dz + 1) and column t % NCOL (x = cx0 - 1 + column); empty when off a closed
+    // edge or past the segment's last column
+    int m = 0, beg = 0;
     if (lane < NT) {
-        const int r = lane / NCOL, k = lane % NCOL;
-        int x = cx - 1 + k, y = cy + r - 1;
+        const int k = lane % NCOL, r = lane / NCOL;
+        int x = cx0 - 1 + k, y = cy0 + r % 3 - 1, z = D == 3 ? cz0 + r / 3 - 1 : 0;
         bool ok = k < ns + 2;
         if (ok && (x < 0 || x >= nx)) { if (G.periodic[0]) x = x < 0 ? x + nx : x - nx; else ok = false; }
         if (ok && (y < 0 || y >= ny)) { if (G.periodic[1]) y = y < 0 ? y + ny : y - ny; else ok = false; }
+        if (D == 3 && ok && (z < 0 || z >= nz)) { if (G.periodic[2]) z = z < 0 ? z + nz : z - nz; else ok = false; }
         if (ok) {
-            const int nc = y * nx + x;
-            const int jb = start[nc];
-            m = start[nc + 1] - jb;
-            tbeg[w][lane] = jb;
-        } else {
-            tbeg[w][lane] = 0;
+            const int nc = (z * ny + y) * nx + x;
+            beg = start[nc];
+            m = start[nc + 1] - beg;
         }
+        tbeg[w][lane] = beg;
     }
     int incl = m;
 #pragma unroll
@@ -497,109 +345,162 @@ __global__ void __launch_bounds__(kBlock) k_nlist_rows2_f32(Buffers B, const dou
     }
     if (lane < NT) tpre[w][lane] = incl - m;
     const int total = __shfl_sync(full, incl, NT - 1);
-    if (lane == NT) tpre[w][NT] = total;
-    __syncwarp();
-    uint32_t *my = buf[w][lane];
+    if (lane == 0) tpre[w][NT] = total;
+    const uint32_t bit = 0x80000000u >> lane, before = ~(0xffffffffu >> lane);
     for (int h0 = hb; h0 < he; h0 += kWarp) {
         const int s = h0 + lane;
         const bool act = s < he;
-        const int kh = (s >= b1) + (s >= b2);           // the lane's cell in the segment
+        const int nh = min(kWarp, he - h0);
+        const int kh = D == 2 ? (s >= b1) + (s >= b2) : 0;      // the lane's cell in the segment
         // an idle lane tests from far away: it fails every distance test
-        float4 oi = make_float4(3e18f, 3e18f, 0.f, 0.f);
+        float4 oi = make_float4(3e18f, 3e18f, 3e18f, 0.f);
         if (act) {
             oi = B.off[s];
-            oi.x = __fadd_rn(oi.x, (float)kh * sf[0]);
+            if (D == 2) oi.x = __fadd_rn(oi.x, (float)kh * sx);
         }
-        uint32_t *out = lists + (size_t)s * Ks;
-        int cnt = 0;
-        int t = 0;
-        for (int c0 = 0; c0 < total; c0 += CH) {
-            const int span = min(total - c0, CH);
-            int take = 0;
-            for (int q0 = 0; q0 < span; q0 += kWarp) {
-                const int q = q0 + lane;
+        const F2 oi2[3] = {both(oi.x), both(oi.y), both(oi.z)};
+        const F2 neg_lo2 = both(neg_lo);
+        uint32_t *out0 = lists + (size_t)h0 * Ks;       // the round's first row
+        int cnt = 0;                                    // list length so far
+        int t = 0;                                      // candidate cell of the next position
+        int p0 = 0;                                     // candidates looked at
+        int take = 0;                                   // staged, not yet tested
+        own[w][lane] = -1;
+        __syncwarp();
+        do {
+            // stage: 32 candidates at a time while they fit
+            while (p0 < total && take <= kStage - kWarp) {
+                const int p = p0 + lane;
                 bool keep = false;
-                float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (q < span) {
-                    const int p = c0 + q;
+                float ex = 0.f, ey = 0.f, ez = 0.f;
+                uint32_t e = 0u;
+                int h = -1;                             // a home particle's own place: which
+                if (p < total) {
                     while (tpre[w][t + 1] <= p) ++t;
                     const int j = tbeg[w][t] + (p - tpre[w][t]);
                     const float4 oj = B.off[j];
                     const int r = t / NCOL, k = t % NCOL;
-                    e.x = __fadd_rn(oj.x, (float)(k - 1) * sf[0]);
-                    e.y = __fadd_rn(oj.y, (float)(r - 1) * sf[1]);
-                    // the column, and the list entry with the row's part of the shift
-                    // code (dx + 1) + 3 (dy + 1) + 9: a lane adds its dx + 1
-                    e.z = __int_as_float(k);
-                    e.w = __uint_as_float(list_entry((uint32_t)j, 3 * r + 9, oj.w != 0.f));
-                    const float bx = fmaxf(fmaxf(-e.x, e.x - seg_w), 0.f);
-                    const float by = fmaxf(fmaxf(-e.y, e.y - sf[1]), 0.f);
-                    keep = bx * bx + by * by < box_cut2;
+                    ex = __fadd_rn(oj.x, (float)(k - 1) * sx);
+                    ey = __fadd_rn(oj.y, (float)(r % 3 - 1) * sy);
+                    const float bx = fmaxf(fmaxf(-ex, ex - seg_w), 0.f);
+                    const float by = fmaxf(fmaxf(-ey, ey - sy), 0.f);
+                    float b = bx * bx + by * by;
+                    if (D == 3) {
+                        ez = __fadd_rn(oj.z, (float)(r / 3 - 1) * sz);
+                        const float bz = fmaxf(fmaxf(-ez, ez - sz), 0.f);
+                        b += bz * bz;
+                    }
+                    keep = b < box_cut2;
+                    // the shift code (dx + 1) + 3 (dy + 1) + 9 (dz + 1) with the column in
+                    // the place of dx + 1: emission takes the home cell's column off it
+                    e = list_entry((uint32_t)j, k + 3 * r + (D == 2 ? 9 : 0), oj.w != 0.f);
+                    if (r == kHomeRow && k >= 1 && k <= ns && j >= h0 && j < h0 + kWarp) h = j - h0;
                 }
                 const unsigned bal = __ballot_sync(full, keep);
-                if (keep) cand[w][take + __popc(bal & lt)] = e;
+                if (keep) {
+                    const int at = take + __popc(bal & lt);
+                    cx[w][0][at] = ex;
+                    cx[w][1][at] = ey;
+                    if constexpr (D == 3) cx[w][2][at] = ez;
+                    ent[w][at] = e;
+                    if (h >= 0) own[w][h] = at;
+                }
                 take += __popc(bal);
+                p0 += kWarp;
             }
-            // pad to a multiple of four with entries that fail every test
-            const int take4 = (take + 3) & ~3;
-            if (take + lane < take4)
-                cand[w][take + lane] = make_float4(-3e18f, -3e18f, __int_as_float(0x7f), __uint_as_float(kNoParticle));
+            const bool end = p0 >= total;
+            if (end && (take & (kWarp - 1))) {
+                // the last chunk is filled up with candidates that fail every test
+                const int at = take + lane;
+                take = (take + kWarp - 1) / kWarp * kWarp;
+                if (at < take) {
+                    cx[w][0][at] = -3e18f;
+                    cx[w][1][at] = -3e18f;
+                    if constexpr (D == 3) cx[w][2][at] = -3e18f;
+                    ent[w][at] = 0u;
+                }
+            }
             __syncwarp();
-            // the tests set one bit (candidate q0 + b: bit b) per candidate of the
-            // lane's three columns closer than the band's top, without branches;
-            // each such candidate is then classified in candidate order: the lane's
-            // own particle is skipped, below the band it is a neighbour, inside the
-            // band (rare) the FP64 test decides
-            for (int q0 = 0; q0 < take4; q0 += kWarp) {
-                const int qn = min(kWarp, take4 - q0);
-                uint32_t maybe = 0u;
-                for (int q = 0; q < qn; q += 4) {
+            const int mine = own[w][lane];
+            const int nfull = take / kWarp;
+            for (int c = 0; c < nfull; ++c) {
+                uint32_t hits = 0u, near = 0xffffffffu;
+                const ulonglong2 *x4 = reinterpret_cast<const ulonglong2 *>(&cx[w][0][c * kWarp]);
+                const ulonglong2 *y4 = reinterpret_cast<const ulonglong2 *>(&cx[w][1][c * kWarp]);
+                const ulonglong2 *z4 = reinterpret_cast<const ulonglong2 *>(&cx[w][D - 1][c * kWarp]);
+#pragma unroll
+                for (int q = 0; q < kWarp / 4; ++q) {
+                    const ulonglong2 X = x4[q], Y = y4[q], Z = z4[q];
+                    uint32_t b[4];                       // candidate i of the chunk: bit 31 - i
+                    near_test2<D>(oi2, F2{X.x}, F2{Y.x}, F2{Z.x}, neg_lo2, b[0], b[1]);
+                    near_test2<D>(oi2, F2{X.y}, F2{Y.y}, F2{Z.y}, neg_lo2, b[2], b[3]);
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        const float4 e = cand[w][q0 + q + u];
-                        const uint32_t dxp = (uint32_t)(__float_as_int(e.z) - kh);   // dx + 1 from the lane's cell
-                        const float d0 = __fsub_rn(oi.x, e.x), d1 = __fsub_rn(oi.y, e.y);
-                        const float q2 = __fmaf_rn(d1, d1, __fmul_rn(d0, d0));
-                        if (q2 < rc2_hi && dxp <= 2u) maybe |= 1u << (q + u);
+                        hits = __funnelshift_l(b[u], hits, 1);
+                        near = min(near, b[u]);
                     }
                 }
-                while (maybe) {
-                    const int b = __ffs(maybe) - 1;
-                    maybe &= maybe - 1u;
-                    const float4 e = cand[w][q0 + b];
-                    const uint32_t ej = __float_as_uint(e.w);
-                    const int j = entry_slot(ej);
-                    if (j == s) continue;
-                    const float d0 = __fsub_rn(oi.x, e.x), d1 = __fsub_rn(oi.y, e.y);
-                    const float q2 = __fmaf_rn(d1, d1, __fmul_rn(d0, d0));
-                    bool in = q2 < rc2_lo;
-                    if (!in) {
+                // the FP64 decision inside the band (rare)
+                if (__any_sync(full, near < band) && near < band) {
+                    for (int q = 0; q < kWarp; ++q) {
+                        const int at = c * kWarp + q;
+                        const float d2 = near_test<D>(oi, cx[w][0][at], cx[w][1][at], cx[w][D - 1][at], neg_lo);
+                        if (__float_as_uint(d2) >= band) continue;
                         double d64[3];
-                        in = sep64<2>(G, xpos, n, s, j, d64) < rc2;
-                    }
-                    if (!in) continue;
-                    const uint32_t dxp = (uint32_t)(__float_as_int(e.z) - kh);
-                    my[cnt & (kBufEntries - 1)] = ej + (dxp << kCodeShift);
-                    ++cnt;
-                    // a full buffer goes out as one aligned sector of the list
-                    if ((cnt & (kBufEntries - 1)) == 0 && cnt <= K) {
-                        const uint4 a = *reinterpret_cast<const uint4 *>(my);
-                        const uint4 c4 = *reinterpret_cast<const uint4 *>(my + 4);
-                        uint4 *dst = reinterpret_cast<uint4 *>(out + (cnt - kBufEntries));
-                        dst[0] = a;
-                        dst[1] = c4;
+                        if (sep64<D>(G, xpos, n, s, entry_slot(ent[w][at]), d64) < G.rc2) hits |= 0x80000000u >> q;
                     }
                 }
+                if (mine >> 5 == c) hits &= ~(0x80000000u >> (mine & 31));    // not itself
+                const int nhit = __popc(hits);
+                // (a list longer than its row is cut there and raises the error below)
+                word[w][lane] = make_uint2(cnt + nhit <= Ks ? hits : 0u, (uint32_t)(lane * Ks + cnt) | (uint32_t)kh << 30);
+                cnt += nhit;
+                __syncwarp();
+                const uint32_t e = ent[w][c * kWarp + lane];
+                const ulonglong2 *wd = reinterpret_cast<const ulonglong2 *>(&word[w][0]);
+                auto put = [&](unsigned long long v) {
+                    const uint32_t hm = (uint32_t)v, at = (uint32_t)(v >> 32);
+                    if (hm & bit) {
+                        const uint32_t o = D == 2 ? at & 0x3fffffffu : at;
+                        out0[o + __popc(hm & before)] = D == 2 ? e - ((at >> 30) << kCodeShift) : e;
+                    }
+                };
+#pragma unroll 4
+                for (int h = 0; h < nh; h += 2) {        // (an idle lane's word is empty)
+                    const ulonglong2 v = wd[h >> 1];
+                    put(v.x);
+                    put(v.y);
+                }
+                __syncwarp();
+            }
+            // the candidates of an unfinished chunk move to the front
+            const int left = take - nfull * kWarp;
+            float fx = 0.f, fy = 0.f, fz = 0.f;
+            uint32_t fe = 0u;
+            if (lane < left) {
+                const int at = nfull * kWarp + lane;
+                fx = cx[w][0][at];
+                fy = cx[w][1][at];
+                fz = cx[w][D - 1][at];
+                fe = ent[w][at];
             }
             __syncwarp();
-        }
+            if (lane < left) {
+                cx[w][0][lane] = fx;
+                cx[w][1][lane] = fy;
+                if constexpr (D == 3) cx[w][2][lane] = fz;
+                ent[w][lane] = fe;
+            }
+            own[w][lane] = mine - nfull * kWarp;        // (tested: negative)
+            __syncwarp();
+            take = left;
+        } while (p0 < total || take > 0);
         if (act) {
-            // the entries since the last full buffer
-            const int tail = cnt & (kBufEntries - 1);
-            for (int k = 0; k < tail; ++k)
-                if (cnt - tail + k < K) out[cnt - tail + k] = my[k];
+            // the row up to a multiple of four (Ks is one): the particle itself
+            for (int k = cnt; (k & 3) && k < Ks; ++k) out0[lane * Ks + k] = list_entry((uint32_t)s, 13, false);
             if (cnt > K) {
                 atomicOr(B.err, kErrCapacity);
+                for (int k = 0; k < Ks; ++k) out0[lane * Ks + k] = list_entry((uint32_t)s, 13, false);
                 cnt = K;
             }
             B.pcount[s] = cnt;
@@ -640,7 +541,7 @@ __global__ void __launch_bounds__(kBlock) k_list_slice(Buffers B, const uint32_t
 
 }  // namespace
 
-static_assert(list_stride(1) % kBufEntries == 0, "a list row holds whole buffers of the 3D builder");
+static_assert(list_stride(1) % 4 == 0, "a list row holds whole 16-byte stores");
 
 // The lists of every slot at xpos into the per-slot layout (slot_list); with
 // `sliced`, also copied into the sliced layout of pj for the kernels that walk
@@ -650,17 +551,17 @@ void launch_nlist(const Buffers &B, const double *xpos, const int *cell, const u
                   bool sliced)
 {
     (void)cell;
-    const int nb = (B.ncell + kWarpsPerBlock - 1) / kWarpsPerBlock;
     const int Ks = list_stride(B.K);
-    if (B.dim == 3 && B.fp32c) {
-        k_nlist_cells3_f32<<<nb, kBlock, 0, st>>>(B, xpos, B.pjt, Ks);
-    } else if (B.fp32c && B.nseg2 >= kRowsMinSegments) {
-        // enough row segments to fill the GPU several times over; fewer, and a
-        // warp per cell keeps more warps busy (both give the same lists)
-        const int nb2 = (B.nseg2 + kWarpsPerBlock - 1) / kWarpsPerBlock;
-        k_nlist_rows2_f32<<<nb2, kBlock, 0, st>>>(B, xpos, B.pjt, Ks);
+    if (B.dim == 2 && B.nseg2 < kRowsMinSegments) {
+        const int nb = (B.ncell + kWarpsPerBlock - 1) / kWarpsPerBlock;
+        k_nlist_cells2<<<nb, kBlock, 0, st>>>(B, xpos, B.pjt, Ks);
+    } else
+    if (B.dim == 2) {
+        const int nb = (B.nseg2 + kListWarps - 1) / kListWarps;
+        k_nlist_home<2><<<nb, kListWarps * kWarp, 0, st>>>(B, xpos, B.pjt, Ks);
     } else {
-        DTSPH_DISPATCH(B.dim, B.fp32c, (k_nlist_cells<D, F32><<<nb, kBlock, 0, st>>>(B, xpos, gid, B.pjt, Ks)));
+        const int nb = (B.ncell + kListWarps - 1) / kListWarps;
+        k_nlist_home<3><<<nb, kListWarps * kWarp, 0, st>>>(B, xpos, B.pjt, Ks);
     }
     if (sliced) k_list_slice<<<(B.n / kWarp + kWarpsPerBlock - 1) / kWarpsPerBlock, kBlock, 0, st>>>(B, B.pjt, Ks);
 }
