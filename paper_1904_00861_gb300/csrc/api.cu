@@ -277,6 +277,18 @@ void dtsph::make_phys(const dtsph_params &p, Phys &P)
         P.kc3 = 0.0;
         P.edac = 0;
     }
+    PairK32 &k = P.k32;
+    k.ed = P.edac ? (float)(P.c_edac / P.c_div) : 0.f;
+    k.visc = (float)(P.c_visc / P.c_p);
+    k.s_ap = (float)(P.c_div * P.sig_h);
+    k.s_F = (float)(P.c_p * P.sig_h);
+    k.inv_h = (float)P.inv_h;
+    k.eta_h2 = (float)P.eta_h2;
+    k.av = (float)(P.m * P.c_av / P.c_p);
+    k.vol = (float)(P.vol / P.c_p);
+    k.use_av = P.use_av;
+    k.steady = P.steady;
+    k.rare = P.use_av || P.steady;
 }
 
 // Range and consistency checks of one parameter set.
@@ -585,7 +597,7 @@ int allocate(dtsph_ctx *c, const int64_t *nf)
     }
     const size_t nd = (size_t)n * d;
     const size_t nwarps = ((size_t)n + kWarp - 1) / kWarp;
-    const size_t npair = nwarps * B.K * kWarp;
+    const size_t npair = nwarps * ((B.K + 3) / 4 * 4) * kWarp;   // (FP32C rows hold the fill up to four)
     Inst *d_inst;
     Geom *d_geo;
     Phys *d_phys;

@@ -100,9 +100,32 @@ __device__ __forceinline__ float4 ld_f4_hint(const float4 *p, uint64_t policy)
     float4 v;
     asm volatile("ld.global.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "l"(p), "l"(policy)
-                 : "memory");
+                 : "l"(p), "l"(policy));
     return v;
+}
+
+// The same for data read once: not kept in L1.
+__device__ __forceinline__ float4 ld_f4_stream(const float4 *p, uint64_t policy)
+{
+    float4 v;
+    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(p), "l"(policy));
+    return v;
+}
+__device__ __forceinline__ uint2 ld_u2_stream(const uint2 *p, uint64_t policy)
+{
+    uint2 v;
+    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;"
+                 : "=r"(v.x), "=r"(v.y)
+                 : "l"(p), "l"(policy));
+    return v;
+}
+
+// Starts bringing `bytes` (a multiple of 16, from a 16-byte boundary) into L2.
+__device__ __forceinline__ void l2_prefetch(const void *p, uint32_t bytes, uint64_t policy)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global.L2::cache_hint [%0], %1, %2;" ::"l"(p), "r"(bytes), "l"(policy));
 }
 
 __device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity)

@@ -77,6 +77,17 @@ struct Geom {
     float rc2_lo, rc2_hi; // FP32 pre-test band: below lo is in, above hi is out
 };
 
+// Constants of the FP32C path's packed pair sums (pair32.cuh), rounded from Phys.
+struct PairK32 {
+    float ed;            // c_edac / c_div (0 without the EDAC term)
+    float visc;          // c_visc / c_p
+    float s_ap, s_F;     // c_div sigma/h, c_p sigma/h
+    float inv_h, eta_h2;
+    float av, vol;       // m alpha h c / rho0 / c_p; m / rho0 / c_p (steady convection)
+    int use_av, steady, rare;   // rare = use_av || steady
+    int pad;
+};
+
 // Physical constants of the pair terms, folded for rho_i = rho_j = rho0 and a
 // uniform mass m (Sec. 3: density held fixed).
 struct Phys {
@@ -110,6 +121,7 @@ struct Phys {
                          // from r^0 that the lists with a skin cover (moving = 2)
     double disp2_reuse;  // (list_skin / 2)^2: the largest squared distance of r^{n+1}
                          // from r^0 that lets the r^0 lists serve the next step
+    PairK32 k32;
 };
 
 // Stop reason of a loop without the pair cache that reached pause_at iterations
@@ -215,11 +227,13 @@ struct Buffers {
     double *vk[2];         // V^k FP64 [dim][n]
     double4_32a *nb64[2];      // FP64: (V, p-hat) packed for neighbour gathers
     float4 *nb32[2];       // FP32C: (V, p-hat) packed for neighbour gathers
-    // pair cache, sliced by warp: entry k of slot i at ((i/32) K + k) 32 + i%32
-    uint32_t *pj;          // list entries (list_entry); after the pair-cache pass slot | kWallBit
     uint32_t *pjt;         // neighbour lists, per slot: entry k of slot s at s Ks + k (Ks = list_stride(K))
+    // pair cache, sliced by warp: FP64 entry k of slot i at ((i/32) K + k) 32 + i%32;
+    // FP32C pairs of entries (pair32.cuh)
+    uint32_t *pj;          // slot | kWallBit of each entry (in 2D FP32C in pc32); particles moving
+                           // in pseudo-time: the sliced lists, one entry per place
     double4_32a *pc64;         // FP64: (gradW, F_ij)
-    float4 *pc32;          // FP32C: (gradW, F_ij); in 2D .w holds the index bits
+    float4 *pc32;          // FP32C: two entries' coefficients in two float4
     int *pcount;           // neighbours of each slot
     // particles moving in pseudo-time (Algorithm 1; allocated only then), order A
     double *xk[2];         // r^{k+1/2} FP64 [dim][n], ping-pong

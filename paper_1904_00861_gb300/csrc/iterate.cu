@@ -14,7 +14,7 @@ static void iterate_lanes(const Buffers &B, unsigned long long cond, int use_con
 {
     const int nb = iterate_tiles(B);
     switch (B.lanes) {
-    case 1: k_iterate<D, F, W, 1><<<nb, kBlock, ring_bytes<D, F>(B.stages), st>>>(B, cond, use_cond); break;
+    case 1: k_iterate<D, F, W, 1><<<nb, kBlock, ring_bytes<F>(B.stages), st>>>(B, cond, use_cond); break;
     case 2: k_iterate<D, F, W, 2><<<nb, kBlock, 0, st>>>(B, cond, use_cond); break;
     case 4: k_iterate<D, F, W, 4><<<nb, kBlock, 0, st>>>(B, cond, use_cond); break;
     default: k_iterate<D, F, W, 8><<<nb, kBlock, 0, st>>>(B, cond, use_cond); break;
@@ -67,14 +67,13 @@ static const void *loop_lanes(int lanes)
 static size_t iterate_smem(const Buffers &B)
 {
     if (B.lanes != 1 || B.form_a) return 0;              // the ring holds cache rows only
-    if (B.dim == 2) return B.fp32c ? ring_bytes<2, true>(B.stages) : ring_bytes<2, false>(B.stages);
-    return B.fp32c ? ring_bytes<3, true>(B.stages) : ring_bytes<3, false>(B.stages);
+    return B.fp32c ? ring_bytes<true>(B.stages) : ring_bytes<false>(B.stages);
 }
 
 template <int D, bool F, bool W>
 static cudaError_t allow_ring_smem()
 {
-    const int bytes = (int)ring_bytes<D, F>(kMaxStages);
+    const int bytes = (int)ring_bytes<F>(kMaxStages);
     cudaError_t e = cudaFuncSetAttribute((const void *)k_iterate<D, F, W, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          bytes);
     if (e == cudaSuccess)

@@ -34,6 +34,7 @@
 #include "bulk.cuh"
 #include "geometry.cuh"
 #include "loop_rules.cuh"
+#include "pair32.cuh"
 #include "pair_terms.cuh"
 
 namespace dtsph {
@@ -49,56 +50,49 @@ constexpr int kWallLanes = 8;
 // Wall values of wall slot s for the iteration whose iterate sits in buffer
 // cur, from the cached fluid neighbours of the slot, by the kWallLanes lanes of
 // a group (sub: lane in the group; gmask: the group's lanes in the warp). Lane
-// sub takes entries sub, sub + kWallLanes, ..., R of them in flight (their
-// coefficients, then their neighbour gathers); the lanes' partial sums then
-// merge in a fixed order, so every run gives the same bits. Adami et al.:
+// sub takes entries (FP32C: pairs of entries) sub, sub + kWallLanes, ..., two in
+// flight (their coefficients, then their neighbour gathers); the lanes' partial
+// sums then merge in a fixed order, so every run gives the same bits. Adami et al.:
 // p_w = sum_f (p_f W + rho0 (g . r_wf) W) / sum_f W (the second term cached as
 // Wg), ghost velocity 2 v_w - sum_f V_f W / sum_f W.
 template <int D, bool F32>
 __device__ __forceinline__ void wall_slot(const Buffers &B, int s, int cur, int sub, unsigned gmask)
 {
-    constexpr int R = 2;
     const int cnt = B.pcount[s];
-    const size_t base = (size_t)(s >> 5) * B.K * kWarp + (s & 31);
     double acc[5] = {0, 0, 0, 0, 0};    // sum W, sum (p W + Wg), sum V W
-    for (int k0 = sub; k0 < cnt; k0 += kWallLanes * R) {
-        double W[R], Wg[R];
-        uint32_t jb[R];
+    auto term = [&](double W, double Wg, uint32_t e, double u, double v, double w, double p) {
+        if (e & kWallBit) return;                        // fluid neighbours only
+        acc[0] += W;
+        acc[1] += p * W + Wg;
+        acc[2] += u * W;
+        acc[3] += v * W;
+        acc[4] += w * W;
+    };
+    if constexpr (F32) {
+        for (int m = sub; 2 * m < cnt; m += kWallLanes) {
+            const CachePair r = cache_pair<D>(B, cache_row(B, s) + m, s & 31);
+            const float4 qa = B.nb32[cur][r.ea & ~kWallBit];     // a wall entry's slot is read and not used
+            const float4 qb = B.nb32[cur][r.eb & ~kWallBit];
+            term(r.c0.x, r.c0.z, r.ea, qa.x, qa.y, qa.z, qa.w);
+            if (2 * m + 1 < cnt) term(r.c0.y, r.c0.w, r.eb, qb.x, qb.y, qb.z, qb.w);
+        }
+    } else {
+        constexpr int R = 2;
+        const size_t base = (size_t)(s >> 5) * B.K * kWarp + (s & 31);
+        for (int k0 = sub; k0 < cnt; k0 += kWallLanes * R) {
+            double4_32a c[R], q[R];
+            uint32_t jb[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const size_t e = base + (size_t)min(k0 + r * kWallLanes, cnt - 1) * kWarp;
-            if (F32) {
-                const float4 c = B.pc32[e];
-                W[r] = c.x;
-                Wg[r] = c.y;
-                jb[r] = D == 2 ? __float_as_uint(c.w) : B.pj[e];
-            } else {
-                const double4_32a c = B.pc64[e];
-                W[r] = c.x;
-                Wg[r] = c.y;
+            for (int r = 0; r < R; ++r) {
+                const size_t e = base + (size_t)min(k0 + r * kWallLanes, cnt - 1) * kWarp;
+                c[r] = B.pc64[e];
                 jb[r] = B.pj[e];
             }
-        }
-        double q[R][4];
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int j = (int)(jb[r] & ~kWallBit);     // a wall entry's slot is read and not used
-            if (F32) {
-                const float4 v = B.nb32[cur][j];
-                q[r][0] = v.x; q[r][1] = v.y; q[r][2] = v.z; q[r][3] = v.w;
-            } else {
-                const double4_32a v = B.nb64[cur][j];
-                q[r][0] = v.x; q[r][1] = v.y; q[r][2] = v.z; q[r][3] = v.w;
-            }
-        }
+            for (int r = 0; r < R; ++r) q[r] = B.nb64[cur][jb[r] & ~kWallBit];
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            if (k0 + r * kWallLanes >= cnt || (jb[r] & kWallBit)) continue;   // fluid neighbours only
-            acc[0] += W[r];
-            acc[1] += q[r][3] * W[r] + Wg[r];
-            acc[2] += q[r][0] * W[r];
-            acc[3] += q[r][1] * W[r];
-            acc[4] += q[r][2] * W[r];
+            for (int r = 0; r < R; ++r)
+                if (k0 + r * kWallLanes < cnt) term(c[r].x, c[r].y, jb[r], q[r].x, q[r].y, q[r].z, q[r].w);
         }
     }
 #pragma unroll
@@ -143,67 +137,29 @@ __global__ void __launch_bounds__(kBlock) k_walls_iter(Buffers B)
     wall_slot<D, F32>(B, s, ls->iter & 1, sub, gmask);
 }
 
-// One entry of the pair cache in registers.
-template <typename T, int D, bool F32>
-struct CacheEntry {
-    T g[3];
-    T F;
-    uint32_t jb;
-    __device__ __forceinline__ void load(const Buffers &B, size_t e)
-    {
-        if (F32) {
-            const float4 c = B.pc32[e];
-            g[0] = (T)c.x;
-            g[1] = (T)c.y;
-            if (D == 3) {
-                g[2] = (T)c.z;
-                F = (T)c.w;
-                jb = B.pj[e];
-            } else {
-                g[2] = T(0);
-                F = (T)c.z;
-                jb = __float_as_uint(c.w);
-            }
-        } else {
-            const double4_32a c = B.pc64[e];
-            g[0] = (T)c.x;
-            g[1] = (T)c.y;
-            g[2] = (T)c.z;
-            F = (T)c.w;
-            jb = B.pj[e];
-        }
-    }
-};
-
-// Pair-cache rows of one warp in shared memory (one lane per slot). The 32 slots
-// of the warp form one slice of the sliced cache, so their entries k = 0, 1, ...
-// are consecutive rows (32 coefficient records, then, where the index is kept
-// apart, 32 indices). Chunks of kRows rows arrive by bulk copies into a ring of
-// S stages (S - 1 chunks in flight while one is used), each completing on its
-// stage's mbarrier. The ring of warp w sits at w * stride(S) in dynamic shared
-// memory: S stages, then S barriers.
-template <int D, bool F32>
-struct RowFmt {
-    static constexpr int kCoef = F32 ? 16 : 32;                 // bytes of one coefficient record
-    static constexpr bool kSepJ = !(F32 && D == 2);             // index in pj (2D FP32C: in .w)
-    static constexpr int kRows = F32 ? 4 : 2;                   // rows per chunk
-    static constexpr int kCoefRow = kWarp * kCoef;
-    static constexpr int kJRow = kSepJ ? kWarp * 4 : 0;
-    static constexpr int kStageBytes = kRows * (kCoefRow + kJRow);
-    static __host__ __device__ constexpr size_t stride(int S)
-    {
-        return ((size_t)S * kStageBytes + (size_t)S * 8 + 127) / 128 * 128;
-    }
-};
-
-// Dynamic shared memory of the one-lane kernels for S stages: one ring per warp.
-template <int D, bool F32>
-__host__ __device__ constexpr size_t ring_bytes(int S)
+// FP64: pair-cache rows of one warp in shared memory (one lane per slot). The 32
+// slots of the warp form one slice of the sliced cache, so their entries k = 0, 1,
+// ... are consecutive rows (32 coefficient records, and 32 indices apart). Chunks
+// of kRows rows arrive by bulk copies into a ring of S stages (S - 1 chunks in
+// flight while one is used), each completing on its stage's mbarrier. The ring of
+// warp w sits at w * kRingStride(S) in dynamic shared memory: S stages, then S
+// barriers. (The FP32C path has no ring: its rows go to registers.)
+constexpr int kRows = 2;                                     // rows per chunk
+constexpr int kCoefRow = kWarp * 32;                         // bytes of a row of coefficients
+constexpr int kJRow = kWarp * 4;                             // bytes of a row of indices
+constexpr int kStageBytes = kRows * (kCoefRow + kJRow);
+__host__ __device__ constexpr size_t ring_stride(int S)
 {
-    return RowFmt<D, F32>::stride(S) * (kBlock / kWarp);
+    return ((size_t)S * kStageBytes + (size_t)S * 8 + 127) / 128 * 128;
 }
 
-template <int D, bool F32>
+// Dynamic shared memory of the one-lane kernels for S stages: one ring per warp.
+template <bool F32>
+__host__ __device__ constexpr size_t ring_bytes(int S)
+{
+    return F32 ? 0 : ring_stride(S) * (kBlock / kWarp);
+}
+
 struct WarpRing {
     unsigned char *buf;    // stage st at buf + st * kStageBytes
     uint64_t *bar;         // S barriers
@@ -226,22 +182,20 @@ struct RingPos {
     bool ok = true;
 };
 
-// This warp's ring in dynamic shared memory (one-lane kernels only).
-template <int D, bool F32>
-__device__ __forceinline__ WarpRing<D, F32> warp_ring(int S)
+// This warp's ring in dynamic shared memory (one-lane FP64 kernels only).
+__device__ __forceinline__ WarpRing warp_ring(int S)
 {
-    using RF = RowFmt<D, F32>;
-    unsigned char *base = dyn_smem + (size_t)(threadIdx.x >> 5) * RF::stride(S);
-    return WarpRing<D, F32>{base, reinterpret_cast<uint64_t *>(base + (size_t)S * RF::kStageBytes), S};
+    unsigned char *base = dyn_smem + (size_t)(threadIdx.x >> 5) * ring_stride(S);
+    return WarpRing{base, reinterpret_cast<uint64_t *>(base + (size_t)S * kStageBytes), S};
 }
 
 // Initialises the mbarriers of every warp's ring (whole block, then syncs).
-template <int D, bool F32, int L>
+template <bool RING>
 __device__ __forceinline__ void ring_init(int S)
 {
-    if constexpr (L == 1) {
+    if constexpr (RING) {
         if ((threadIdx.x & 31) == 0) {
-            const WarpRing<D, F32> rg = warp_ring<D, F32>(S);
+            const WarpRing rg = warp_ring(S);
             for (int st = 0; st < S; ++st) mbar_init(&rg.bar[st], 1);
             mbar_fence_init();
         }
@@ -250,36 +204,23 @@ __device__ __forceinline__ void ring_init(int S)
 }
 
 // The prescribed velocity of list entry jb's particle if it is a wall particle
-// (the V_j of the divergence term; the packed copy of V^n of order A, in the
-// working precision), else zeros. Issued with the neighbour-state gathers.
-template <int D, bool F32, typename T>
-__device__ __forceinline__ void wall_velocity(const Buffers &B, uint32_t jb, T *vw)
+// (the V_j of the divergence term; the packed copy of V^n of order A), else zeros.
+// Issued with the neighbour-state gathers.
+template <int D>
+__device__ __forceinline__ void wall_velocity(const Buffers &B, uint32_t jb, double *vw)
 {
-    vw[0] = vw[1] = vw[2] = T(0);
+    vw[0] = vw[1] = vw[2] = 0.0;
     if (!(jb & kWallBit)) return;
     const int j = (int)(jb & ~kWallBit);
-    if constexpr (F32) {
-        if (D == 2) {
-            const float2 w = *reinterpret_cast<const float2 *>(&B.wv32[j]);
-            vw[0] = (T)w.x;
-            vw[1] = (T)w.y;
-        } else {
-            const float4 w = B.wv32[j];
-            vw[0] = (T)w.x;
-            vw[1] = (T)w.y;
-            vw[2] = (T)w.z;
-        }
+    if (D == 2) {
+        const double2 w = *reinterpret_cast<const double2 *>(&B.wv64[j]);
+        vw[0] = w.x;
+        vw[1] = w.y;
     } else {
-        if (D == 2) {
-            const double2 w = *reinterpret_cast<const double2 *>(&B.wv64[j]);
-            vw[0] = (T)w.x;
-            vw[1] = (T)w.y;
-        } else {
-            const double4_32a w = B.wv64[j];
-            vw[0] = (T)w.x;
-            vw[1] = (T)w.y;
-            vw[2] = (T)w.z;
-        }
+        const double4_32a w = B.wv64[j];
+        vw[0] = w.x;
+        vw[1] = w.y;
+        vw[2] = w.z;
     }
 }
 
@@ -287,134 +228,213 @@ __device__ __forceinline__ void wall_velocity(const Buffers &B, uint32_t jb, T *
 template <bool F32>
 using Real = typename std::conditional<F32, float, double>::type;
 
-// Phase 1 of an iteration for slot s: L lanes per particle split its cached pair
-// list (lane l takes entries l, l+L, ...), accumulate the two rates
-// (Kahan-compensated FP32 on the FP32C path) and merge their partial sums with
-// warp shuffles; with one lane the warp's rows stream through the warp's
-// shared-memory ring. The rates, in the working precision, are valid on lane
-// lane_in = 0 of the particle's group.
-template <int D, bool F32, bool WALLS, int L, bool FA = false>
-__device__ __forceinline__ void pair_sums(const Buffers &B, const Phys &P, const Geom &G, int cur, int s, int lane_in,
-                                          bool active, RingPos &rp, Real<F32> &apT, Real<F32> *FT)
+// The shift table of the uncached FP32C form and the geometry of the uncached
+// FP64 form, per block.
+struct FormGeom {
+    float4 sh[kCodes];
+    Geom G;
+};
+
+// Loads what the uncached form needs of instance inst (whole block; sync after).
+template <bool F32, bool FA>
+__device__ __forceinline__ void load_form_geom(const Buffers &B, int inst, FormGeom &fg)
 {
-    using T = typename std::conditional<F32, float, double>::type;
-    using Acc = typename std::conditional<F32, Kahan, Plain64>::type;
-    const PairConst<T> k = pair_const<T>(P);
-    T vi[3] = {T(0), T(0), T(0)}, pi = T(0);
+    if constexpr (FA && F32) {
+        if (threadIdx.x < kCodes) fg.sh[threadIdx.x] = code_shift(B.geo[inst], threadIdx.x);
+    } else if constexpr (FA) {
+        for (int w = threadIdx.x; w < (int)(sizeof(Geom) / 4); w += blockDim.x)
+            reinterpret_cast<int *>(&fg.G)[w] = reinterpret_cast<const int *>(B.geo + inst)[w];
+    }
+}
+
+// Phase 1 of an iteration for slot s, FP32C (pair32.cuh): the particle's L lanes
+// share its pairs of list entries (lane l takes pairs l, l + L, ...); the rates
+// are valid on every lane of the group. FA: the geometry recomputed from the
+// lists, with the cache pass's operations, so that both forms give the same bits.
+//
+// With the cache, the warp's rows are consecutive: 2 KB (2D) or 2.5 KB (3D) per
+// round of two pairs. With one lane per particle they go to registers, the next
+// round's loads issued before this round's gathers and arithmetic, and a cache
+// that exceeds L2 is prefetched into it B.stages rounds ahead by one bulk
+// instruction a round. (The earlier shared-memory ring of bulk copies took its
+// space from the L1 that serves the neighbour gathers and a wait and a shared read
+// per row: 128^3 0.975 ms an iteration, now 0.882 ms, of 0.70 ms at the HBM rate;
+// the 64-vortex batch 0.228, now 0.210 ms. Without the cache, where the packed
+// arithmetic halved the instructions: 1.335, now 1.242 ms, and 0.299, now 0.255
+// ms, bound by the gathers' L1 tag lookups, about 18 lines a request.)
+template <int D, bool WALLS, int L, bool FA>
+__device__ __forceinline__ void pair_sums32(const Buffers &B, const Phys &P, const FormGeom &fg, int cur, int s,
+                                            int lane_in, bool active, float &apT, float *FT)
+{
+    const PairK32 k = P.k32;
+    const float4 *nb = B.nb32[cur];
+    float vi[3] = {0.f, 0.f, 0.f}, pi = 0.f;
     int cnt = 0;
     if (active) {
-        if (F32) {
-            float4 q = B.nb32[cur][s];
-            vi[0] = q.x; vi[1] = q.y; vi[2] = q.z; pi = q.w;
-        } else {
-            double4_32a q = B.nb64[cur][s];
-            vi[0] = (T)q.x; vi[1] = (T)q.y; vi[2] = (T)q.z; pi = (T)q.w;
-        }
+        const float4 q = nb[s];
+        vi[0] = q.x; vi[1] = q.y; vi[2] = q.z; pi = q.w;
         cnt = B.pcount[s];
     }
-    Acc ap, Fa[3];
-    // the pair terms of one cache entry with its gathered neighbour state
-    using Q = typename std::conditional<F32, float4, double4_32a>::type;
-    const Q *nbq = F32 ? (const Q *)(const void *)B.nb32[cur] : (const Q *)(const void *)B.nb64[cur];
-    // vw: the prescribed velocity of a wall neighbour (the divergence term's
-    // V_j), gathered with the neighbour states
-    // (one call for both kinds of neighbour: a warp whose lanes hold both runs
-    // the pair arithmetic once)
-    auto pair = [&](const CacheEntry<T, D, F32> &ce, const Q &q, const T *vw) {
-        const T vj[3] = {(T)q.x, (T)q.y, (T)q.z};
-        const T pj = (T)q.w;
-        if constexpr (WALLS) {
-            const bool wall = (ce.jb & kWallBit) != 0;
-            const T vd[3] = {wall ? vw[0] : vj[0], wall ? vw[1] : vj[1], wall ? vw[2] : vj[2]};
-            pair_accumulate<D, T, Acc>(k, ce.g, ce.F, vi, pi, vd, vj, pj, ap, Fa);
-        } else {
-            pair_accumulate<D, T, Acc>(k, ce.g, ce.F, vi, pi, vj, vj, pj, ap, Fa);
+    Sums32<D> A;
+    auto wall = [&](uint32_t e, const float4 &q, float *w) {
+        w[0] = q.x; w[1] = q.y; w[2] = q.z;
+        if (e & kWallBit) {
+            const float4 v = B.wv32[e & ~kWallBit];
+            w[0] = v.x; w[1] = v.y; w[2] = v.z;
         }
     };
     if constexpr (FA) {
-        // Form A: the geometry of every pair recomputed from the lists at r^0
-        // with k_pair_cache's operations (offset_sep or listed_sep, then
-        // grad_coef), so every coefficient has the bits the cache would hold and
-        // both forms give the same results; the entries keep the order of the
-        // cached rows (lane l takes l, l + L, ..., R in flight per round)
         static_assert(!WALLS, "the wall values come from the cache");
-        const uint32_t *lst = slot_list(B, s);
-        const float4 oi = F32 && active ? B.off[s] : make_float4(0.f, 0.f, 0.f, 0.f);
-        constexpr int R = 4;
-        for (int q0 = lane_in; q0 < cnt; q0 += L * R) {
-            uint32_t jbv[R];
-            if constexpr (L == 1) {
-                // four consecutive entries in one 16-byte load; an entry past the
-                // count repeats entry q0, so its gathers stay in bounds
-                const uint4 v = *reinterpret_cast<const uint4 *>(lst + q0);
-                jbv[0] = v.x;
-                jbv[1] = q0 + 1 < cnt ? v.y : v.x;
-                jbv[2] = q0 + 2 < cnt ? v.z : v.x;
-                jbv[3] = q0 + 3 < cnt ? v.w : v.x;
-            } else {
-#pragma unroll
-                for (int r = 0; r < R; ++r) jbv[r] = lst[min(q0 + r * L, cnt - 1)];
-            }
-            float4 ov[R];
-            Q qv[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int j = entry_slot(jbv[r]);
-                ov[r] = F32 ? B.off[j] : make_float4(0.f, 0.f, 0.f, 0.f);
-                qv[r] = nbq[j];
-            }
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                if (q0 + r * L >= cnt) break;
-                const int code = entry_code(jbv[r]);
-                T d[3], r2;
-                if constexpr (F32) {
-                    offset_sep<D, T>(G, oi, ov[r], code, d, r2);
-                } else {
-                    int dx, dy, dz;
-                    decode_shift(code, dx, dy, dz);
-                    listed_sep<D, F32, T>(G, B.xp_a, B.off, B.n, s, entry_slot(jbv[r]), oi, dx, dy, dz, d, r2);
-                }
-                T g[3], F;
-                grad_coef<D, T>(P, d, r2, g, F);
-                CacheEntry<T, D, F32> ce;
-                ce.g[0] = g[0];
-                ce.g[1] = g[1];
-                ce.g[2] = D == 3 ? g[2] : T(0);
-                ce.F = F;
-                ce.jb = jbv[r] & ~kCodeMask;
-                pair(ce, qv[r], nullptr);
-            }
-        }
-    } else if constexpr (L == 1) {
-        // the warp's rows stream through its shared-memory ring; the
-        // neighbour states of a chunk's rows are gathered together
-        using RF = RowFmt<D, F32>;
-        constexpr int R = RF::kRows;
-        const int S = B.stages;
-        constexpr unsigned full = 0xffffffffu;
-        const int lane = threadIdx.x & 31;
-        const WarpRing<D, F32> rg = warp_ring<D, F32>(S);
-        const int cmax = __reduce_max_sync(full, cnt);
-        const int nch = rp.ok ? (cmax + R - 1) / R : 0;
-        const size_t row0 = (size_t)(s >> 5) * B.K;      // first row of the warp's slice
-        const unsigned char *gcoef =
-            (F32 ? (const unsigned char *)B.pc32 : (const unsigned char *)B.pc64) + row0 * RF::kCoefRow;
-        const unsigned char *gj = (const unsigned char *)B.pj + row0 * (kWarp * 4);
+        const float4 oi = active ? B.off[s] : make_float4(0.f, 0.f, 0.f, 0.f);
+        list_sums32<D, false, L>(k, fg.sh, slot_list(B, s), cnt, lane_in, oi, vi, pi, B.off, nb, wall, A);
+    } else {
         // a cache larger than L2 streams through it once per pass (first to
         // leave); a smaller one stays like the rest; the neighbour states,
         // gathered again every pass, stay
         const uint64_t pol_stream = B.l2_stream ? l2_policy_evict_first() : l2_policy_evict_normal();
         const uint64_t pol_keep = l2_policy_evict_last();
+        const int np = list_pairs(cnt);
+        const size_t row0 = cache_row(B, s);
+        // the terms of two records (pairs m and, if `two`, another)
+        auto terms = [&](const CachePair &r, const CachePair &t, bool two) {
+            float4 q[4];
+            float w[4][3];
+            const uint32_t e[4] = {r.ea, r.eb, t.ea, t.eb};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                q[i] = ld_f4_hint(nb + (WALLS ? e[i] & ~kWallBit : e[i]), pol_keep);
+                if constexpr (WALLS) wall(e[i], q[i], w[i]);
+            }
+            F2 g[D], F;
+            cache_coefs<D>(r, g, F);
+            pair2_accumulate<D, WALLS>(k, g, F, vi, pi, q[0], q[1], w[0], w[1], A);
+            if (!two) return;
+            cache_coefs<D>(t, g, F);
+            pair2_accumulate<D, WALLS>(k, g, F, vi, pi, q[2], q[3], w[2], w[3], A);
+        };
+        auto load = [&](int m) { return cache_pair_stream<D>(B, row0 + m, s & 31, pol_stream); };
+        if constexpr (L == 1) {
+            const int nr = np / 2;                       // rounds of two pairs
+            const int lead = B.l2_stream ? B.stages : 0;
+            const int nw = lead ? __reduce_max_sync(0xffffffffu, nr) : 0;   // the warp's rounds
+            auto ahead = [&](int t) {                    // rounds t.. of the warp into L2
+                if (t < nw && (threadIdx.x & 31) == 0) {
+                    l2_prefetch(B.pc32 + (row0 + 2 * t) * 2 * kWarp, 4 * kWarp * 16, pol_stream);
+                    if constexpr (D == 3)
+                        l2_prefetch(reinterpret_cast<const uint2 *>(B.pj) + (row0 + 2 * t) * kWarp, 2 * kWarp * 8, pol_stream);
+                }
+            };
+            for (int t = 1; t < lead; ++t) ahead(t);
+            CachePair a0, a1, b0, b1;
+            if (nr > 0) {
+                a0 = load(0);
+                a1 = load(1);
+            }
+            for (int t = 0; t < nr; t += 2) {
+                if (lead) ahead(t + lead);
+                if (t + 1 < nr) {
+                    b0 = load(2 * t + 2);
+                    b1 = load(2 * t + 3);
+                }
+                terms(a0, a1, true);
+                if (t + 1 >= nr) break;
+                if (lead) ahead(t + 1 + lead);
+                if (t + 2 < nr) {
+                    a0 = load(2 * t + 4);
+                    a1 = load(2 * t + 5);
+                }
+                terms(b0, b1, true);
+            }
+        } else {
+            for (int m = lane_in; m < np; m += 2 * L) {
+                const bool two = m + L < np;
+                const CachePair r = load(m), t = load(two ? m + L : m);
+                terms(r, t, two);
+            }
+        }
+    }
+    rates32<D, L>(k, A, apT, FT);
+}
+
+// Phase 1 of an iteration for slot s, FP64: L lanes per particle split its cached
+// pair list (lane l takes entries l, l+L, ...), accumulate the two rates and
+// merge their partial sums with warp shuffles; with one lane the warp's rows stream
+// through the warp's shared-memory ring. The rates are valid on lane lane_in = 0
+// of the particle's group.
+template <int D, bool WALLS, int L, bool FA>
+__device__ __forceinline__ void pair_sums64(const Buffers &B, const Phys &P, const FormGeom &fg, int cur, int s,
+                                            int lane_in, bool active, RingPos &rp, double &apT, double *FT)
+{
+    const PairConst<double> k = pair_const<double>(P);
+    const double4_32a *nb = B.nb64[cur];
+    double vi[3] = {0, 0, 0}, pi = 0;
+    int cnt = 0;
+    if (active) {
+        const double4_32a q = nb[s];
+        vi[0] = q.x; vi[1] = q.y; vi[2] = q.z; pi = q.w;
+        cnt = B.pcount[s];
+    }
+    Plain64 ap, Fa[3];
+    // the terms of one entry with its gathered neighbour state; vw: the prescribed
+    // velocity of a wall neighbour (the divergence term's V_j), gathered with the
+    // neighbour states (one call for both kinds of neighbour: a warp whose lanes
+    // hold both runs the pair arithmetic once)
+    auto pair = [&](const double *g, double F, uint32_t jb, const double4_32a &q, const double *vw) {
+        const double vj[3] = {q.x, q.y, q.z};
+        if constexpr (WALLS) {
+            const bool wall = (jb & kWallBit) != 0;
+            const double vd[3] = {wall ? vw[0] : vj[0], wall ? vw[1] : vj[1], wall ? vw[2] : vj[2]};
+            pair_accumulate<D, double, Plain64>(k, g, F, vi, pi, vd, vj, q.w, ap, Fa);
+        } else {
+            pair_accumulate<D, double, Plain64>(k, g, F, vi, pi, vj, vj, q.w, ap, Fa);
+        }
+    };
+    constexpr int R = 4;
+    if constexpr (FA) {
+        // Form A: the geometry of every pair recomputed from the lists at r^0
+        // with k_pair_cache's operations, so every coefficient has the bits the
+        // cache would hold; the entries keep the order of the cached rows (lane l
+        // takes l, l + L, ..., R in flight per round)
+        static_assert(!WALLS, "the wall values come from the cache");
+        const uint32_t *lst = slot_list(B, s);
+        for (int q0 = lane_in; q0 < cnt; q0 += L * R) {
+            uint32_t jbv[R];
+            double4_32a qv[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) jbv[r] = lst[min(q0 + r * L, cnt - 1)];
+#pragma unroll
+            for (int r = 0; r < R; ++r) qv[r] = nb[entry_slot(jbv[r])];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if (q0 + r * L >= cnt) break;
+                double d[3], r2, g[3], F;
+                r2 = sep64<D>(fg.G, B.xp_a, B.n, s, entry_slot(jbv[r]), d);
+                grad_coef<D, double>(P, d, r2, g, F);
+                pair(g, F, jbv[r], qv[r], nullptr);
+            }
+        }
+    } else if constexpr (L == 1) {
+        // the warp's rows stream through its shared-memory ring; the neighbour
+        // states of a chunk's rows are gathered together
+        constexpr int R = kRows;
+        const int S = B.stages;
+        constexpr unsigned full = 0xffffffffu;
+        const int lane = threadIdx.x & 31;
+        const WarpRing rg = warp_ring(S);
+        const int cmax = __reduce_max_sync(full, cnt);
+        const int nch = rp.ok ? (cmax + R - 1) / R : 0;
+        const size_t row0 = (size_t)(s >> 5) * B.K;      // first row of the warp's slice
+        const unsigned char *gcoef = (const unsigned char *)B.pc64 + row0 * kCoefRow;
+        const unsigned char *gj = (const unsigned char *)B.pj + row0 * kJRow;
+        const uint64_t pol_stream = B.l2_stream ? l2_policy_evict_first() : l2_policy_evict_normal();
         auto issue = [&](int c) {        // lane 0: chunk c into its stage
             const int st = (int)((rp.pos + (uint32_t)c) % (uint32_t)S);
             const int r0 = c * R, nr = min(R, cmax - r0);
-            const uint32_t bc = (uint32_t)(nr * RF::kCoefRow), bj = (uint32_t)(nr * RF::kJRow);
-            unsigned char *stg = rg.buf + (size_t)st * RF::kStageBytes;
+            const uint32_t bc = (uint32_t)(nr * kCoefRow), bj = (uint32_t)(nr * kJRow);
+            unsigned char *stg = rg.buf + (size_t)st * kStageBytes;
             mbar_arrive_expect_tx(&rg.bar[st], bc + bj);
-            bulk_g2s_hint(stg, gcoef + (size_t)r0 * RF::kCoefRow, bc, &rg.bar[st], pol_stream);
-            if (RF::kSepJ)
-                bulk_g2s_hint(stg + R * RF::kCoefRow, gj + (size_t)r0 * RF::kJRow, bj, &rg.bar[st], pol_stream);
+            bulk_g2s_hint(stg, gcoef + (size_t)r0 * kCoefRow, bc, &rg.bar[st], pol_stream);
+            bulk_g2s_hint(stg + R * kCoefRow, gj + (size_t)r0 * kJRow, bj, &rg.bar[st], pol_stream);
         };
         if (lane == 0)
             for (int c = 0; c < S && c < nch; ++c) issue(c);
@@ -424,44 +444,26 @@ __device__ __forceinline__ void pair_sums(const Buffers &B, const Phys &P, const
             const int st = (int)(q % (uint32_t)S);
             if (!mbar_wait(&rg.bar[st], (q / (uint32_t)S) & 1u)) break;
             const int r0 = c * R, nr = min(R, cmax - r0);
-            const unsigned char *stg = rg.buf + (size_t)st * RF::kStageBytes;
+            const unsigned char *stg = rg.buf + (size_t)st * kStageBytes;
             // gather the neighbour states of the chunk's rows first (R loads
             // in flight per lane), then run the pair terms
             uint32_t jbv[R];
-            Q qv[R];
-            T wv[R][3];
+            double4_32a qv[R];
+            double wv[R][3];
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 if (r < nr && r0 + r < cnt) {
-                    jbv[r] = RF::kSepJ
-                                 ? ((const uint32_t *)(stg + R * RF::kCoefRow + r * RF::kJRow))[lane]
-                                 : __float_as_uint(((const float4 *)(stg + r * RF::kCoefRow))[lane].w);
-                    if constexpr (F32)
-                        qv[r] = ld_f4_hint(reinterpret_cast<const float4 *>(nbq) + (jbv[r] & ~kWallBit), pol_keep);
-                    else
-                        qv[r] = nbq[jbv[r] & ~kWallBit];
-                    if constexpr (WALLS) wall_velocity<D, F32, T>(B, jbv[r], wv[r]);
+                    jbv[r] = ((const uint32_t *)(stg + R * kCoefRow + r * kJRow))[lane];
+                    qv[r] = nb[jbv[r] & ~kWallBit];
+                    if constexpr (WALLS) wall_velocity<D>(B, jbv[r], wv[r]);
                 }
             }
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 if (r < nr && r0 + r < cnt) {
-                    CacheEntry<T, D, F32> ce;
-                    if (F32) {
-                        const float4 v = ((const float4 *)(stg + r * RF::kCoefRow))[lane];
-                        ce.g[0] = (T)v.x;
-                        ce.g[1] = (T)v.y;
-                        ce.g[2] = D == 3 ? (T)v.z : T(0);
-                        ce.F = D == 3 ? (T)v.w : (T)v.z;
-                    } else {
-                        const double4_32a v = ((const double4_32a *)(stg + r * RF::kCoefRow))[lane];
-                        ce.g[0] = (T)v.x;
-                        ce.g[1] = (T)v.y;
-                        ce.g[2] = (T)v.z;
-                        ce.F = (T)v.w;
-                    }
-                    ce.jb = jbv[r];
-                    pair(ce, qv[r], wv[r]);
+                    const double4_32a v = ((const double4_32a *)(stg + r * kCoefRow))[lane];
+                    const double g[3] = {v.x, v.y, v.z};
+                    pair(g, v.w, jbv[r], qv[r], wv[r]);
                 }
             }
             __syncwarp();
@@ -487,21 +489,28 @@ __device__ __forceinline__ void pair_sums(const Buffers &B, const Phys &P, const
         // R entries per round: their cache entries, then their neighbour
         // gathers, then the pair terms, so R loads of each kind are in flight
         // per lane (the entries keep the order lane_in, lane_in + L, ...)
-        constexpr int R = 4;
         for (int k0 = lane_in; k0 < cnt; k0 += L * R) {
-            CacheEntry<T, D, F32> ce[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) ce[r].load(B, base + (size_t)min(k0 + r * L, cnt - 1) * kWarp);
-            Q qv[R];
-            T wv[R][3];
+            double4_32a ce[R];
+            uint32_t jb[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                qv[r] = nbq[ce[r].jb & ~kWallBit];
-                if constexpr (WALLS) wall_velocity<D, F32, T>(B, ce[r].jb, wv[r]);
+                const size_t e = base + (size_t)min(k0 + r * L, cnt - 1) * kWarp;
+                ce[r] = B.pc64[e];
+                jb[r] = B.pj[e];
+            }
+            double4_32a qv[R];
+            double wv[R][3];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                qv[r] = nb[jb[r] & ~kWallBit];
+                if constexpr (WALLS) wall_velocity<D>(B, jb[r], wv[r]);
             }
 #pragma unroll
             for (int r = 0; r < R; ++r)
-                if (k0 + r * L < cnt) pair(ce[r], qv[r], wv[r]);
+                if (k0 + r * L < cnt) {
+                    const double g[3] = {ce[r].x, ce[r].y, ce[r].z};
+                    pair(g, ce[r].w, jb[r], qv[r], wv[r]);
+                }
         }
     }
 #pragma unroll
@@ -510,9 +519,9 @@ __device__ __forceinline__ void pair_sums(const Buffers &B, const Phys &P, const
 #pragma unroll
         for (int a = 0; a < D; ++a) Fa[a].shfl_merge(o);
     }
-    apT = (T)ap.value();
+    apT = ap.value();
 #pragma unroll
-    for (int a = 0; a < D; ++a) FT[a] = (T)Fa[a].value();
+    for (int a = 0; a < D; ++a) FT[a] = Fa[a].value();
 }
 
 // Phase 2 of an iteration: the BDF2 pseudo-acceleration and update, FP64
@@ -594,7 +603,7 @@ __device__ __forceinline__ void update_and_residuals(const Buffers &B, const Phy
 // work runs with every lane busy); with one lane per particle that thread is the
 // particle's phase-1 lane, so the rates stay in registers.
 template <int D, bool F32, bool WALLS, int L, bool FA = false>
-__device__ __forceinline__ void tile_iteration(const Buffers &B, const Phys &P, const Geom &G, int cur, int tile,
+__device__ __forceinline__ void tile_iteration(const Buffers &B, const Phys &P, const FormGeom &fg, int cur, int tile,
                                                TileShared<typename std::conditional<F32, float, double>::type, D, L> &sh,
                                                RingPos &rp, double &blk_ap, double &blk_av)
 {
@@ -606,7 +615,8 @@ __device__ __forceinline__ void tile_iteration(const Buffers &B, const Phys &P, 
     const int s = tile * PPB + grp;
     const bool active = s < n && B.gid_a[s] < (uint32_t)B.nf;   // fluid (not wall, not padding)
     T apT = T(0), FT[3] = {T(0), T(0), T(0)};
-    pair_sums<D, F32, WALLS, L, FA>(B, P, G, cur, s, lane_in, active, rp, apT, FT);
+    if constexpr (F32) pair_sums32<D, WALLS, L, FA>(B, P, fg, cur, s, lane_in, active, apT, FT);
+    else pair_sums64<D, WALLS, L, FA>(B, P, fg, cur, s, lane_in, active, rp, apT, FT);
     double w_ap = 0, w_av = 0;
     if constexpr (L == 1) {
         update_and_residuals<D, F32>(B, P, cur, s, active, apT, FT, w_ap, w_av);
@@ -648,20 +658,19 @@ __device__ __forceinline__ void tile_iteration(const Buffers &B, const Phys &P, 
 // applies its stop rules; the last block of all sets the while-node condition
 // (some instance still iterating).
 template <int D, bool F32, bool WALLS, int L, bool FA = false>
-__global__ void __launch_bounds__(kBlock, L == 1 && !FA ? (F32 ? (D == 2 ? 4 : 3) : 1) : (F32 ? 3 : 1))
+__global__ void __launch_bounds__(kBlock, F32 ? (L == 1 && !FA && D == 3 ? 2 : 3) : 1)
     k_iterate(Buffers B, unsigned long long cond, int use_cond)
 {
     using T = typename std::conditional<F32, float, double>::type;
     constexpr int PPB = kBlock / L;
     __shared__ TileShared<T, D, L> sh;
     __shared__ Phys P;
-    __shared__ Geom G;
+    __shared__ FormGeom fg;
     __shared__ int last, tlo_sh;
     if (!use_cond && B.ctrl->active == 0) return;     // whole grid agrees: nothing to do
-    // (ring_init ends with the barrier that publishes thread 0's set-up of the
-    // block's shared state; without the ring the barrier stays)
-    if constexpr (!FA) ring_init<D, F32, L>(B.stages);
-    else __syncthreads();
+    // (ends with the barrier that publishes thread 0's set-up of the block's
+    // shared state, ring or not)
+    ring_init<!F32 && L == 1 && !FA>(B.stages);
     RingPos rp;
     const int inst = block_instance(B, blockIdx.x * PPB);
     LoopState *ls = B.ls + inst;
@@ -673,12 +682,10 @@ __global__ void __launch_bounds__(kBlock, L == 1 && !FA ? (F32 ? (D == 2 ? 4 : 3
     if (work) {
         for (int w = threadIdx.x; w < (int)(sizeof(Phys) / 4); w += blockDim.x)
             reinterpret_cast<int *>(&P)[w] = reinterpret_cast<const int *>(B.phys + inst)[w];
-        if constexpr (FA)
-            for (int w = threadIdx.x; w < (int)(sizeof(Geom) / 4); w += blockDim.x)
-                reinterpret_cast<int *>(&G)[w] = reinterpret_cast<const int *>(B.geo + inst)[w];
+        load_form_geom<F32, FA>(B, inst, fg);
         __syncthreads();
         double a = 0, b = 0;
-        tile_iteration<D, F32, WALLS, L, FA>(B, P, G, it & 1, blockIdx.x, sh, rp, a, b);
+        tile_iteration<D, F32, WALLS, L, FA>(B, P, fg, it & 1, blockIdx.x, sh, rp, a, b);
         if (threadIdx.x == 0) {
             B.blk[2 * blockIdx.x] = a;
             B.blk[2 * blockIdx.x + 1] = b;
@@ -820,7 +827,7 @@ __device__ __forceinline__ int dealt_instance(const int *pre, int ni, int k)
 // decisions; tiles of finished instances are skipped. Walls get their own phase
 // and barrier before the fluid phase.
 template <int D, bool F32, bool WALLS, int L, bool FA = false>
-__global__ void __launch_bounds__(kBlock, L == 1 && !FA ? ((F32 && D == 2 && !WALLS) ? 4 : 3) : (F32 ? 3 : 2))
+__global__ void __launch_bounds__(kBlock, F32 ? (L == 1 && !FA && D == 3 ? 2 : 3) : L == 1 && !FA ? 3 : 2)
     k_loop(Buffers B)
 {
     using T = typename std::conditional<F32, float, double>::type;
@@ -828,7 +835,7 @@ __global__ void __launch_bounds__(kBlock, L == 1 && !FA ? ((F32 && D == 2 && !WA
     __shared__ TileShared<T, D, L> sh;
     __shared__ LoopState st;
     __shared__ Phys P;
-    __shared__ Geom G;
+    __shared__ FormGeom fg;
     __shared__ int stop, ok_sh, p_inst;
     __shared__ int act_pre[kDealMaxInst + 1];
     if constexpr (!WALLS) {
@@ -842,10 +849,9 @@ __global__ void __launch_bounds__(kBlock, L == 1 && !FA ? ((F32 && D == 2 && !WA
         stop = 0;
         p_inst = -1;
     }
-    // (ring_init ends with the barrier that publishes thread 0's set-up of the
-    // block's shared state; without the ring the barrier stays)
-    if constexpr (!FA) ring_init<D, F32, L>(B.stages);
-    else __syncthreads();
+    // (ends with the barrier that publishes thread 0's set-up of the block's
+    // shared state, ring or not)
+    ring_init<!F32 && L == 1 && !FA>(B.stages);
     RingPos rp;
     unsigned int epoch = 0;
     // (one instance: from the loop state's iteration, 0 at the start of a step,
@@ -888,14 +894,12 @@ __global__ void __launch_bounds__(kBlock, L == 1 && !FA ? ((F32 && D == 2 && !WA
                 __syncthreads();
                 for (int w = threadIdx.x; w < (int)(sizeof(Phys) / 4); w += blockDim.x)
                     reinterpret_cast<int *>(&P)[w] = reinterpret_cast<const int *>(B.phys + inst)[w];
-                if constexpr (FA)
-                    for (int w = threadIdx.x; w < (int)(sizeof(Geom) / 4); w += blockDim.x)
-                        reinterpret_cast<int *>(&G)[w] = reinterpret_cast<const int *>(B.geo + inst)[w];
+                load_form_geom<F32, FA>(B, inst, fg);
                 __syncthreads();
                 if (threadIdx.x == 0) p_inst = inst;
             }
             double a = 0, b = 0;
-            tile_iteration<D, F32, WALLS, L, FA>(B, P, G, cur, t, sh, rp, a, b);
+            tile_iteration<D, F32, WALLS, L, FA>(B, P, fg, cur, t, sh, rp, a, b);
             if (threadIdx.x == 0) {
                 blk[2 * t] = a;
                 blk[2 * t + 1] = b;
@@ -985,24 +989,23 @@ __device__ __forceinline__ int block_min(int v, int *scratch)
 // tile and every decision is computed as in k_loop, so the results are the
 // same bits.
 template <int D, bool F32, int L, bool FA = false>
-__global__ void __launch_bounds__(kBlock, L == 1 && !FA ? ((F32 && D == 2) ? 4 : 3) : (F32 ? 3 : 2))
+__global__ void __launch_bounds__(kBlock, F32 ? (L == 1 && !FA && D == 3 ? 2 : 3) : L == 1 && !FA ? 3 : 2)
     k_loop_async(Buffers B)
 {
     using T = typename std::conditional<F32, float, double>::type;
     constexpr int PPB = kBlock / L;
     __shared__ TileShared<T, D, L> sh;
     __shared__ Phys P;
-    __shared__ Geom G;
+    __shared__ FormGeom fg;
     __shared__ int p_inst, w_inst, w_tile, w_it, last_sh, quit;
     __shared__ int mins[kBlock / kWarp];
     if (skip_form(B)) return;         // the step runs the other pair-term form
     const int ntiles = (B.n + PPB - 1) / PPB;
     const int ni = B.ninst;
     if (threadIdx.x == 0) p_inst = -1;
-    // (ring_init ends with the barrier that publishes thread 0's set-up of the
-    // block's shared state; without the ring the barrier stays)
-    if constexpr (!FA) ring_init<D, F32, L>(B.stages);
-    else __syncthreads();
+    // (ends with the barrier that publishes thread 0's set-up of the block's
+    // shared state, ring or not)
+    ring_init<!F32 && L == 1 && !FA>(B.stages);
     RingPos rp;
     unsigned long long wait_from = 0;
     bool waiting = false;
@@ -1065,14 +1068,12 @@ __global__ void __launch_bounds__(kBlock, L == 1 && !FA ? ((F32 && D == 2) ? 4 :
         if (inst != p_inst) {
             for (int w = threadIdx.x; w < (int)(sizeof(Phys) / 4); w += blockDim.x)
                 reinterpret_cast<int *>(&P)[w] = reinterpret_cast<const int *>(B.phys + inst)[w];
-            if constexpr (FA)
-                for (int w = threadIdx.x; w < (int)(sizeof(Geom) / 4); w += blockDim.x)
-                    reinterpret_cast<int *>(&G)[w] = reinterpret_cast<const int *>(B.geo + inst)[w];
+            load_form_geom<F32, FA>(B, inst, fg);
             __syncthreads();
             if (threadIdx.x == 0) p_inst = inst;
         }
         double a = 0, b = 0;
-        tile_iteration<D, F32, false, L, FA>(B, P, G, it & 1, t, sh, rp, a, b);
+        tile_iteration<D, F32, false, L, FA>(B, P, fg, it & 1, t, sh, rp, a, b);
         int tlo, thi;
         instance_tiles(B.inst[inst], PPB, tlo, thi);
         double *blk = B.blk + (size_t)(it & 1) * 2 * ntiles;

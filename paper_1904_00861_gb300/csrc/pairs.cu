@@ -7,6 +7,7 @@
 // under the distance test, which most candidates fail.
 #include "geometry.cuh"
 #include "loop_rules.cuh"
+#include "pair32.cuh"
 
 namespace dtsph {
 
@@ -94,11 +95,12 @@ template <int D, bool F32, bool PRED, bool WALLS, int L>
 __global__ void __launch_bounds__(kBlock, F32 ? (D == 2 ? 4 : 3) : 1) k_state_n(Buffers B)
 {
     using T = typename std::conditional<F32, float, double>::type;
-    using Acc = typename std::conditional<F32, Kahan, Plain64>::type;
     constexpr int SPB = kBlock / L;
     __shared__ Geom G;
     __shared__ Phys P;
+    __shared__ float4 sh[kCodes];
     const int inst = block_instance(B, blockIdx.x * SPB);
+    if (F32 && threadIdx.x < kCodes) sh[threadIdx.x] = code_shift(B.geo[inst], threadIdx.x);
     block_copy(G, B.geo[inst]);
     block_copy(P, B.phys[inst]);
     const int n = B.n;
@@ -106,77 +108,63 @@ __global__ void __launch_bounds__(kBlock, F32 ? (D == 2 ? 4 : 3) : 1) k_state_n(
     // every lane stays to the end: the partial sums are merged by full-warp shuffles
     const uint32_t gs = s < n ? B.gid_b[s] : kNoParticle;
     const bool fluid = gs < (uint32_t)B.nf;
-    const auto *nb = nb_ptr<T>(B, 1);
-    const PairConst<T> k = pair_const<T>(P);
-    Acc ap, Fa[3];
-    {
-        const typename Packed<T>::type qi = fluid ? nb[s] : typename Packed<T>::type{};
-        const T vi[3] = {(T)qi.x, (T)qi.y, (T)qi.z};
-        const T pi = (T)qi.w;
-        const float4 oi = F32 && fluid ? B.off[s] : make_float4(0, 0, 0, 0);
-        const uint32_t *lst = slot_list(B, s);
-        const int cnt = fluid ? B.pcount[s] : 0;
-        // R entries per round: their indices, then their gathers (neighbour
-        // state and, FP32C, offset), then the pair terms, so that R loads are in
-        // flight per lane; the entries keep their order
+    T apT = T(0), FT[3] = {T(0), T(0), T(0)};
+    const int cnt = fluid ? B.pcount[s] : 0;
+    const uint32_t *lst = slot_list(B, s);
+    if constexpr (F32) {
+        const PairK32 k = P.k32;
+        const float4 *nb = B.nb32[1];
+        const float4 qi = fluid ? nb[s] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 oi = fluid ? B.off[s] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float vi[3] = {qi.x, qi.y, qi.z};
+        auto wall = [&](uint32_t e, const float4 &q, float *w) {
+            w[0] = q.x; w[1] = q.y; w[2] = q.z;
+            if (e & kWallBit)
+                for (int a = 0; a < D; ++a) w[a] = (float)B.vn_b[(size_t)a * n + entry_slot(e)];
+        };
+        Sums32<D> A;
+        list_sums32<D, WALLS, L>(k, sh, lst, cnt, lane_in, oi, vi, qi.w, B.off, nb, wall, A);
+        rates32<D, L>(k, A, apT, FT);
+    } else {
+        const double4_32a *nb = B.nb64[1];
+        const PairConst<double> k = pair_const<double>(P);
+        Plain64 ap, Fa[3];
+        const double4_32a qi = fluid ? nb[s] : make_double4_32a(0, 0, 0, 0);
+        const double vi[3] = {qi.x, qi.y, qi.z};
+        // R entries per round: their indices, then their gathers, then the pair
+        // terms, so that R loads are in flight per lane; the entries keep their order
         constexpr int R = 4;
-        using Q = typename Packed<T>::type;
         for (int q0 = lane_in; q0 < cnt; q0 += L * R) {
             uint32_t jbv[R];
-            int cv[R];
-            if constexpr (L == 1) {
-                // four consecutive entries in one 16-byte load (rows start on
-                // 32-byte boundaries and q0 is a multiple of four); an entry
-                // past the count repeats entry q0, so its gathers stay in bounds
-                const uint4 v = *reinterpret_cast<const uint4 *>(lst + q0);
-                jbv[0] = v.x;
-                jbv[1] = q0 + 1 < cnt ? v.y : v.x;
-                jbv[2] = q0 + 2 < cnt ? v.z : v.x;
-                jbv[3] = q0 + 3 < cnt ? v.w : v.x;
-            } else {
+            double4_32a qv[R];
 #pragma unroll
-                for (int r = 0; r < R; ++r) jbv[r] = lst[min(q0 + r * L, cnt - 1)];
-            }
+            for (int r = 0; r < R; ++r) jbv[r] = lst[min(q0 + r * L, cnt - 1)];
 #pragma unroll
-            for (int r = 0; r < R; ++r) cv[r] = entry_code(jbv[r]);
-            Q qv[R];
-            float4 ov[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int j = entry_slot(jbv[r]);
-                qv[r] = nb[j];
-                ov[r] = F32 ? B.off[j] : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
+            for (int r = 0; r < R; ++r) qv[r] = nb[entry_slot(jbv[r])];
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 if (q0 + r * L >= cnt) break;
-                const uint32_t jb = jbv[r];
-                const int j = entry_slot(jb);
-                T d[3], r2;
-                if (F32) {
-                    offset_sep<D, T>(G, oi, ov[r], cv[r], d, r2);
-                } else {
-                    int dx, dy, dz;
-                    decode_shift(cv[r], dx, dy, dz);
-                    listed_sep<D, F32, T>(G, B.x_b, B.off, n, s, j, oi, dx, dy, dz, d, r2);
+                const int j = entry_slot(jbv[r]);
+                double d[3], g[3], F;
+                const double r2 = sep64<D>(G, B.x_b, n, s, j, d);
+                grad_coef<D, double>(P, d, r2, g, F);
+                const double vv[3] = {qv[r].x, qv[r].y, qv[r].z};
+                double vd[3] = {vv[0], vv[1], vv[2]};
+                if (WALLS && (jbv[r] & kWallBit)) {
+                    for (int a = 0; a < D; ++a) vd[a] = B.vn_b[(size_t)a * n + j];
                 }
-                T g[3], F;
-                grad_coef<D, T>(P, d, r2, g, F);
-                const auto qj = qv[r];
-                const T vv[3] = {(T)qj.x, (T)qj.y, (T)qj.z};
-                T vd[3] = {vv[0], vv[1], vv[2]};
-                if (WALLS && (jb & kWallBit)) {
-                    for (int a = 0; a < D; ++a) vd[a] = (T)B.vn_b[(size_t)a * n + j];
-                }
-                pair_accumulate<D, T, Acc>(k, g, F, vi, pi, vd, vv, (T)qj.w, ap, Fa);
+                pair_accumulate<D, double, Plain64>(k, g, F, vi, qi.w, vd, vv, qv[r].w, ap, Fa);
             }
         }
-    }
 #pragma unroll
-    for (int o = L / 2; o > 0; o >>= 1) {
-        ap.shfl_merge(o);
+        for (int o = L / 2; o > 0; o >>= 1) {
+            ap.shfl_merge(o);
 #pragma unroll
-        for (int a = 0; a < D; ++a) Fa[a].shfl_merge(o);
+            for (int a = 0; a < D; ++a) Fa[a].shfl_merge(o);
+        }
+        apT = ap.value();
+#pragma unroll
+        for (int a = 0; a < D; ++a) FT[a] = Fa[a].value();
     }
     if (gs == kNoParticle || lane_in != 0) return;
     if (!fluid) {
@@ -185,9 +173,9 @@ __global__ void __launch_bounds__(kBlock, F32 ? (D == 2 ? 4 : 3) : 1) k_state_n(
         }
         return;
     }
-    const double apv = (double)(T)ap.value();
+    const double apv = (double)apT;
     double Fv[3];
-    for (int a = 0; a < D; ++a) Fv[a] = __dadd_rn((double)(T)Fa[a].value(), P.g[a]);
+    for (int a = 0; a < D; ++a) Fv[a] = __dadd_rn((double)FT[a], P.g[a]);
     B.ap_b[s] = apv;
     for (int a = 0; a < D; ++a) B.f_b[(size_t)a * n + s] = Fv[a];
     if (PRED && P.steady) {
@@ -220,89 +208,110 @@ __global__ void __launch_bounds__(kBlock, F32 ? (D == 2 ? 4 : 3) : 1) k_state_n(
 
 // --------------------------------------------------------------- pair cache
 
-// The cache entries of slot s (its list, in the sliced layout); lane threadIdx.x % L
-// of the slot's group takes entries lane, lane + L, ...
-template <int D, bool F32, int L>
-__device__ __forceinline__ void pair_cache_slot(const Buffers &B, const Geom &G, const Phys &P,
-                                                const double *__restrict__ xpos, const uint32_t *__restrict__ gid,
-                                                int s)
+// The cache records of slot s (its list, in the sliced layout), FP32C: lane
+// threadIdx.x % L of the slot's group takes the pairs of entries lane, lane + L, ...,
+// two in flight.
+template <int D, int L>
+__device__ __forceinline__ void pair_cache_slot32(const Buffers &B, const Phys &P, const float4 *sh,
+                                                  const uint32_t *__restrict__ gid, int s)
 {
-    using T = typename std::conditional<F32, float, double>::type;
-    const int lane_in = threadIdx.x % L;
-    const int n = B.n;
+    const PairK32 k = P.k32;
     const bool wall_s = gid[s] >= (uint32_t)B.nf;
-    const uint32_t *lst = slot_list(B, s);                    // the list, per slot
-    const size_t base = (size_t)(s >> 5) * B.K * kWarp + (s & 31);   // the cache rows, sliced
-    const float4 oi = F32 ? B.off[s] : make_float4(0, 0, 0, 0);
-    const T sigma = (T)(P.sig_h * P.h);
-    const int cnt = B.pcount[s];
-    // R entries per round, their offsets gathered together (as in k_state_n)
-    constexpr int R = 4;
-    for (int q0 = lane_in; q0 < cnt; q0 += L * R) {
-        uint32_t jbv[R];
-        int cv[R];
+    const uint32_t *lst = slot_list(B, s);
+    const size_t row0 = cache_row(B, s);
+    const float4 oi = B.off[s];
+    const int np = list_pairs(B.pcount[s]);
+    auto put = [&](int m, uint32_t ea, uint32_t eb, float4 oa, float4 ob) {
+        CachePair c;
+        if (wall_s) {
+            // (a wall row's fill holds W(0); the wall values count the list's entries only)
+            float W[2], Wg[2];
+            const float sigma = (float)(P.sig_h * P.h);
+            const uint32_t e[2] = {ea, eb};
+            const float4 o[2] = {oa, ob};
 #pragma unroll
-        if constexpr (L == 1) {
-            // four consecutive entries in one 16-byte load (as in k_state_n);
-            // an entry past the count repeats entry q0
-            const uint4 v = *reinterpret_cast<const uint4 *>(lst + q0);
-            jbv[0] = v.x;
-            jbv[1] = q0 + 1 < cnt ? v.y : v.x;
-            jbv[2] = q0 + 2 < cnt ? v.z : v.x;
-            jbv[3] = q0 + 3 < cnt ? v.w : v.x;
+            for (int i = 0; i < 2; ++i) {
+                float d[3];
+                entry_sep<D>(sh, oi, o[i], e[i], d);
+                float r2 = __fmaf_rn(d[1], d[1], __fmul_rn(d[0], d[0]));
+                if (D == 3) r2 = __fmaf_rn(d[2], d[2], r2);
+                W[i] = __fmul_rn(sigma, quintic_w<float>(__fmul_rn(sqrtf(r2), k.inv_h)));
+                float gr = 0.f;
+                for (int a = 0; a < D; ++a) gr += (float)P.g[a] * d[a];
+                Wg[i] = (float)P.rho0 * gr * W[i];
+            }
+            c.c0 = make_float4(W[0], W[1], Wg[0], Wg[1]);
+            c.c1 = make_float4(0.f, 0.f, 0.f, 0.f);
         } else {
-#pragma unroll
-            for (int r = 0; r < R; ++r) jbv[r] = lst[min(q0 + r * L, cnt - 1)];
+            F2 g[D], F;
+            entry_grad2<D>(k, sh, oi, oa, ob, ea, eb, g, F);
+            unpack2(g[0], c.c0.x, c.c0.y);
+            unpack2(g[1], c.c0.z, c.c0.w);
+            if constexpr (D == 3) {
+                unpack2(g[2], c.c1.x, c.c1.y);
+                unpack2(F, c.c1.z, c.c1.w);
+            } else {
+                unpack2(F, c.c1.x, c.c1.y);
+            }
         }
-#pragma unroll
-        for (int r = 0; r < R; ++r) cv[r] = entry_code(jbv[r]);
-        float4 ov[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) ov[r] = F32 ? B.off[entry_slot(jbv[r])] : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int q = q0 + r * L;
-            if (q >= cnt) break;
-            const size_t e = base + (size_t)q * kWarp;
-            const uint32_t jb = jbv[r] & ~kCodeMask;      // what the pseudo-time loop reads
-            const int j = entry_slot(jb);
-            T d[3], r2;
-            if (F32) {
-                offset_sep<D, T>(G, oi, ov[r], cv[r], d, r2);
-            } else {
-                int dx, dy, dz;
-                decode_shift(cv[r], dx, dy, dz);
-                listed_sep<D, F32, T>(G, xpos, B.off, n, s, j, oi, dx, dy, dz, d, r2);
-            }
-            T c4[4] = {T(0), T(0), T(0), T(0)};
-            if (wall_s) {
-                const T W = Ar<T>::mul(sigma, quintic_w<T>(Ar<T>::mul(sqrt(r2), (T)P.inv_h)));
-                T gr = T(0);
-                for (int a = 0; a < D; ++a) gr += (T)P.g[a] * d[a];
-                c4[0] = W;
-                c4[1] = (T)P.rho0 * gr * W;
-            } else {
-                // layout (gradW, F_ij); FP32C in 2D packs (gx, gy, F_ij, index bits)
-                T g[3], F;
-                grad_coef<D, T>(P, d, r2, g, F);
-                c4[0] = g[0];
-                c4[1] = g[1];
-                if (F32 && D == 2) {
-                    c4[2] = F;
-                } else {
-                    c4[2] = D == 3 ? g[2] : T(0);
-                    c4[3] = F;
-                }
-            }
-            if (F32) {
-                float4 v = make_float4((float)c4[0], (float)c4[1], (float)c4[2], (float)c4[3]);
-                if (D == 2) v.w = __uint_as_float(jb);
-                B.pc32[e] = v;
-            } else {
-                B.pc64[e] = make_double4_32a((double)c4[0], (double)c4[1], (double)c4[2], (double)c4[3]);
-            }
-            if (!(F32 && D == 2)) B.pj[e] = jb;           // the loop reads the index from pj
+        const uint32_t ja = ea & ~kCodeMask, jb = eb & ~kCodeMask;      // what the pseudo-time loop reads
+        float4 *p = B.pc32 + (row0 + m) * 2 * kWarp + (s & 31);
+        if constexpr (D == 3) {
+            reinterpret_cast<uint2 *>(B.pj)[(row0 + m) * kWarp + (s & 31)] = make_uint2(ja, jb);
+        } else {
+            c.c1.z = __uint_as_float(ja);
+            c.c1.w = __uint_as_float(jb);
         }
+        p[0] = c.c0;
+        p[kWarp] = c.c1;
+    };
+    for (int m = threadIdx.x % L; m < np; m += 2 * L) {
+        const bool two = L == 1 || m + L < np;          // (one lane: the pairs come in twos)
+        uint32_t e[4];
+        if constexpr (L == 1) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(lst + 2 * m);
+            e[0] = v.x; e[1] = v.y; e[2] = v.z; e[3] = v.w;
+        } else {
+            const uint2 v = *reinterpret_cast<const uint2 *>(lst + 2 * m);
+            const uint2 u = *reinterpret_cast<const uint2 *>(lst + 2 * (two ? m + L : m));
+            e[0] = v.x; e[1] = v.y; e[2] = u.x; e[3] = u.y;
+        }
+        float4 o[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) o[r] = B.off[entry_slot(e[r])];
+        put(m, e[0], e[1], o[0], o[1]);
+        if (two) put(m + L, e[2], e[3], o[2], o[3]);
+    }
+}
+
+// The same for FP64, entry by entry.
+template <int D, int L>
+__device__ __forceinline__ void pair_cache_slot64(const Buffers &B, const Geom &G, const Phys &P,
+                                                  const double *__restrict__ xpos, const uint32_t *__restrict__ gid,
+                                                  int s)
+{
+    const bool wall_s = gid[s] >= (uint32_t)B.nf;
+    const uint32_t *lst = slot_list(B, s);                           // the list, per slot
+    const size_t base = (size_t)(s >> 5) * B.K * kWarp + (s & 31);   // the cache rows, sliced
+    const double sigma = P.sig_h * P.h;
+    const int cnt = B.pcount[s];
+    for (int q = threadIdx.x % L; q < cnt; q += L) {
+        const size_t e = base + (size_t)q * kWarp;
+        const uint32_t jb = lst[q] & ~kCodeMask;      // what the pseudo-time loop reads
+        double d[3], g[3] = {0, 0, 0}, F = 0;
+        const double r2 = sep64<D>(G, xpos, B.n, s, entry_slot(jb), d);
+        if (wall_s) {
+            const double W = Ar<double>::mul(sigma, quintic_w<double>(Ar<double>::mul(sqrt(r2), P.inv_h)));
+            double gr = 0;
+            for (int a = 0; a < D; ++a) gr += P.g[a] * d[a];
+            g[0] = W;
+            g[1] = P.rho0 * gr * W;
+        } else {
+            // layout (gradW, F_ij)
+            grad_coef<D, double>(P, d, r2, g, F);
+        }
+        B.pc64[e] = make_double4_32a(g[0], g[1], D == 3 && !wall_s ? g[2] : 0.0, F);
+        B.pj[e] = jb;
     }
 }
 
@@ -314,10 +323,10 @@ template <int D, bool F32, int L>
 __global__ void __launch_bounds__(kBlock) k_pair_cache(Buffers B, const double *__restrict__ xpos,
                                                        const uint32_t *__restrict__ gid)
 {
-    using T = typename std::conditional<F32, float, double>::type;
     constexpr int SPB = kBlock / L;
     __shared__ Geom G;
     __shared__ Phys P;
+    __shared__ float4 sh[kCodes];
     if (skip_form(B)) return;            // the step runs the other pair-term form
     if (blockIdx.x == 0 && B.form_run != 2) {    // (2: a paused loop goes on with the cache)
         reset_loops(B);
@@ -331,12 +340,16 @@ __global__ void __launch_bounds__(kBlock) k_pair_cache(Buffers B, const double *
         const int inst = block_instance(B, bt * SPB);
         if (inst != p_inst) {
             __syncthreads();                 // the previous tile is done with G and P
+            if (F32 && threadIdx.x < kCodes) sh[threadIdx.x] = code_shift(B.geo[inst], threadIdx.x);
             block_copy(G, B.geo[inst]);
             block_copy(P, B.phys[inst]);
             p_inst = inst;
         }
         const int s = bt * SPB + threadIdx.x / L;
-        if (s < B.n && gid[s] != kNoParticle) pair_cache_slot<D, F32, L>(B, G, P, xpos, gid, s);
+        if (s < B.n && gid[s] != kNoParticle) {
+            if constexpr (F32) pair_cache_slot32<D, L>(B, P, sh, gid, s);
+            else pair_cache_slot64<D, L>(B, G, P, xpos, gid, s);
+        }
     }
 }
 
