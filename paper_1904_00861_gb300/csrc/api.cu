@@ -733,7 +733,7 @@ int enqueue_pre_loop(dtsph_ctx *c, cudaStream_t st)
         Br.relist_run = 1;
         k += launch_binning(Br, Br.x_a, Br.gid_a, st);
         k += launch_permute_a_to_b(Br, st);
-        launch_nlist(Br, Br.x_b, Br.cell_b, Br.gid_b, st, false);
+        launch_nlist(Br, Br.x_b, st);
         Br.relist_run = 0;
         k += 1 + launch_same_order_a_to_b(Br, st);
         k += launch_state_n(B, true, st, false);
@@ -749,14 +749,14 @@ int enqueue_pre_loop(dtsph_ctx *c, cudaStream_t st)
     } else if (B.form_sel) {
         // both forms in the graph: the reset kernel picks the step's form; the
         // pair-cache pass returns at once when the step recomputes the terms
-        launch_nlist(B, B.xp_a, B.cell_a, B.gid_a, st, false);
+        launch_nlist(B, B.xp_a, st);
         k += 1 + launch_loop_reset(B, st);
         k += launch_pair_cache_pass(B, B.xp_a, B.gid_a, st);
     } else if (B.form_a) {
-        launch_nlist(B, B.xp_a, B.cell_a, B.gid_a, st, false);   // the loop recomputes the pair terms
+        launch_nlist(B, B.xp_a, st);   // the loop recomputes the pair terms
         k += 1 + launch_loop_reset(B, st);
     } else {
-        k += launch_pair_cache(B, B.xp_a, B.cell_a, B.gid_a, st);   // also resets the loop state
+        k += launch_pair_cache(B, B.xp_a, B.gid_a, st);   // also resets the loop state
     }
     return k;
 }
@@ -1049,7 +1049,7 @@ int autotune(dtsph_ctx *c)
     else CK(cudaMemsetAsync(B.nb64[0], 0, (size_t)B.n * sizeof(double4_32a), c->stream));
     c->launches += launch_binning(B, B.x_a, B.gid_a, c->stream);
     c->launches += launch_permute_a_to_b(B, c->stream);
-    c->launches += launch_pair_cache(B, B.x_b, B.cell_b, B.gid_b, c->stream);
+    c->launches += launch_pair_cache(B, B.x_b, B.gid_b, c->stream);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(c->stream));
     std::vector<TuneChoice> cand;
@@ -1125,7 +1125,7 @@ int measure_form_costs(dtsph_ctx *c)
     for (auto &ev : e) CK(cudaEventCreate(&ev));
     float t_cache = 0;
     for (int rep = 0; rep <= kReps; ++rep) {          // the first is a warm-up
-        launch_nlist(B, B.x_b, B.cell_b, B.gid_b, c->stream, false);
+        launch_nlist(B, B.x_b, c->stream);
         CK(cudaEventRecord(e[0], c->stream));
         launch_pair_cache_pass(B, B.x_b, B.gid_b, c->stream);   // leaves lists and cache for the loops below
         CK(cudaEventRecord(e[1], c->stream));
@@ -1493,7 +1493,7 @@ int dtsph_step(dtsph_ctx *c, int32_t nsteps)
         c->launches += launch_binning(B, B.x_a, B.gid_a, c->stream);
         c->launches += launch_permute_a_to_b(B, c->stream);
         c->launches += launch_adopt_b(B, c->stream);
-        launch_nlist(B, B.x_a, B.cell_a, B.gid_a, c->stream, false);
+        launch_nlist(B, B.x_a, c->stream);
         c->launches += 1;
         CK(cudaMemsetAsync(B.relist, 0, sizeof(int), c->stream));
         CK(cudaGetLastError());
@@ -1612,7 +1612,7 @@ int dtsph_build_neighbors(dtsph_ctx *c)
     c->lists_ready = false;                       // the lists are rebuilt at r^n in order B
     c->launches += launch_binning(B, B.x_a, B.gid_a, c->stream);
     c->launches += launch_permute_a_to_b(B, c->stream);
-    c->launches += launch_pair_cache(B, B.x_b, B.cell_b, B.gid_b, c->stream);
+    c->launches += launch_pair_cache(B, B.x_b, B.gid_b, c->stream);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(c->stream));
     int r = device_error(c);
@@ -1666,7 +1666,7 @@ int dtsph_probe_iterate(dtsph_ctx *c, int32_t launches, float *ms_per_launch, do
             return fail(c, DTSPH_E_STATE, "with particles moving in pseudo-time the probe needs a run without shifting");
         c->launches += launch_binning(B, B.x_a, B.gid_a, c->stream);
         c->launches += launch_permute_a_to_b(B, c->stream);
-        c->launches += launch_pair_cache(B, B.x_b, B.cell_b, B.gid_b, c->stream);
+        c->launches += launch_pair_cache(B, B.x_b, B.gid_b, c->stream);
         CK(cudaGetLastError());
         if (int r = device_error(c)) return r;
         B.gid_a = B.gid_b;

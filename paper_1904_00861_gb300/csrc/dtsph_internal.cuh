@@ -230,8 +230,7 @@ struct Buffers {
     uint32_t *pjt;         // neighbour lists, per slot: entry k of slot s at s Ks + k (Ks = list_stride(K))
     // pair cache, sliced by warp: FP64 entry k of slot i at ((i/32) K + k) 32 + i%32;
     // FP32C pairs of entries (pair32.cuh)
-    uint32_t *pj;          // slot | kWallBit of each entry (in 2D FP32C in pc32); particles moving
-                           // in pseudo-time: the sliced lists, one entry per place
+    uint32_t *pj;          // slot | kWallBit of each entry (in 2D FP32C in pc32)
     double4_32a *pc64;         // FP64: (gradW, F_ij)
     float4 *pc32;          // FP32C: two entries' coefficients in two float4
     int *pcount;           // neighbours of each slot
@@ -303,15 +302,14 @@ int launch_scatter_same(const Buffers &B, const double *x, const double *v, cons
                         cudaStream_t st);
 // Neighbour lists of every slot at positions xpos (order of the latest binning);
 // one launch.
-void launch_nlist(const Buffers &B, const double *xpos, const int *cell, const uint32_t *gid, cudaStream_t st,
-                  bool sliced);
+void launch_nlist(const Buffers &B, const double *xpos, cudaStream_t st);
 // The state-n pass at r^n in order B: its lists built first, or (build_lists
 // false) the r^0 lists of the previous step, built with list_skin, as they are.
 int launch_state_n(const Buffers &B, bool predictor, cudaStream_t st, bool build_lists = true);
 int launch_loop_resume(const Buffers &B, cudaStream_t st);
 int launch_restart_steps(const Buffers &B, cudaStream_t st);
 int launch_pair_cache_pass(const Buffers &B, const double *xpos, const uint32_t *gid, cudaStream_t st);
-int launch_pair_cache(const Buffers &B, const double *xpos, const int *cell, const uint32_t *gid, cudaStream_t st);
+int launch_pair_cache(const Buffers &B, const double *xpos, const uint32_t *gid, cudaStream_t st);
 int launch_walls_iter(const Buffers &B, cudaStream_t st);
 int launch_iterate(const Buffers &B, unsigned long long cond_handle, int use_cond, cudaStream_t st);
 int launch_outer(const Buffers &B, cudaStream_t st);

@@ -13,10 +13,8 @@
 //    candidate against that home particle. A ballot ranks the hits, which join the
 //    home particle's list as one contiguous run.
 // The lists are written per slot (slot s at s Ks + k, Ks = K rounded up to 8), each
-// row filled up to a multiple of four with entries of the slot itself; the
-// state-n, pair-cache and uncached-loop passes read them there, and only the pass
-// of particles moving in pseudo-time gets a copy sliced by warp (k_list_slice:
-// entry k of slot s at ((s/32) K + k) 32 + s%32).
+// row filled up to a multiple of four with entries of the slot itself, where
+// every pass reads them.
 //
 // The tests are those of the neighbour definition: FP64 positions, squares
 // summed in axis order without FMA, minimum image on periodic axes. Both
@@ -509,48 +507,13 @@ __global__ void __launch_bounds__(kListWarps * kWarp) k_nlist_home(Buffers B, co
     }
 }
 
-// The per-slot lists (slot s at s Ks + k) into the sliced layout, one warp per 32
-// slots: 32-entry pieces of the 32 lists pass through a shared-memory tile, read
-// as whole list segments and written as whole rows.
-__global__ void __launch_bounds__(kBlock) k_list_slice(Buffers B, const uint32_t *__restrict__ lists, int Ks)
-{
-    __shared__ uint32_t tile[kWarpsPerBlock][kWarp][kWarp + 1];
-    constexpr unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & (kWarp - 1), w = threadIdx.x >> 5;
-    const int s0 = (blockIdx.x * kWarpsPerBlock + w) * kWarp;
-    if (s0 >= B.n) return;                              // whole warp (n is a multiple of 32)
-    const int K = B.K;
-    // the builder writes the counts of the slots in cells; a padding slot's count
-    // is whatever the array holds, so every count is clamped to [0, K] and the
-    // accesses below stay inside the slot's own lists whatever memory held
-    const int cnt = min(max(B.pcount[s0 + lane], 0), K);
-    const int cmax = __reduce_max_sync(full, cnt);
-    uint32_t *rows = B.pj + (size_t)(s0 >> 5) * K * kWarp;
-    for (int k0 = 0; k0 < cmax; k0 += kWarp) {
-        for (int r = 0; r < kWarp; ++r) {
-            const int cr = __shfl_sync(full, cnt, r);
-            if (k0 + lane < cr) tile[w][lane][r] = lists[(size_t)(s0 + r) * Ks + k0 + lane];
-        }
-        __syncwarp();
-        const int kn = min(kWarp, cmax - k0);
-        for (int kk = 0; kk < kn; ++kk)
-            if (k0 + kk < cnt) rows[(size_t)(k0 + kk) * kWarp + lane] = tile[w][kk][lane];
-        __syncwarp();
-    }
-}
-
 }  // namespace
 
 static_assert(list_stride(1) % 4 == 0, "a list row holds whole 16-byte stores");
 
-// The lists of every slot at xpos into the per-slot layout (slot_list); with
-// `sliced`, also copied into the sliced layout of pj for the kernels that walk
-// them every pseudo-iteration (the moving pass). The passes that read a list
-// once per step (state n, pair cache, shifting) read the per-slot layout.
-void launch_nlist(const Buffers &B, const double *xpos, const int *cell, const uint32_t *gid, cudaStream_t st,
-                  bool sliced)
+// The lists of every slot at xpos (order of the latest binning); one launch.
+void launch_nlist(const Buffers &B, const double *xpos, cudaStream_t st)
 {
-    (void)cell;
     const int Ks = list_stride(B.K);
     if (B.dim == 2 && B.nseg2 < kRowsMinSegments) {
         const int nb = (B.ncell + kWarpsPerBlock - 1) / kWarpsPerBlock;
@@ -563,7 +526,6 @@ void launch_nlist(const Buffers &B, const double *xpos, const int *cell, const u
         const int nb = (B.ncell + kListWarps - 1) / kListWarps;
         k_nlist_home<3><<<nb, kListWarps * kWarp, 0, st>>>(B, xpos, B.pjt, Ks);
     }
-    if (sliced) k_list_slice<<<(B.n / kWarp + kWarpsPerBlock - 1) / kWarpsPerBlock, kBlock, 0, st>>>(B, B.pjt, Ks);
 }
 
 }  // namespace dtsph

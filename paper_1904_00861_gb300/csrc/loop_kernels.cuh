@@ -35,7 +35,7 @@
 #include "geometry.cuh"
 #include "loop_rules.cuh"
 #include "pair32.cuh"
-#include "pair_terms.cuh"
+#include "pair64.cuh"
 
 namespace dtsph {
 
@@ -276,6 +276,7 @@ __device__ __forceinline__ void pair_sums32(const Buffers &B, const Phys &P, con
         cnt = B.pcount[s];
     }
     Sums32<D> A;
+    NoMove mv;
     auto wall = [&](uint32_t e, const float4 &q, float *w) {
         w[0] = q.x; w[1] = q.y; w[2] = q.z;
         if (e & kWallBit) {
@@ -286,7 +287,7 @@ __device__ __forceinline__ void pair_sums32(const Buffers &B, const Phys &P, con
     if constexpr (FA) {
         static_assert(!WALLS, "the wall values come from the cache");
         const float4 oi = active ? B.off[s] : make_float4(0.f, 0.f, 0.f, 0.f);
-        list_sums32<D, false, L>(k, fg.sh, slot_list(B, s), cnt, lane_in, oi, vi, pi, B.off, nb, wall, A);
+        list_sums32<D, false, L>(k, fg.sh, slot_list(B, s), cnt, lane_in, oi, vi, pi, B.off, nb, wall, A, mv);
     } else {
         // a cache larger than L2 streams through it once per pass (first to
         // leave); a smaller one stays like the rest; the neighbour states,
@@ -307,10 +308,10 @@ __device__ __forceinline__ void pair_sums32(const Buffers &B, const Phys &P, con
             }
             F2 g[D], F;
             cache_coefs<D>(r, g, F);
-            pair2_accumulate<D, WALLS>(k, g, F, vi, pi, q[0], q[1], w[0], w[1], A);
+            pair2_accumulate<D, WALLS>(k, g, F, vi, pi, q[0], q[1], w[0], w[1], A, mv);
             if (!two) return;
             cache_coefs<D>(t, g, F);
-            pair2_accumulate<D, WALLS>(k, g, F, vi, pi, q[2], q[3], w[2], w[3], A);
+            pair2_accumulate<D, WALLS>(k, g, F, vi, pi, q[2], q[3], w[2], w[3], A, mv);
         };
         auto load = [&](int m) { return cache_pair_stream<D>(B, row0 + m, s & 31, pol_stream); };
         if constexpr (L == 1) {
@@ -374,7 +375,7 @@ __device__ __forceinline__ void pair_sums64(const Buffers &B, const Phys &P, con
         vi[0] = q.x; vi[1] = q.y; vi[2] = q.z; pi = q.w;
         cnt = B.pcount[s];
     }
-    Plain64 ap, Fa[3];
+    Sums64<D> A;
     // the terms of one entry with its gathered neighbour state; vw: the prescribed
     // velocity of a wall neighbour (the divergence term's V_j), gathered with the
     // neighbour states (one call for both kinds of neighbour: a warp whose lanes
@@ -384,9 +385,9 @@ __device__ __forceinline__ void pair_sums64(const Buffers &B, const Phys &P, con
         if constexpr (WALLS) {
             const bool wall = (jb & kWallBit) != 0;
             const double vd[3] = {wall ? vw[0] : vj[0], wall ? vw[1] : vj[1], wall ? vw[2] : vj[2]};
-            pair_accumulate<D, double, Plain64>(k, g, F, vi, pi, vd, vj, q.w, ap, Fa);
+            pair64_accumulate<D, true>(k, g, F, vi, pi, vd, vj, q.w, A);
         } else {
-            pair_accumulate<D, double, Plain64>(k, g, F, vi, pi, vj, vj, q.w, ap, Fa);
+            pair64_accumulate<D, false>(k, g, F, vi, pi, vj, vj, q.w, A);
         }
     };
     constexpr int R = 4;
@@ -397,6 +398,9 @@ __device__ __forceinline__ void pair_sums64(const Buffers &B, const Phys &P, con
         // takes l, l + L, ..., R in flight per round)
         static_assert(!WALLS, "the wall values come from the cache");
         const uint32_t *lst = slot_list(B, s);
+        double xi[3] = {0, 0, 0};
+        if (active)
+            for (int a = 0; a < D; ++a) xi[a] = B.xp_a[(size_t)a * B.n + s];
         for (int q0 = lane_in; q0 < cnt; q0 += L * R) {
             uint32_t jbv[R];
             double4_32a qv[R];
@@ -407,9 +411,9 @@ __device__ __forceinline__ void pair_sums64(const Buffers &B, const Phys &P, con
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 if (q0 + r * L >= cnt) break;
-                double d[3], r2, g[3], F;
-                r2 = sep64<D>(fg.G, B.xp_a, B.n, s, entry_slot(jbv[r]), d);
-                grad_coef<D, double>(P, d, r2, g, F);
+                double d[3], g[3], F;
+                const double r2 = listed_sep64<D>(fg.G, xi, B.xp_a, B.n, entry_slot(jbv[r]), d);
+                grad64<D>(P, d, r2, g, F);
                 pair(g, F, jbv[r], qv[r], nullptr);
             }
         }
@@ -513,15 +517,7 @@ __device__ __forceinline__ void pair_sums64(const Buffers &B, const Phys &P, con
                 }
         }
     }
-#pragma unroll
-    for (int o = L / 2; o > 0; o >>= 1) {
-        ap.shfl_merge(o);
-#pragma unroll
-        for (int a = 0; a < D; ++a) Fa[a].shfl_merge(o);
-    }
-    apT = ap.value();
-#pragma unroll
-    for (int a = 0; a < D; ++a) FT[a] = Fa[a].value();
+    rates64<D, L>(P, k, A, apT, FT);
 }
 
 // Phase 2 of an iteration: the BDF2 pseudo-acceleration and update, FP64

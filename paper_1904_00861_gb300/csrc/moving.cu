@@ -22,8 +22,9 @@
 // raises kErrSkin, so every pair within 3h of the moved positions is listed:
 // the sums equal those over neighbours updated at every pass (the pairs beyond
 // 3h add exact zeros).
-#include "geometry.cuh"
 #include "loop_rules.cuh"
+#include "pair32.cuh"
+#include "pair64.cuh"
 
 namespace dtsph {
 
@@ -117,11 +118,10 @@ __global__ void __launch_bounds__(kBlock) k_move_walls(Buffers B)
     const auto *nb = nb_ptr<T>(B, cur);
     const double sigma = P.sig_h * P.h;
     double sw = 0, sp = 0, sg = 0, sv[3] = {0, 0, 0};
-    const size_t base = (size_t)(s >> 5) * B.K * kWarp + (s & 31);
+    const uint32_t *lst = slot_list(B, s);
     const int cnt = B.pcount[s];
     for (int k = 0; k < cnt; ++k) {
-        const size_t e = base + (size_t)k * kWarp;
-        const uint32_t jb = B.pj[e];
+        const uint32_t jb = lst[k];
         if (jb & kWallBit) continue;            // fluid neighbours only
         const int j = entry_slot(jb);
         T d[3];
@@ -151,19 +151,19 @@ __global__ void __launch_bounds__(kBlock) k_move_walls(Buffers B)
 }
 
 // One moving iteration over all slots, L lanes per slot (lane l takes the list
-// entries l, l + L, ...; the partial sums merge by warp shuffles and the first
-// lane updates the particle) and one tile of kBlock / L slots per block; the last
-// block of an instance applies its stop rules, the last block of all sets the
-// while-node condition (as the frozen iterate kernel).
-template <int D, bool F32, int L>
+// entries, FP32C: pairs of entries, l, l + L, ...; the partial sums merge by warp
+// shuffles and the first lane updates the particle) and one tile of kBlock / L
+// slots per block; the last block of an instance applies its stop rules, the last
+// block of all sets the while-node condition (as the frozen iterate kernel). The
+// pair arithmetic is that of the frozen passes (pair32.cuh, pair64.cuh).
+template <int D, bool F32, bool WALLS, int L>
 __global__ void __launch_bounds__(kBlock) k_move_iter(Buffers B, unsigned long long cond, int use_cond)
 {
     constexpr int PPB = kBlock / L;
     using T = typename std::conditional<F32, float, double>::type;
-    using Acc = typename std::conditional<F32, Kahan, Plain64>::type;
-    using A = Ar<T>;
     __shared__ Geom G;
     __shared__ Phys P;
+    __shared__ float4 sh[kCodes];
     __shared__ double red[2][kBlock / kWarp];
     __shared__ int last, tlo_sh;
     if (!use_cond && B.ctrl->active == 0) return;   // whole grid agrees: nothing to do
@@ -176,123 +176,97 @@ __global__ void __launch_bounds__(kBlock) k_move_iter(Buffers B, unsigned long l
     const int it = ls->iter;
     const bool work = mine && !ls->done;
     if (work) {
+        if (F32 && threadIdx.x < kCodes) sh[threadIdx.x] = code_shift(B.geo[inst], threadIdx.x);
         block_copy(G, B.geo[inst]);
         block_copy(P, B.phys[inst]);
         const int cur = it & 1, nxt = cur ^ 1;
         const int s = blockIdx.x * PPB + threadIdx.x / L, lane_in = threadIdx.x % L;
         const bool fl = s < n && B.gid_a[s] < (uint32_t)B.nf;
         double r_ap = 0.0, r_av = 0.0;
-        Acc ap, Fa[3], gp[3];
-        const PairConst<T> k = pair_const<T>(P);
-        if (fl) {
-            const auto *nb = nb_ptr<T>(B, cur);
-            const auto qi = nb[s];
-            const T vi[3] = {(T)qi.x, (T)qi.y, (T)qi.z};
-            const T pi = (T)qi.w;
-            double xh[3] = {0, 0, 0}, vt[3] = {0, 0, 0};
-            T xi[3] = {T(0), T(0), T(0)}, ti[3] = {T(0), T(0), T(0)};
+        // the frozen rates and sum m (p_i + p_j) / rho0^2 gradW_ij
+        T apT = T(0), FT[3] = {T(0), T(0), T(0)}, gpT[3] = {T(0), T(0), T(0)};
+        const int cnt = fl ? B.pcount[s] : 0;
+        const uint32_t *lst = slot_list(B, s);
+        if constexpr (F32) {
+            const PairK32 k = P.k32;
+            const float4 *nb = B.nb32[cur];
+            const float4 qi = fl ? nb[s] : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 oi = fl ? B.offk[cur][s] : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float vi[3] = {qi.x, qi.y, qi.z};
+            Sums32<D> A;
+            Move32<D> mv;
 #pragma unroll
-            for (int a = 0; a < D; ++a) {
-                const size_t q = (size_t)a * n + s;
-                xh[a] = B.xk[cur][q];
-                xi[a] = (T)xh[a];
-                vt[a] = B.vt[q];
-                ti[a] = (T)vt[a];
-            }
-            const float4 oi = F32 ? B.offk[cur][s] : make_float4(0.f, 0.f, 0.f, 0.f);
-            const T rc2k = (T)(9.0 * P.h * P.h);
-            const size_t base = (size_t)(s >> 5) * B.K * kWarp + (s & 31);
-            const int cnt = B.pcount[s];
-            // R entries per round: their indices, then their gathers, then the
-            // pair terms, so that R loads are in flight per lane (the entries
-            // stay in the order lane_in, lane_in + L, ...)
-            constexpr int R = F32 ? 4 : 2;
-            using Q = typename Packed<T>::type;
+            for (int a = 0; a < 3; ++a) mv.t[a] = fl && a < D ? (float)B.vt[(size_t)a * n + s] : 0.f;
+            auto wall = [&](uint32_t e, const float4 &q, float *w) {
+                w[0] = q.x; w[1] = q.y; w[2] = q.z;
+                if (e & kWallBit) {
+                    const float4 v = B.wv32[entry_slot(e)];
+                    w[0] = v.x; w[1] = v.y; w[2] = v.z;
+                }
+            };
+            list_sums32<D, WALLS, L>(k, sh, lst, cnt, lane_in, oi, vi, qi.w, B.offk[cur], nb, wall, A, mv);
+            rates32<D, L>(k, A, apT, FT);
+#pragma unroll
+            for (int a = 0; a < D; ++a) gpT[a] = -__fmul_rn(k.s_F, merged32<L>(mv.np[a]));
+        } else {
+            const PairConst<double> k = pair_const<double>(P);
+            const double4_32a *nb = B.nb64[cur];
+            const double *xk = B.xk[cur];
+            const double4_32a qi = fl ? nb[s] : make_double4_32a(0, 0, 0, 0);
+            const double vi[3] = {qi.x, qi.y, qi.z};
+            double xi[3] = {0, 0, 0}, ti[3] = {0, 0, 0}, gp[3] = {0, 0, 0}, fc[3] = {0, 0, 0};
+            if (fl)
+                for (int a = 0; a < D; ++a) {
+                    xi[a] = xk[(size_t)a * n + s];
+                    ti[a] = B.vt[(size_t)a * n + s];
+                }
+            Sums64<D> A;
+            // R entries per round: their indices, then their gathers, then the pair
+            // terms (the entries stay in the order lane_in, lane_in + L, ...)
+            constexpr int R = 2;
             for (int q0 = lane_in; q0 < cnt; q0 += L * R) {
                 uint32_t jbv[R];
-                int codev[R];
+                double4_32a qv[R];
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const int q = q0 + r * L;
-                    const size_t e = base + (size_t)min(q, cnt - 1) * kWarp;
-                    jbv[r] = B.pj[e];
-                    codev[r] = entry_code(jbv[r]);
-                }
-                Q qv[R];
-                float4 ov[R];
-                T xj[R][3];
+                for (int r = 0; r < R; ++r) jbv[r] = lst[min(q0 + r * L, cnt - 1)];
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const int j = entry_slot(jbv[r]);
-                    qv[r] = nb[j];
-                    if (F32) {
-                        ov[r] = B.offk[cur][j];
-                    } else {
-#pragma unroll
-                        for (int a = 0; a < D; ++a) xj[r][a] = (T)B.xk[cur][(size_t)a * n + j];
-                    }
-                }
+                for (int r = 0; r < R; ++r) qv[r] = nb[entry_slot(jbv[r])];
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     if (q0 + r * L >= cnt) break;
-                    const uint32_t jb = jbv[r];
-                    const int j = entry_slot(jb);
-                    T d[3], r2;
-                    if (F32) {
-                        int dx, dy, dz;
-                        decode_shift(codev[r], dx, dy, dz);
-                        float f0, f1, f2;
-                        const float q2 = sep32<D>(shifted_offset<D>(oi, dx, dy, dz, G.s_f), ov[r], f0, f1, f2);
-                        d[0] = (T)f0;
-                        d[1] = (T)f1;
-                        if (D == 3) d[2] = (T)f2;
-                        r2 = (T)q2;
-                    } else {
+                    const int j = entry_slot(jbv[r]);
+                    double d[3], g[3], F;
+                    const double r2 = listed_sep64<D>(G, xi, xk, n, j, d);
+                    grad64<D>(P, d, r2, g, F);
+                    const double vv[3] = {qv[r].x, qv[r].y, qv[r].z};
+                    double vd[3] = {vv[0], vv[1], vv[2]};
+                    if (WALLS && (jbv[r] & kWallBit)) {
 #pragma unroll
-                        for (int a = 0; a < D; ++a) {
-                            double v = __dsub_rn((double)xi[a], (double)xj[r][a]);
-                            if (G.periodic[a]) {
-                                if (v > G.halfL[a]) v = __dsub_rn(v, G.L[a]);
-                                else if (v < -G.halfL[a]) v = __dadd_rn(v, G.L[a]);
-                            }
-                            d[a] = (T)v;
-                        }
-                        r2 = A::add(A::mul(d[0], d[0]), A::mul(d[1], d[1]));
-                        if (D == 3) r2 = A::add(r2, A::mul(d[2], d[2]));
+                        for (int a = 0; a < D; ++a) vd[a] = B.vn_a[(size_t)a * n + j];
                     }
-                    if (!(r2 < rc2k)) continue;          // outside the kernel support: adds nothing
-                    T g[3], F;
-                    grad_coef<D, T>(P, d, r2, g, F);
-                    const Q qj = qv[r];
-                    const T vv[3] = {(T)qj.x, (T)qj.y, (T)qj.z};
-                    T vd[3] = {vv[0], vv[1], vv[2]};
-                    if (jb & kWallBit) {
-#pragma unroll
-                        for (int a = 0; a < D; ++a) vd[a] = (T)B.vn_a[(size_t)a * n + j];
-                    }
-                    const T pj = (T)qj.w;
-                    pair_accumulate<D, T, Acc>(k, g, F, vi, pi, vd, vv, pj, ap, Fa);
+                    pair64_accumulate<D, WALLS>(k, g, F, vi, qi.w, vd, vv, qv[r].w, A);
                     // advective terms of Eqs. (dp-dtau) and (discrete_ME)
-                    T tg = T(0);
+                    double tg = 0.0;
 #pragma unroll
-                    for (int a = 0; a < D; ++a) tg = A::fma(ti[a], g[a], tg);
-                    const T pp = A::mul(k.c_p, A::add(pi, pj));
+                    for (int a = 0; a < D; ++a) tg = __fma_rn(ti[a], g[a], tg);
+                    const double pp = __dadd_rn(qi.w, qv[r].w);
 #pragma unroll
                     for (int a = 0; a < D; ++a) {
-                        gp[a].add(A::mul(pp, g[a]));
-                        Fa[a].add(A::mul(A::mul(k.vol, A::add(vi[a], vd[a])), tg));
+                        gp[a] = __fma_rn(pp, g[a], gp[a]);
+                        fc[a] = __fma_rn(__dadd_rn(vi[a], vd[a]), tg, fc[a]);
                     }
                 }
             }
-        }
-        // every lane takes part in the merges
-#pragma unroll
-        for (int o = L / 2; o > 0; o >>= 1) {
-            ap.shfl_merge(o);
+            rates64<D, L>(P, k, A, apT, FT);
 #pragma unroll
             for (int a = 0; a < D; ++a) {
-                Fa[a].shfl_merge(o);
-                gp[a].shfl_merge(o);
+#pragma unroll
+                for (int o = L / 2; o > 0; o >>= 1) {
+                    gp[a] = __dadd_rn(gp[a], __shfl_xor_sync(0xffffffffu, gp[a], o));
+                    fc[a] = __dadd_rn(fc[a], __shfl_xor_sync(0xffffffffu, fc[a], o));
+                }
+                gpT[a] = __dmul_rn(__dmul_rn(k.c_p, P.sig_h), gp[a]);
+                FT[a] = __fma_rn(__dmul_rn(k.vol, P.sig_h), fc[a], FT[a]);
             }
         }
         if (fl && lane_in == 0) {
@@ -304,9 +278,9 @@ __global__ void __launch_bounds__(kBlock) k_move_iter(Buffers B, unsigned long l
                 vt[a] = B.vt[q];
             }
             // update in FP64
-            double apv = (double)(T)ap.value();
+            double apv = (double)apT;
 #pragma unroll
-            for (int a = 0; a < D; ++a) apv = __fma_rn(vt[a], (double)(T)gp[a].value(), apv);
+            for (int a = 0; a < D; ++a) apv = __fma_rn(vt[a], (double)gpT[a], apv);
             double vnew[3] = {0, 0, 0}, xn[3] = {0, 0, 0};
             double av2 = 0.0;
             const double hdt = 0.5 * P.dtau;
@@ -314,7 +288,7 @@ __global__ void __launch_bounds__(kBlock) k_move_iter(Buffers B, unsigned long l
             for (int a = 0; a < D; ++a) {
                 const size_t q = (size_t)a * n + s;
                 const double vk = B.vk[cur][q];
-                const double Fv = (double)(T)Fa[a].value();
+                const double Fv = (double)FT[a];
                 const double av = __fma_rn(P.kappa, Fv, -__fma_rn(P.kc3, vk, B.s_a[q]));
                 vnew[a] = __fma_rn(P.dtau, av, vk);
                 B.vk[nxt][q] = vnew[a];
@@ -418,7 +392,7 @@ __global__ void __launch_bounds__(kBlock) k_move_iter(Buffers B, unsigned long l
 
 int launch_move_prepare(const Buffers &B, cudaStream_t st)
 {
-    launch_nlist(B, B.xp_a, B.cell_a, B.gid_a, st, true);   // walked every pass: sliced
+    launch_nlist(B, B.xp_a, st);
     if (B.fp32c) k_move_init<true><<<blocks(B.n), kBlock, 0, st>>>(B);
     else k_move_init<false><<<blocks(B.n), kBlock, 0, st>>>(B);
     return 2;
@@ -433,10 +407,17 @@ int launch_move_iteration(const Buffers &B, unsigned long long cond, int use_con
     }
     // n is a multiple of kSlotAlign, so the tiles of kBlock / L slots cover it exactly
     const int L = B.lanes, nb = (int)((long long)B.n * L / kBlock);
-    if (L == 1) DTSPH_DISPATCH(B.dim, B.fp32c, (k_move_iter<D, F32, 1><<<nb, kBlock, 0, st>>>(B, cond, use_cond)));
-    else if (L == 2) DTSPH_DISPATCH(B.dim, B.fp32c, (k_move_iter<D, F32, 2><<<nb, kBlock, 0, st>>>(B, cond, use_cond)));
-    else if (L == 4) DTSPH_DISPATCH(B.dim, B.fp32c, (k_move_iter<D, F32, 4><<<nb, kBlock, 0, st>>>(B, cond, use_cond)));
-    else DTSPH_DISPATCH(B.dim, B.fp32c, (k_move_iter<D, F32, 8><<<nb, kBlock, 0, st>>>(B, cond, use_cond)));
+    auto go = [&](auto lanes) {
+        constexpr int LL = decltype(lanes)::value;
+        if (B.nw > 0) DTSPH_DISPATCH(B.dim, B.fp32c, (k_move_iter<D, F32, true, LL><<<nb, kBlock, 0, st>>>(B, cond, use_cond)));
+        else DTSPH_DISPATCH(B.dim, B.fp32c, (k_move_iter<D, F32, false, LL><<<nb, kBlock, 0, st>>>(B, cond, use_cond)));
+    };
+    switch (L) {
+    case 1: go(std::integral_constant<int, 1>()); break;
+    case 2: go(std::integral_constant<int, 2>()); break;
+    case 4: go(std::integral_constant<int, 4>()); break;
+    default: go(std::integral_constant<int, 8>()); break;
+    }
     return k + 1;
 }
 

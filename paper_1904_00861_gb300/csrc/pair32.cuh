@@ -106,13 +106,25 @@ __device__ __forceinline__ void grad2(const PairK32 &k, const F2 *d, F2 *g, F2 &
     F = mul2(mul2(w, r), pack2(rcp_fast(da), rcp_fast(db)));
 }
 
+// What particles moving in pseudo-time add (Eqs. dp-dtau, discrete_ME): their
+// pseudo-velocity t and sum -(p_i + p_j) g; NoMove for particles fixed in it.
+template <int D>
+struct Move32 {
+    static constexpr bool on = true;
+    float t[3];
+    Kahan2 np[D];
+};
+struct NoMove {
+    static constexpr bool on = false;
+};
+
 // The contribution of two neighbours with states qa and qb (V, p) to the sums.
 // WALLS: wa, wb are their velocities in the divergence term (a wall's prescribed
 // one), the states' being those of the viscous terms (a wall's ghost velocity).
-template <int D, bool WALLS>
+template <int D, bool WALLS, typename M>
 __device__ __forceinline__ void pair2_accumulate(const PairK32 &k, const F2 *g, F2 F, const float *vi, float pi,
                                                  float4 qa, float4 qb, const float *wa, const float *wb,
-                                                 Sums32<D> &A)
+                                                 Sums32<D> &A, M &mv)
 {
     const float va[3] = {qa.x, qa.y, qa.z}, vb[3] = {qb.x, qb.y, qb.z};
     F2 dv[D];
@@ -127,6 +139,15 @@ __device__ __forceinline__ void pair2_accumulate(const PairK32 &k, const F2 *g, 
     A.ap.add(fma2(mul2(both(k.ed), dp), F, y));
     F2 np = pack2(__fsub_rn(-pi, qa.w), __fsub_rn(-pi, qb.w));    // -(p_i + p_j)
     F2 conv = both(0.f);
+    if constexpr (M::on) {
+        // advection: (V_i + V_j) m/rho0 (V~_i . g), and the pressure sum that V~_i meets
+        conv = mul2(both(mv.t[0]), g[0]);
+#pragma unroll
+        for (int a = 1; a < D; ++a) conv = fma2(both(mv.t[a]), g[a], conv);
+        conv = mul2(both(k.vol), conv);
+#pragma unroll
+        for (int a = 0; a < D; ++a) mv.np[a].add(fma2(np, g[a], mv.np[a].nc));
+    }
     // the terms that most runs do without (artificial viscosity, the steady-mode
     // convection) sit behind one uniform test
     if (k.rare) {
@@ -159,29 +180,30 @@ __device__ __forceinline__ void pair2_accumulate(const PairK32 &k, const F2 *g, 
 #pragma unroll
     for (int a = 0; a < D; ++a) {
         F2 z = fma2(cv, dv[a], fma2(np, g[a], A.F[a].nc));
-        if (k.rare && k.steady)
+        if (M::on || (k.rare && k.steady))
             z = fma2(conv, WALLS ? pack2(__fadd_rn(vi[a], wa[a]), __fadd_rn(vi[a], wb[a]))
                                  : pack2(__fadd_rn(vi[a], va[a]), __fadd_rn(vi[a], vb[a])), z);
         A.F[a].add(z);
     }
 }
 
-// The even and odd sums merged, then those of the particle's L lanes; the rates
-// with their factors.
+// A sum's even and odd halves merged, then the particle's L lanes.
+template <int L>
+__device__ __forceinline__ float merged32(const Kahan2 &a)
+{
+    Kahan m = a.merged();
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) m.shfl_merge(o);
+    return m.value();
+}
+
+// The rates with their factors.
 template <int D, int L>
 __device__ __forceinline__ void rates32(const PairK32 &k, const Sums32<D> &A, float &ap, float *F)
 {
-    Kahan m = A.ap.merged();
+    ap = __fmul_rn(k.s_ap, merged32<L>(A.ap));
 #pragma unroll
-    for (int o = L / 2; o > 0; o >>= 1) m.shfl_merge(o);
-    ap = __fmul_rn(k.s_ap, m.value());
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        Kahan f = A.F[a].merged();
-#pragma unroll
-        for (int o = L / 2; o > 0; o >>= 1) f.shfl_merge(o);
-        F[a] = __fmul_rn(k.s_F, f.value());
-    }
+    for (int a = 0; a < D; ++a) F[a] = __fmul_rn(k.s_F, merged32<L>(A.F[a]));
 }
 
 // Displacement of the home offset for every shift code: o_i moves by minus the
@@ -224,10 +246,10 @@ __host__ __device__ __forceinline__ int list_pairs(int cnt) { return (cnt + 3) /
 // The sums over the list lst of a particle by L lanes (lane_in takes the pairs
 // lane_in, lane_in + L, ..., two in flight): offsets off, states nb, geometry
 // recomputed. wall(entry, w) gives a neighbour's divergence-term velocity (WALLS).
-template <int D, bool WALLS, int L, typename WV>
+template <int D, bool WALLS, int L, typename WV, typename M>
 __device__ __forceinline__ void list_sums32(const PairK32 &k, const float4 *sh, const uint32_t *__restrict__ lst,
                                             int cnt, int lane_in, float4 oi, const float *vi, float pi,
-                                            const float4 *off, const float4 *nb, WV wall, Sums32<D> &A)
+                                            const float4 *off, const float4 *nb, WV wall, Sums32<D> &A, M &mv)
 {
     const int np = list_pairs(cnt);
     for (int m = lane_in; m < np; m += 2 * L) {
@@ -255,7 +277,7 @@ __device__ __forceinline__ void list_sums32(const PairK32 &k, const float4 *sh, 
             if (r == 2 && !two) break;
             F2 g[D], F;
             entry_grad2<D>(k, sh, oi, o[r], o[r + 1], e[r], e[r + 1], g, F);
-            pair2_accumulate<D, WALLS>(k, g, F, vi, pi, q[r], q[r + 1], w[r], w[r + 1], A);
+            pair2_accumulate<D, WALLS>(k, g, F, vi, pi, q[r], q[r + 1], w[r], w[r + 1], A, mv);
         }
     }
 }

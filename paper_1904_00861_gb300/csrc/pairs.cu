@@ -8,6 +8,7 @@
 #include "geometry.cuh"
 #include "loop_rules.cuh"
 #include "pair32.cuh"
+#include "pair64.cuh"
 
 namespace dtsph {
 
@@ -16,13 +17,17 @@ namespace {
 // ---------------------------------------------------------------- walls, state n
 
 // The list walkers below give each slot a group of L lanes; lane l of a group
-// takes the list entries l, l + L, ... Summing kernels merge the lanes' partial
-// sums by shuffles, so their summation order depends on L alone: they use the
-// fixed kSumLanes, which keeps every context (solo or batched, any size) on
-// the same order. One lane per slot measured fastest on large problems and
-// costs little on small ones. Block b covers slots b * (kBlock / L) ...
+// takes the list entries (FP32C: pairs of entries) l, l + L, ... Summing kernels
+// merge the lanes' partial sums by shuffles, so their summation order depends on L
+// alone: they use a fixed L per path, which keeps every context (solo or batched,
+// any size) on the same order. FP32C: one lane per slot measured fastest on large
+// problems and costs little on small ones. FP64: eight, a small problem's chain of
+// pairs being what its pass takes (1,024 2D particles: 139 us with one lane, 14 us
+// now, the factored sums included), at no cost to large ones, which the FP64
+// pipe bounds. Block b covers slots b * (kBlock / L) ...
 
-constexpr int kSumLanes = 1;
+template <bool F32>
+constexpr int kSumLanes = F32 ? 1 : 8;
 
 // Adami et al. wall values at state n in order B: p_w = (sum_f p_f W + rho0 g .
 // sum_f r_wf W) / sum_f W, ghost velocity 2 v_w - sum_f V_f W / sum_f W; written
@@ -123,12 +128,16 @@ __global__ void __launch_bounds__(kBlock, F32 ? (D == 2 ? 4 : 3) : 1) k_state_n(
                 for (int a = 0; a < D; ++a) w[a] = (float)B.vn_b[(size_t)a * n + entry_slot(e)];
         };
         Sums32<D> A;
-        list_sums32<D, WALLS, L>(k, sh, lst, cnt, lane_in, oi, vi, qi.w, B.off, nb, wall, A);
+        NoMove mv;
+        list_sums32<D, WALLS, L>(k, sh, lst, cnt, lane_in, oi, vi, qi.w, B.off, nb, wall, A, mv);
         rates32<D, L>(k, A, apT, FT);
     } else {
         const double4_32a *nb = B.nb64[1];
         const PairConst<double> k = pair_const<double>(P);
-        Plain64 ap, Fa[3];
+        Sums64<D> A;
+        double xi[3] = {0, 0, 0};
+        if (fluid)
+            for (int a = 0; a < D; ++a) xi[a] = B.x_b[(size_t)a * n + s];
         const double4_32a qi = fluid ? nb[s] : make_double4_32a(0, 0, 0, 0);
         const double vi[3] = {qi.x, qi.y, qi.z};
         // R entries per round: their indices, then their gathers, then the pair
@@ -146,25 +155,20 @@ __global__ void __launch_bounds__(kBlock, F32 ? (D == 2 ? 4 : 3) : 1) k_state_n(
                 if (q0 + r * L >= cnt) break;
                 const int j = entry_slot(jbv[r]);
                 double d[3], g[3], F;
-                const double r2 = sep64<D>(G, B.x_b, n, s, j, d);
-                grad_coef<D, double>(P, d, r2, g, F);
+                const double r2 = listed_sep64<D>(G, xi, B.x_b, n, j, d);
+                grad64<D>(P, d, r2, g, F);
                 const double vv[3] = {qv[r].x, qv[r].y, qv[r].z};
-                double vd[3] = {vv[0], vv[1], vv[2]};
-                if (WALLS && (jbv[r] & kWallBit)) {
-                    for (int a = 0; a < D; ++a) vd[a] = B.vn_b[(size_t)a * n + j];
+                if constexpr (WALLS) {
+                    double vd[3] = {vv[0], vv[1], vv[2]};
+                    if (jbv[r] & kWallBit)
+                        for (int a = 0; a < D; ++a) vd[a] = B.vn_b[(size_t)a * n + j];
+                    pair64_accumulate<D, true>(k, g, F, vi, qi.w, vd, vv, qv[r].w, A);
+                } else {
+                    pair64_accumulate<D, false>(k, g, F, vi, qi.w, vv, vv, qv[r].w, A);
                 }
-                pair_accumulate<D, double, Plain64>(k, g, F, vi, qi.w, vd, vv, qv[r].w, ap, Fa);
             }
         }
-#pragma unroll
-        for (int o = L / 2; o > 0; o >>= 1) {
-            ap.shfl_merge(o);
-#pragma unroll
-            for (int a = 0; a < D; ++a) Fa[a].shfl_merge(o);
-        }
-        apT = ap.value();
-#pragma unroll
-        for (int a = 0; a < D; ++a) FT[a] = Fa[a].value();
+        rates64<D, L>(P, k, A, apT, FT);
     }
     if (gs == kNoParticle || lane_in != 0) return;
     if (!fluid) {
@@ -295,11 +299,13 @@ __device__ __forceinline__ void pair_cache_slot64(const Buffers &B, const Geom &
     const size_t base = (size_t)(s >> 5) * B.K * kWarp + (s & 31);   // the cache rows, sliced
     const double sigma = P.sig_h * P.h;
     const int cnt = B.pcount[s];
+    double xi[3] = {0, 0, 0};
+    for (int a = 0; a < D; ++a) xi[a] = xpos[(size_t)a * B.n + s];
     for (int q = threadIdx.x % L; q < cnt; q += L) {
         const size_t e = base + (size_t)q * kWarp;
         const uint32_t jb = lst[q] & ~kCodeMask;      // what the pseudo-time loop reads
         double d[3], g[3] = {0, 0, 0}, F = 0;
-        const double r2 = sep64<D>(G, xpos, B.n, s, entry_slot(jb), d);
+        const double r2 = listed_sep64<D>(G, xi, xpos, B.n, entry_slot(jb), d);
         if (wall_s) {
             const double W = Ar<double>::mul(sigma, quintic_w<double>(Ar<double>::mul(sqrt(r2), P.inv_h)));
             double gr = 0;
@@ -307,8 +313,8 @@ __device__ __forceinline__ void pair_cache_slot64(const Buffers &B, const Geom &
             g[0] = W;
             g[1] = P.rho0 * gr * W;
         } else {
-            // layout (gradW, F_ij)
-            grad_coef<D, double>(P, d, r2, g, F);
+            // layout (g, F)
+            grad64<D>(P, d, r2, g, F);
         }
         B.pc64[e] = make_double4_32a(g[0], g[1], D == 3 && !wall_s ? g[2] : 0.0, F);
         B.pj[e] = jb;
@@ -459,33 +465,32 @@ int nlist_lanes(int n)
 // Neighbour lists at r^n (order B), then the wall values and the state-n pass.
 int launch_state_n(const Buffers &B, bool predictor, cudaStream_t st, bool build_lists)
 {
-    constexpr int L = kSumLanes;
-    const int nb = (int)(((long long)B.n * L + kBlock - 1) / kBlock);
     int k = 0;
     if (build_lists) {
-        launch_nlist(B, B.x_b, B.cell_b, B.gid_b, st, false);
+        launch_nlist(B, B.x_b, st);
         k = 1;
     }
-    if (B.nw > 0) {
-        DTSPH_DISPATCH(B.dim, B.fp32c, (k_walls_state_n<D, F32, L><<<nb, kBlock, 0, st>>>(B)));
-        ++k;
-    }
-    const bool w = B.nw > 0;
-    if (predictor && w)
-        DTSPH_DISPATCH(B.dim, B.fp32c, (k_state_n<D, F32, true, true, L><<<nb, kBlock, 0, st>>>(B)));
-    else if (predictor)
-        DTSPH_DISPATCH(B.dim, B.fp32c, (k_state_n<D, F32, true, false, L><<<nb, kBlock, 0, st>>>(B)));
-    else if (w)
-        DTSPH_DISPATCH(B.dim, B.fp32c, (k_state_n<D, F32, false, true, L><<<nb, kBlock, 0, st>>>(B)));
-    else
-        DTSPH_DISPATCH(B.dim, B.fp32c, (k_state_n<D, F32, false, false, L><<<nb, kBlock, 0, st>>>(B)));
+    DTSPH_DISPATCH(B.dim, B.fp32c, {
+        constexpr int L = kSumLanes<F32>;
+        const int nb = (int)(((long long)B.n * L + kBlock - 1) / kBlock);
+        if (B.nw > 0) {
+            k_walls_state_n<D, F32, L><<<nb, kBlock, 0, st>>>(B);
+            ++k;
+            if (predictor) k_state_n<D, F32, true, true, L><<<nb, kBlock, 0, st>>>(B);
+            else k_state_n<D, F32, false, true, L><<<nb, kBlock, 0, st>>>(B);
+        } else if (predictor) {
+            k_state_n<D, F32, true, false, L><<<nb, kBlock, 0, st>>>(B);
+        } else {
+            k_state_n<D, F32, false, false, L><<<nb, kBlock, 0, st>>>(B);
+        }
+    });
     return k + 1;
 }
 
 // Neighbour lists at xpos, then the pair coefficients.
-int launch_pair_cache(const Buffers &B, const double *xpos, const int *cell, const uint32_t *gid, cudaStream_t st)
+int launch_pair_cache(const Buffers &B, const double *xpos, const uint32_t *gid, cudaStream_t st)
 {
-    launch_nlist(B, xpos, cell, gid, st, false);
+    launch_nlist(B, xpos, st);
     return 1 + launch_pair_cache_pass(B, xpos, gid, st);
 }
 
@@ -507,7 +512,7 @@ int launch_shift(const Buffers &B, cudaStream_t st)
 {
     int k = launch_binning(B, B.x_a, B.gid_a, st);            // cells at r^{n+1}
     k += launch_permute_a_to_b(B, st);
-    launch_nlist(B, B.x_b, B.cell_b, B.gid_b, st, false);
+    launch_nlist(B, B.x_b, st);
     DTSPH_DISPATCH(B.dim, B.fp32c, (k_shift<D, F32><<<(B.n + kBlock - 1) / kBlock, kBlock, 0, st>>>(B)));
     return k + 2;
 }
