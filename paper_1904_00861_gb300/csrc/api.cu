@@ -1049,6 +1049,10 @@ int autotune(dtsph_ctx *c)
     else CK(cudaMemsetAsync(B.nb64[0], 0, (size_t)B.n * sizeof(double4_32a), c->stream));
     c->launches += launch_binning(B, B.x_a, B.gid_a, c->stream);
     c->launches += launch_permute_a_to_b(B, c->stream);
+    // the loop runs in order A: the lists' order becomes it (with walls in the
+    // caller's order, the candidates would run wall rows as fluid rows, stop on
+    // non-finite residuals and show times that no step has)
+    c->launches += launch_adopt_b(B, c->stream);
     c->launches += launch_pair_cache(B, B.x_b, B.gid_b, c->stream);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(c->stream));
@@ -1120,6 +1124,7 @@ int measure_form_costs(dtsph_ctx *c)
     else CK(cudaMemsetAsync(B.nb64[0], 0, (size_t)B.n * sizeof(double4_32a), c->stream));
     c->launches += launch_binning(B, B.x_a, B.gid_a, c->stream);
     c->launches += launch_permute_a_to_b(B, c->stream);
+    c->launches += launch_adopt_b(B, c->stream);   // (the loop runs in order A)
     constexpr int kReps = 5;
     cudaEvent_t e[2];
     for (auto &ev : e) CK(cudaEventCreate(&ev));

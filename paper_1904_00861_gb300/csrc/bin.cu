@@ -442,8 +442,8 @@ int launch_same_order_a_to_b(const Buffers &B, cudaStream_t st)
 }
 
 // Order B becomes order A as it is (the particles binned at r^n, before the
-// first step that reuses the r^0 lists): slot, cell and the state that order A
-// carries between steps.
+// first step that reuses the r^0 lists, and before the candidates of the loop are
+// timed): slot, cell and the state that order A carries between steps.
 __global__ void __launch_bounds__(kBlock) k_adopt_b(Buffers B)
 {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -457,10 +457,17 @@ __global__ void __launch_bounds__(kBlock) k_adopt_b(Buffers B)
     for (int a = 0; a < B.dim; ++a) {
         const size_t q = (size_t)a * n + s;
         B.x_a[q] = B.x_b[q];
+        B.xp_a[q] = B.x_b[q];            // (the positions of the lists)
         B.vn_a[q] = B.vn_b[q];
         B.vnm1_a[q] = B.vnm1_b[q];
     }
     B.pn_a[s] = B.pn_b[s];
+    if (B.wslot_a && g >= (uint32_t)B.nf) {
+        B.wslot_a[g - (uint32_t)B.nf] = s;
+        double u[3] = {0, 0, 0};
+        for (int a = 0; a < B.dim; ++a) u[a] = B.vn_b[(size_t)a * n + s];
+        store_wall_velocity(B, s, u);
+    }
 }
 
 int launch_adopt_b(const Buffers &B, cudaStream_t st)

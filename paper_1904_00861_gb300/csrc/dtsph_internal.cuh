@@ -248,6 +248,8 @@ struct Buffers {
     InstLoop *il;          // [ninst] work counters of the decoupled batch loop (null without it)
     const int *sched;      // [ninst] instances by ascending tile count (the decoupled loop's search order)
     int async_loop;        // 1: batches without walls run the decoupled loop kernel
+    int res_q, res_rows;   // the resident loop (iterate_res.cu): slots per block, cache rows a
+                           // thread keeps in shared memory
     int form_a;            // 1: the loop recomputes the pair geometry from the lists (no pair cache)
     // the per-step choice of the pair-term form (form = 0), in the step graph
     // only (null elsewhere): k_loop_reset writes the step's form to *form_sel
@@ -327,6 +329,15 @@ int launch_move_iteration(const Buffers &B, unsigned long long cond_handle, int 
 int launch_shift(const Buffers &B, cudaStream_t st);
 // Persistent pseudo-time loop (one cooperative launch per real step): grid size
 // (co-resident blocks, at most one per tile) and the launch itself.
+// An instance that fits one block per SM takes the resident loop (launch_loop
+// chooses; the grid is then its own).
+struct ResShape {
+    const void *fn;
+    int q, rows, grid, threads;
+    size_t smem;
+};
+bool resident_shape(const Buffers &B, ResShape *S);
+int resident_prepare();
 int loop_grid(const Buffers &B, int *grid);
 cudaError_t launch_loop(const Buffers &B, int grid, cudaStream_t st);
 int launch_loop_reset(const Buffers &B, cudaStream_t st);

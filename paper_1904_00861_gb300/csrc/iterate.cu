@@ -126,19 +126,31 @@ int loop_grid(const Buffers &B, int *grid)
 
 cudaError_t launch_loop(const Buffers &B, int grid, cudaStream_t st)
 {
+    Buffers b = B;
+    const void *fn = nullptr;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kBlock);
-    cfg.dynamicSmemBytes = iterate_smem(B);
+    ResShape R;
+    if (resident_shape(B, &R)) {
+        fn = R.fn;
+        b.res_q = R.q;
+        b.res_rows = R.rows;
+        cfg.gridDim = dim3(R.grid);
+        cfg.blockDim = dim3(R.threads);
+        cfg.dynamicSmemBytes = R.smem;
+    } else {
+        fn = loop_function(B);
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3(kBlock);
+        cfg.dynamicSmemBytes = iterate_smem(B);
+    }
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    Buffers b = B;
     void *args[] = {(void *)&b};
-    return cudaLaunchKernelExC(&cfg, loop_function(B), args);
+    return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
 int launch_outer(const Buffers &B, cudaStream_t st)
@@ -163,7 +175,7 @@ int iterate_prepare()
     if (e == cudaSuccess) e = allow_ring_smem<3, true, true>();
     if (e == cudaSuccess) e = allow_ring_smem<3, false, false>();
     if (e == cudaSuccess) e = allow_ring_smem<3, false, true>();
-    return e == cudaSuccess ? 0 : -1;
+    return e == cudaSuccess ? resident_prepare() : -1;
 }
 
 int launch_loop_reset(const Buffers &B, cudaStream_t st)

@@ -66,7 +66,7 @@ __device__ __forceinline__ void wall_slot(const Buffers &B, int s, int cur, int 
         acc[1] += p * W + Wg;
         acc[2] += u * W;
         acc[3] += v * W;
-        acc[4] += w * W;
+        if (D == 3) acc[4] += w * W;
     };
     if constexpr (F32) {
         for (int m = sub; 2 * m < cnt; m += kWallLanes) {
@@ -98,15 +98,14 @@ __device__ __forceinline__ void wall_slot(const Buffers &B, int s, int cur, int 
 #pragma unroll
     for (int o = kWallLanes / 2; o > 0; o >>= 1)
 #pragma unroll
-        for (int t = 0; t < 5; ++t) acc[t] += __shfl_xor_sync(gmask, acc[t], o);
+        for (int t = 0; t < D + 2; ++t) acc[t] += __shfl_xor_sync(gmask, acc[t], o);
     if (sub != 0) return;
-    const double sw = acc[0];
-    double gv[3];
-    for (int a = 0; a < 3; ++a) {
-        const double vw = a < D ? B.vn_a[(size_t)a * B.n + s] : 0.0;
-        gv[a] = 2.0 * vw - (sw > 0 ? acc[2 + a] / sw : 0.0);
-    }
-    double pw = sw > 0 ? acc[1] / sw : 0.0;
+    // (FP64 instructions are what this phase takes: one reciprocal for all)
+    const double sw = acc[0], inv = sw > 0 ? rcp_step(sw) : 0.0;
+    double gv[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int a = 0; a < D; ++a) gv[a] = 2.0 * B.vn_a[(size_t)a * B.n + s] - acc[2 + a] * inv;
+    double pw = acc[1] * inv;
     if (pw < 0.0 && B.phys[B.inst_of[s]].free_surface) pw = 0.0;   // free-surface runs (Sec. 3.2)
     if (F32) B.nb32[cur][s] = make_float4((float)gv[0], (float)gv[1], (float)gv[2], (float)pw);
     else B.nb64[cur][s] = make_double4_32a(gv[0], gv[1], gv[2], pw);
@@ -528,36 +527,28 @@ __device__ __forceinline__ void pair_sums64(const Buffers &B, const Phys &P, con
 // the FP64 pipe: the residual terms are summed per warp with error-free
 // two-sum compensation (a double-float sum, accurate to ~1e-12 of the total)
 // and the warp totals are carried on in FP64. The FP64 path sums in FP64.
-// For slot s2 (fl: a fluid slot) with its rates apT, FT from phase 1, by every
-// lane of the warp; the warp's residual sums come back on lane 0.
+// update_slot: for one slot (fl: a fluid slot) with its rates apT, FT from phase 1,
+// by every lane of the warp: V^k and p-hat become iterate k + 1's; src is s_a's
+// part; the warp's residual sums come back on lane 0.
 template <int D, bool F32>
-__device__ __forceinline__ void update_and_residuals(const Buffers &B, const Phys &P, int cur, int s2, bool fl,
-                                                     Real<F32> apT, const Real<F32> *FT, double &w_ap, double &w_av)
+__device__ __forceinline__ void update_slot(const Phys &P, bool fl, Real<F32> apT, const Real<F32> *FT, double *vk,
+                                            const double *src, Real<F32> &p, double &w_ap, double &w_av)
 {
-    const int nxt = cur ^ 1;
-    const int n = B.n;
-    if (F32) {
+    if constexpr (F32) {
         float r_ap = 0.f, r_av = 0.f;
         if (fl) {
-            const float apf = (float)apT;
-            float vnf[3] = {0.f, 0.f, 0.f};
             float av2 = 0.f;
 #pragma unroll
             for (int a = 0; a < D; ++a) {
-                const size_t q = (size_t)a * n + s2;
-                const double vk = B.vk[cur][q];
                 const double Fv = (double)FT[a];
-                const double av = __fma_rn(P.kappa, Fv, -__fma_rn(P.kc3, vk, B.s_a[q]));
-                const double vnew = __fma_rn(P.dtau, av, vk);
-                B.vk[nxt][q] = vnew;
-                vnf[a] = (float)vnew;
+                const double av = __fma_rn(P.kappa, Fv, -__fma_rn(P.kc3, vk[a], src[a]));
+                vk[a] = __fma_rn(P.dtau, av, vk[a]);
                 const float avf = (float)av;
                 av2 = __fmaf_rn(avf, avf, av2);
             }
-            const float pnew = __fmaf_rn(P.dtau_f, apf, B.nb32[cur][s2].w);
-            B.nb32[nxt][s2] = make_float4(vnf[0], vnf[1], vnf[2], pnew);
+            p = __fmaf_rn(P.dtau_f, apT, p);
             r_av = sqrtf(av2);
-            r_ap = fabsf(apf);
+            r_ap = fabsf(apT);
         }
         float sa = r_ap, ea = 0.f, sb = r_av, eb = 0.f;
         warp_sum2(sa, ea);
@@ -567,26 +558,53 @@ __device__ __forceinline__ void update_and_residuals(const Buffers &B, const Phy
     } else {
         double r_ap = 0.0, r_av = 0.0;
         if (fl) {
-            const double apv = (double)apT;
-            double vnew[3] = {0, 0, 0};
             double av2 = 0.0;
 #pragma unroll
             for (int a = 0; a < D; ++a) {
-                const size_t q = (size_t)a * n + s2;
-                const double vk = B.vk[cur][q];
-                const double Fv = (double)FT[a];
-                const double av = __fma_rn(P.kappa, Fv, -__fma_rn(P.kc3, vk, B.s_a[q]));
-                vnew[a] = __fma_rn(P.dtau, av, vk);
-                B.vk[nxt][q] = vnew[a];
+                const double av = __fma_rn(P.kappa, FT[a], -__fma_rn(P.kc3, vk[a], src[a]));
+                vk[a] = __fma_rn(P.dtau, av, vk[a]);
                 av2 = __fma_rn(av, av, av2);
             }
-            const double pnew = __fma_rn(P.dtau, apv, B.nb64[cur][s2].w);
-            B.nb64[nxt][s2] = make_double4_32a(vnew[0], vnew[1], vnew[2], pnew);
+            p = __fma_rn(P.dtau, apT, p);
             r_av = sqrt(av2);
-            r_ap = fabs(apv);
+            r_ap = fabs(apT);
         }
         w_ap = warp_sum<double>(r_ap);
         w_av = warp_sum<double>(r_av);
+    }
+}
+
+// The packed (V, p-hat) of slot s in buffer `buf`.
+template <int D, bool F32>
+__device__ __forceinline__ void store_state(const Buffers &B, int buf, int s, const double *v, Real<F32> p)
+{
+    if constexpr (F32) B.nb32[buf][s] = make_float4((float)v[0], (float)v[1], D == 3 ? (float)v[2] : 0.f, p);
+    else B.nb64[buf][s] = make_double4_32a(v[0], v[1], D == 3 ? v[2] : 0.0, p);
+}
+
+// For slot s2 by every lane of the warp: loads, update_slot, stores.
+template <int D, bool F32>
+__device__ __forceinline__ void update_and_residuals(const Buffers &B, const Phys &P, int cur, int s2, bool fl,
+                                                     Real<F32> apT, const Real<F32> *FT, double &w_ap, double &w_av)
+{
+    const int nxt = cur ^ 1;
+    double vk[3] = {0, 0, 0}, src[3] = {0, 0, 0};
+    Real<F32> p = 0;
+    if (fl) {
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            const size_t q = (size_t)a * B.n + s2;
+            vk[a] = B.vk[cur][q];
+            src[a] = B.s_a[q];
+        }
+        if constexpr (F32) p = B.nb32[cur][s2].w;
+        else p = B.nb64[cur][s2].w;
+    }
+    update_slot<D, F32>(P, fl, apT, FT, vk, src, p, w_ap, w_av);
+    if (fl) {
+#pragma unroll
+        for (int a = 0; a < D; ++a) B.vk[nxt][(size_t)a * B.n + s2] = vk[a];
+        store_state<D, F32>(B, nxt, s2, vk, p);
     }
 }
 
@@ -725,28 +743,33 @@ __device__ __forceinline__ unsigned long long global_ns()
 
 // Grid barrier for a cooperative launch (all blocks resident): arrival counter
 // `bar`, reset to 0 before the launch; the epoch-th barrier waits for
-// epoch * gridDim.x arrivals. The wait gives up after limit_ns (one second
-// unless a test shortens it), raises kErrBarrier and returns false (the caller
-// then stops iterating).
+// epoch * gridDim.x arrivals: a release arrival of the block's writes, acquire
+// polls. The wait gives up after limit_ns (one second unless a test shortens it),
+// raises kErrBarrier and returns false (the caller then stops iterating).
 __device__ bool grid_barrier(unsigned int *bar, unsigned int epoch, uint32_t *err, int &ok_sh,
                              unsigned long long limit_ns)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
         const unsigned int target = epoch * gridDim.x;
-        __threadfence();
-        atomicAdd(bar, 1u);
-        int ok = 1;
-        const unsigned long long t0 = global_ns();
-        while (*(volatile unsigned int *)bar < target) {
-            __nanosleep(32);
-            if (global_ns() - t0 > limit_ns) {
-                atomicOr(err, kErrBarrier);
-                ok = 0;
-                break;
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        int ok = 1, polls = 0;
+        unsigned long long t0 = 0;
+        for (;;) {
+            unsigned int v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            if (v >= target) break;
+            // (the clock every 64 polls: reading it costs more than a poll)
+            if (limit_ns == 0 || (++polls & 63) == 0) {
+                const unsigned long long now = global_ns();
+                if (t0 == 0) t0 = now;
+                if (limit_ns == 0 || now - t0 > limit_ns) {
+                    atomicOr(err, kErrBarrier);
+                    ok = 0;
+                    break;
+                }
             }
         }
-        __threadfence();
         ok_sh = ok;
     }
     __syncthreads();

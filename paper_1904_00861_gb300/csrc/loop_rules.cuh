@@ -6,25 +6,40 @@
 
 namespace dtsph {
 
-// Stop rules of Sec. 3.4 on the residual history (ring of the last 16).
+// Stop rules of Sec. 3.4 on the residual history (ring of the last 16). One thread
+// runs them between an iteration's barrier and the next iteration, where every
+// dependent FP64 instruction counts (an iteration of a small problem took 6 to 12 us
+// in its reduction and these rules), so they compare the residuals, which are
+// not negative, as integers of the same order, and divide only where the product
+// form lies within rounding of the threshold.
 __device__ inline int stop_rule(const LoopState &L, int k1)
 {
-    double rp = L.hist_p[(k1 - 1) & 15], rv = L.hist_v[(k1 - 1) & 15];
-    if (!isfinite(rp) || !isfinite(rv)) return 3;
+    const long long kInf = 0x7ff0000000000000ll;
+    const long long rp = __double_as_longlong(L.hist_p[(k1 - 1) & 15]), rv = __double_as_longlong(L.hist_v[(k1 - 1) & 15]);
+    if ((rp & kInf) == kInf || (rv & kInf) == kInf) return 3;
     if (L.fixed_iters > 0) return k1 >= L.fixed_iters ? 4 : -1;
-    if (rp < L.eps && rv < L.eps) return 0;
+    const long long eps = __double_as_longlong(L.eps);
+    if (rp < eps && rv < eps) return 0;
     int w = L.stag_window;
     if (w > 0 && k1 >= w) {
         bool stag = true;
         for (int which = 0; which < 2 && stag; ++which) {
             const double *h = which ? L.hist_v : L.hist_p;
-            double lo = h[(k1 - 1) & 15], hi = lo;
+            long long lo = __double_as_longlong(h[(k1 - 1) & 15]), hi = lo;
             for (int t = k1 - w; t < k1; ++t) {
-                double v = h[t & 15];
-                lo = fmin(lo, v);
-                hi = fmax(hi, v);
+                const long long v = __double_as_longlong(h[t & 15]);
+                lo = min(lo, v);
+                hi = max(hi, v);
             }
-            if (!(hi > 0.0 && (hi - lo) / hi < L.stag_tol)) stag = false;
+            if (hi <= 0) {
+                stag = false;
+                break;
+            }
+            // (hi - lo) / hi < stag_tol: by hi - lo against stag_tol hi, 4096 units in
+            // the last place apart; nearer, by the quotient
+            const double top = __longlong_as_double(hi), d = __dsub_rn(top, __longlong_as_double(lo));
+            const long long gap = __double_as_longlong(d) - __double_as_longlong(__dmul_rn(L.stag_tol, top));
+            stag = gap < -4096 || (gap <= 4096 && d / top < L.stag_tol);
         }
         if (stag) return 1;
     }
@@ -44,6 +59,18 @@ __device__ __forceinline__ T warp_sum(T v)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Warp sums of a (result on lanes 0-15) and b (on lanes 16-31), as warp_sum forms
+// them (xor 16, 8, 4, 2, 1): after the first step each half of the warp carries one.
+__device__ __forceinline__ double warp_sum_halves(double a, double b)
+{
+    const bool up = threadIdx.x & 16;
+    const double keep = up ? b : a, give = up ? a : b;
+    double v = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 
@@ -73,14 +100,10 @@ __device__ __forceinline__ void reduce_tiles(const double *blk, int ntiles, doub
         a += __ldcg(&blk[2 * q]);
         b += __ldcg(&blk[2 * q + 1]);
     }
-    a = warp_sum<double>(a);
-    b = warp_sum<double>(b);
+    const double v = warp_sum_halves(a, b);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     __syncthreads();
-    if (lane == 0) {
-        red[0][wid] = a;
-        red[1][wid] = b;
-    }
+    if ((lane & 15) == 0) red[lane >> 4][wid] = v;
     __syncthreads();
     if (threadIdx.x == 0) {
         sa = 0;
