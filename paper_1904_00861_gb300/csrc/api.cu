@@ -731,32 +731,28 @@ int enqueue_pre_loop(dtsph_ctx *c, cudaStream_t st)
         // r^n as without reuse; either way the state-n pass runs on the lists
         Buffers Br = B;
         Br.relist_run = 1;
-        k += launch_binning(Br, Br.x_a, Br.gid_a, st);
-        k += launch_permute_a_to_b(Br, st);
+        k += launch_bin_a_to_b(Br, st);
         launch_nlist(Br, Br.x_b, st);
         Br.relist_run = 0;
         k += 1 + launch_same_order_a_to_b(Br, st);
         k += launch_state_n(B, true, st, false);
     } else {
-        k += launch_binning(B, B.x_a, B.gid_a, st);      // cells at r^n
-        k += launch_permute_a_to_b(B, st);
+        k += launch_bin_a_to_b(B, st);                    // cells at r^n
         k += launch_state_n(B, true, st);                 // walls, rates, predictor
     }
-    k += launch_binning(B, B.xp_b, B.gid_b, st);         // cells at r^0
-    k += launch_permute_b_to_a(B, st);
+    k += launch_bin_b_to_a(B, st);                       // cells at r^0; resets the loop, picks the form
     if (B.xk[0]) {
         k += launch_move_prepare(B, st);                          // particles moving in pseudo-time
     } else if (B.form_sel) {
-        // both forms in the graph: the reset kernel picks the step's form; the
-        // pair-cache pass returns at once when the step recomputes the terms
+        // both forms in the graph: the pair-cache pass returns at once when the
+        // step recomputes the terms
         launch_nlist(B, B.xp_a, st);
-        k += 1 + launch_loop_reset(B, st);
-        k += launch_pair_cache_pass(B, B.xp_a, B.gid_a, st);
+        k += 1 + launch_pair_cache_pass(B, B.xp_a, B.gid_a, st);
     } else if (B.form_a) {
         launch_nlist(B, B.xp_a, st);   // the loop recomputes the pair terms
-        k += 1 + launch_loop_reset(B, st);
+        k += 1;
     } else {
-        k += launch_pair_cache(B, B.xp_a, B.gid_a, st);   // also resets the loop state
+        k += launch_pair_cache(B, B.xp_a, B.gid_a, st);
     }
     return k;
 }
@@ -1047,8 +1043,7 @@ int autotune(dtsph_ctx *c)
     CK(cudaMemsetAsync(B.s_a, 0, nd * sizeof(double), c->stream));
     if (B.fp32c) CK(cudaMemsetAsync(B.nb32[0], 0, (size_t)B.n * sizeof(float4), c->stream));
     else CK(cudaMemsetAsync(B.nb64[0], 0, (size_t)B.n * sizeof(double4_32a), c->stream));
-    c->launches += launch_binning(B, B.x_a, B.gid_a, c->stream);
-    c->launches += launch_permute_a_to_b(B, c->stream);
+    c->launches += launch_bin_a_to_b(B, c->stream);
     // the loop runs in order A: the lists' order becomes it (with walls in the
     // caller's order, the candidates would run wall rows as fluid rows, stop on
     // non-finite residuals and show times that no step has)
@@ -1122,8 +1117,7 @@ int measure_form_costs(dtsph_ctx *c)
     CK(cudaMemsetAsync(B.s_a, 0, nd * sizeof(double), c->stream));
     if (B.fp32c) CK(cudaMemsetAsync(B.nb32[0], 0, (size_t)B.n * sizeof(float4), c->stream));
     else CK(cudaMemsetAsync(B.nb64[0], 0, (size_t)B.n * sizeof(double4_32a), c->stream));
-    c->launches += launch_binning(B, B.x_a, B.gid_a, c->stream);
-    c->launches += launch_permute_a_to_b(B, c->stream);
+    c->launches += launch_bin_a_to_b(B, c->stream);
     c->launches += launch_adopt_b(B, c->stream);   // (the loop runs in order A)
     constexpr int kReps = 5;
     cudaEvent_t e[2];
@@ -1495,8 +1489,7 @@ int dtsph_step(dtsph_ctx *c, int32_t nsteps)
         // bin at r^n, make that order A, list to 3h + list_skin: what the
         // steps' state-n pass reads
         const Buffers &B = c->B;
-        c->launches += launch_binning(B, B.x_a, B.gid_a, c->stream);
-        c->launches += launch_permute_a_to_b(B, c->stream);
+        c->launches += launch_bin_a_to_b(B, c->stream);
         c->launches += launch_adopt_b(B, c->stream);
         launch_nlist(B, B.x_a, c->stream);
         c->launches += 1;
@@ -1591,14 +1584,12 @@ int dtsph_eval_rates(dtsph_ctx *c, double *ap, double *F)
     CK(cudaSetDevice(c->device));
     const Buffers &B = c->B;
     c->lists_ready = false;                       // the lists are rebuilt at r^n in order B
-    c->launches += launch_binning(B, B.x_a, B.gid_a, c->stream);
-    c->launches += launch_permute_a_to_b(B, c->stream);
+    c->launches += launch_bin_a_to_b(B, c->stream);
     c->launches += launch_state_n(B, false, c->stream);
     const size_t bf = (size_t)B.nf * B.dim * sizeof(double), bp = (size_t)B.nf * sizeof(double);
     double *tmp = nullptr;
     CK(cudaMallocAsync((void **)&tmp, bf + bp, c->stream));
-    c->launches += launch_unpermute(B, B.gid_b, B.ap_b, tmp, 1, c->stream);
-    c->launches += launch_unpermute(B, B.gid_b, B.f_b, tmp + B.nf, B.dim, c->stream);
+    c->launches += launch_rates_out(B, tmp, tmp + B.nf, nullptr, c->stream);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(ap, tmp, bp, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaMemcpyAsync(F, tmp + B.nf, bf, cudaMemcpyDeviceToHost, c->stream));
@@ -1615,8 +1606,7 @@ int dtsph_build_neighbors(dtsph_ctx *c)
     CK(cudaSetDevice(c->device));
     const Buffers &B = c->B;
     c->lists_ready = false;                       // the lists are rebuilt at r^n in order B
-    c->launches += launch_binning(B, B.x_a, B.gid_a, c->stream);
-    c->launches += launch_permute_a_to_b(B, c->stream);
+    c->launches += launch_bin_a_to_b(B, c->stream);
     c->launches += launch_pair_cache(B, B.x_b, B.gid_b, c->stream);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(c->stream));
@@ -1669,8 +1659,7 @@ int dtsph_probe_iterate(dtsph_ctx *c, int32_t launches, float *ms_per_launch, do
     if (c->prm[0].shifting) {
         if (B.xk[0])
             return fail(c, DTSPH_E_STATE, "with particles moving in pseudo-time the probe needs a run without shifting");
-        c->launches += launch_binning(B, B.x_a, B.gid_a, c->stream);
-        c->launches += launch_permute_a_to_b(B, c->stream);
+        c->launches += launch_bin_a_to_b(B, c->stream);
         c->launches += launch_pair_cache(B, B.x_b, B.gid_b, c->stream);
         CK(cudaGetLastError());
         if (int r = device_error(c)) return r;

@@ -8,28 +8,15 @@
 // context are binned together: instance i's cells are numbered from its
 // cell_off, and the scan places its particles at its own (tile-aligned) slot
 // range.
-#include "dtsph_internal.cuh"
+#include "geometry.cuh"
+#include "loop_rules.cuh"
 
 namespace dtsph {
 
 namespace {
 
-__device__ __forceinline__ int cell_coord(double xa, double lo, double hi, double inv_s, int nc, int periodic,
-                                          uint32_t *err)
-{
-    int k = (int)floor((xa - lo) * inv_s);
-    if (k < 0) {
-        if (!periodic && xa < lo) atomicOr(err, kErrDomain);
-        k = 0;
-    }
-    if (k >= nc) {
-        if (!periodic && xa > hi) atomicOr(err, kErrDomain);
-        k = nc - 1;
-    }
-    return k;
-}
-
-// Cell (global index) of every particle of the source order; -1 for padding.
+// Cell (global index) of every particle of the source order; -1 for padding. (The
+// keys at r^0 are counted by the state-n pass that predicts the positions.)
 __global__ void __launch_bounds__(kBlock) k_bin_keys(Buffers B, const double *__restrict__ x,
                                                      const uint32_t *__restrict__ gid)
 {
@@ -42,15 +29,9 @@ __global__ void __launch_bounds__(kBlock) k_bin_keys(Buffers B, const double *__
     }
     const int inst = B.inst_of[i];
     const Geom &G = B.geo[inst];
-    int c = 0, mult = 1;
-    for (int a = 0; a < G.dim; ++a) {
-        int k = cell_coord(x[(size_t)a * B.n + i], G.lo[a], G.hi[a], G.inv_s[a], G.nc[a], G.periodic[a], B.err);
-        c += k * mult;
-        mult *= G.nc[a];
-    }
-    c += B.inst[inst].cell_off;
-    B.key[i] = c;
-    B.slot[i] = atomicAdd(&B.cell_count[c], 1);
+    double xi[3] = {0, 0, 0};
+    for (int a = 0; a < G.dim; ++a) xi[a] = x[(size_t)a * B.n + i];
+    count_key(B, G, B.inst[inst].cell_off, i, xi);
 }
 
 // Exclusive scan of the per-cell counts, shifted so that each instance's
@@ -145,29 +126,60 @@ __device__ __forceinline__ int cell_instance(const Buffers &B, int c)
 }
 
 // PER cells per thread; MULTI: several blocks, each with the carry of the
-// blocks before it (else one block scans every cell, with no carry)
+// blocks before it (else one block scans every cell, with no carry). A thread's
+// cells lie side by side, in 16-byte pieces (with 4-byte accesses PER apart, 32 lines
+// a request, the scan of a tank's 11,000 cells took 18 us; a binning there takes 13
+// us less now, the launch saved by k_rank_move included).
 template <int PER, bool MULTI>
 __global__ void __launch_bounds__(kScanThreads) k_scan_final(Buffers B)
 {
     if (skip_relist(B)) return;   // (the step graph: relisting or not)
-    const int base = blockIdx.x * kScanThreads * PER + threadIdx.x * PER;
+    static_assert(PER % 4 == 0, "whole pieces");
+    const int base = (blockIdx.x * kScanThreads + threadIdx.x) * PER;
     int v[PER];
     int s = 0;
+    int4 *count = reinterpret_cast<int4 *>(B.cell_count + base), *first = reinterpret_cast<int4 *>(B.cell_start + base);
+    const bool whole = base + PER <= B.ncell;
+    if (whole) {
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        v[k] = base + k < B.ncell ? B.cell_count[base + k] : 0;
-        s += v[k];
+        for (int k = 0; k < PER / 4; ++k) {
+            const int4 q = count[k];
+            v[4 * k] = q.x; v[4 * k + 1] = q.y; v[4 * k + 2] = q.z; v[4 * k + 3] = q.w;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < PER; ++k) v[k] = base + k < B.ncell ? B.cell_count[base + k] : 0;
     }
+#pragma unroll
+    for (int k = 0; k < PER; ++k) s += v[k];
     int run = block_exclusive_scan(s) + (MULTI ? B.scan_tmp[blockIdx.x] : 0);
     if (base < B.ncell) {
-        int inst = cell_instance(B, base);
+        int inst = B.ninst > 1 ? cell_instance(B, base) : 0;
+        int shift = B.inst[inst].shift, next = inst + 1 < B.ninst ? B.inst[inst + 1].cell_off : 0x7fffffff;
+#pragma unroll
         for (int k = 0; k < PER; ++k) {
             const int c = base + k;
-            if (c >= B.ncell) break;
-            while (inst + 1 < B.ninst && B.inst[inst + 1].cell_off <= c) ++inst;
-            B.cell_start[c] = run + B.inst[inst].shift;
-            run += v[k];
-            B.cell_count[c] = 0;
+            while (next <= c) {
+                shift = B.inst[++inst].shift;
+                next = inst + 1 < B.ninst ? B.inst[inst + 1].cell_off : 0x7fffffff;
+            }
+            const int n = v[k];
+            v[k] = run + shift;
+            run += n;
+        }
+        if (whole) {
+#pragma unroll
+            for (int k = 0; k < PER / 4; ++k) {
+                first[k] = make_int4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+                count[k] = make_int4(0, 0, 0, 0);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < PER; ++k)
+                if (base + k < B.ncell) {
+                    B.cell_start[base + k] = v[k];
+                    B.cell_count[base + k] = 0;
+                }
         }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) B.cell_start[B.ncell] = B.n;
@@ -181,25 +193,6 @@ __global__ void __launch_bounds__(kBlock) k_scatter(Buffers B)
     const int c = B.key[i];
     if (c < 0) return;
     B.unsorted[B.cell_start[c] + B.slot[i]] = i;
-}
-
-// Orders each cell by caller index: the particle in unsorted slot t moves to
-// start[c] + (number of particles of its cell with a smaller caller index).
-// One thread per slot; cells hold a few tens of particles; padding slots (never
-// written by the scatter) stay -1.
-__global__ void __launch_bounds__(kBlock) k_cell_rank(Buffers B, const uint32_t *__restrict__ gid)
-{
-    if (skip_relist(B)) return;   // (the step graph: relisting or not)
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= B.n) return;
-    const int i = B.unsorted[t];
-    if (i < 0) return;
-    const int c = B.key[i];
-    const uint32_t gi = gid[i];
-    const int b = B.cell_start[c], e = B.cell_start[c + 1];
-    int rank = 0;
-    for (int u = b; u < e; ++u) rank += gid[B.unsorted[u]] < gi;
-    B.perm[b + rank] = i;
 }
 
 // FP32 offset of slot s from the origin of its cell; .w is 1 for a wall particle.
@@ -236,8 +229,6 @@ __device__ __forceinline__ float4 cell_offset_near(const Geom &G, int local_cell
     return make_float4(f[0], f[1], f[2], wall ? 1.f : 0.f);
 }
 
-// A -> B at the start of a step: state n, and the packed (V^n, p^n) that the
-// state-n pair pass gathers.
 // The packed copy of a wall slot's prescribed velocity that the loop gathers
 // with the neighbour states (contexts with walls only).
 __device__ __forceinline__ void store_wall_velocity(const Buffers &B, int s, const double *u)
@@ -246,24 +237,17 @@ __device__ __forceinline__ void store_wall_velocity(const Buffers &B, int s, con
     if (B.wv64) B.wv64[s] = make_double4_32a(u[0], u[1], u[2], 0.0);
 }
 
-// SAME: order B is order A (the r^0 lists of the previous step serve this
-// step): every slot keeps its place and its cell of that binning, and the FP32
-// offsets are taken at r^n from that cell's origin.
+// A -> B at the start of a step, the particle in slot o of order A to slot s of
+// order B: state n, and the packed (V^n, p^n) that the state-n pair pass gathers.
+// SAME: order B is order A (the r^0 lists of the previous step serve this step):
+// every slot keeps its place and its cell of that binning, and the FP32 offsets are
+// taken at r^n from that cell's origin.
 template <bool SAME>
-__global__ void __launch_bounds__(kBlock) k_permute_a_to_b(Buffers B)
+__device__ __forceinline__ void move_a_to_b(const Buffers &B, int o, int s, int cell)
 {
-    if (skip_relist(B)) return;   // (the step graph: relisting or not)
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= B.n) return;
-    const int o = SAME ? (B.gid_a[s] == kNoParticle ? -1 : s) : B.perm[s];
-    if (o < 0) {
-        B.gid_b[s] = kNoParticle;
-        return;
-    }
     const int n = B.n, dim = B.dim;
     const uint32_t g = B.gid_a[o];
     B.gid_b[s] = g;
-    const int cell = SAME ? B.cell_a[s] : B.key[o];
     B.cell_b[s] = cell;
     double v[3] = {0, 0, 0};
     for (int a = 0; a < dim; ++a) {
@@ -286,25 +270,25 @@ __global__ void __launch_bounds__(kBlock) k_permute_a_to_b(Buffers B)
     }
 }
 
-// B -> A after the predictor: the loop order. Carries r^n, r^0, V^n, the BDF2
-// source, and seeds iterate 0 (V^0, p-hat^0).
-__global__ void __launch_bounds__(kBlock) k_permute_b_to_a(Buffers B)
+__global__ void __launch_bounds__(kBlock) k_same_a_to_b(Buffers B)
 {
+    if (skip_relist(B)) return;   // (the step graph: relisting or not)
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (B.relist && s == 0) *B.relist = 0;   // the step's relisting, if any, is done
     if (s >= B.n) return;
-    const int o = B.perm[s];
-    if (o < 0) {
-        B.gid_a[s] = kNoParticle;
-        return;
-    }
+    if (B.gid_a[s] == kNoParticle) B.gid_b[s] = kNoParticle;
+    else move_a_to_b<true>(B, s, s, B.cell_a[s]);
+}
+
+// B -> A after the predictor, slot o of order B to slot s of order A, the loop
+// order. Carries r^n, r^0, V^n, the BDF2 source, and seeds iterate 0 (V^0, p-hat^0).
+__device__ __forceinline__ void move_b_to_a(const Buffers &B, int o, int s, int cell)
+{
     const int n = B.n, dim = B.dim;
     const uint32_t g = B.gid_b[o];
     B.gid_a[s] = g;
     const bool wall = g >= (uint32_t)B.nf;
     if (B.slot_of && !wall) B.slot_of[g] = s;
     if (B.wslot_a && wall) B.wslot_a[g - (uint32_t)B.nf] = s;
-    const int cell = B.key[o];
     B.cell_a[s] = cell;
     double v[3] = {0, 0, 0}, u[3] = {0, 0, 0};
     for (int a = 0; a < dim; ++a) {
@@ -328,6 +312,46 @@ __global__ void __launch_bounds__(kBlock) k_permute_b_to_a(Buffers B)
     }
 }
 
+// Orders each cell by caller index and moves the particles there: the particle in
+// unsorted slot t goes to start[c] + (number of particles of its cell with a smaller
+// caller index). One thread per slot; cells hold a few tens of particles; padding
+// slots (never written by the scatter, -1) stay where they are. Moving them in
+// the same pass saves a launch and the permutation's round trip. TO_A: the
+// binning at r^0 into order A; its first block also resets the pseudo-time loop
+// (and picks the step's pair-term form).
+template <bool TO_A>
+__global__ void __launch_bounds__(kBlock) k_rank_move(Buffers B)
+{
+    if (skip_relist(B)) return;   // (the step graph: relisting or not)
+    if constexpr (TO_A) {
+        if (blockIdx.x == 0) {
+            if (threadIdx.x == 0 && B.relist) *B.relist = 0;   // the step's relisting, if any, is done
+            if (B.form_sel) select_form(B);
+            reset_loops(B);
+        }
+    }
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= B.n) return;
+    const int i = B.unsorted[t];
+    if (i < 0) {
+        (TO_A ? B.gid_a : B.gid_b)[t] = kNoParticle;
+        return;
+    }
+    const uint32_t *gid = TO_A ? B.gid_b : B.gid_a;
+    const int c = B.key[i];
+    const uint32_t gi = gid[i];
+    const int b = B.cell_start[c], e = B.cell_start[c + 1];
+    int rank = 0;
+    for (int u = b; u < e; ++u) rank += gid[B.unsorted[u]] < gi;
+    const int s = b + rank;
+    if constexpr (TO_A) {
+        move_b_to_a(B, i, s, c);
+    } else {
+        B.perm[s] = i;
+        move_a_to_b<false>(B, i, s, c);
+    }
+}
+
 // Caller order -> order A from AoS inputs: slot s of instance i holds its fluid
 // particle s - slot_off (caller index foff + ...), then its walls, then padding.
 // An input coordinate: flags a non-finite value; on a periodic axis brings a
@@ -347,16 +371,12 @@ __device__ __forceinline__ double input_coord(double xa, const Geom &G, int a, u
     return y;
 }
 
-__global__ void __launch_bounds__(kBlock) k_scatter_in(Buffers B, const double *__restrict__ x,
-                                                       const double *__restrict__ v, const double *__restrict__ p,
-                                                       const double *__restrict__ vprev,
-                                                       const double *__restrict__ xw, const double *__restrict__ vw)
+__device__ __forceinline__ void scatter_slot(const Buffers &B, const Inst &I, const Geom &G, int s,
+                                             const double *__restrict__ x, const double *__restrict__ v,
+                                             const double *__restrict__ p, const double *__restrict__ vprev,
+                                             const double *__restrict__ xw, const double *__restrict__ vw)
 {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= B.n) return;
     const int n = B.n, dim = B.dim;
-    const Inst I = B.inst[B.inst_of[s]];
-    const Geom &G = B.geo[B.inst_of[s]];
     const int local = s - I.slot_off;
     if (local < I.nf) {
         const size_t f = (size_t)I.foff + local;
@@ -387,6 +407,54 @@ __global__ void __launch_bounds__(kBlock) k_scatter_in(Buffers B, const double *
     }
 }
 
+__global__ void __launch_bounds__(kBlock) k_scatter_in(Buffers B, const double *__restrict__ x,
+                                                       const double *__restrict__ v, const double *__restrict__ p,
+                                                       const double *__restrict__ vprev,
+                                                       const double *__restrict__ xw, const double *__restrict__ vw)
+{
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= B.n) return;
+    const int i = B.inst_of[s];
+    scatter_slot(B, B.inst[i], B.geo[i], s, x, v, p, vprev, xw, vw);
+}
+
+// The first launch of the allocation-free rate evaluation (one instance): its tables
+// from values into device memory, the cell counters and the permutation slots that
+// the counting sort expects cleared, and the particles into order A.
+__global__ void __launch_bounds__(kBlock) k_begin_one(Buffers B, Inst I, Geom G, Phys P, const double *__restrict__ x,
+                                                      const double *__restrict__ v, const double *__restrict__ p,
+                                                      const double *__restrict__ xw, const double *__restrict__ vw)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t == 0) {
+        *const_cast<Inst *>(B.inst) = I;
+        *const_cast<Geom *>(B.geo) = G;
+        *const_cast<Phys *>(B.phys) = P;
+    }
+    for (int c = t; c < B.ncell; c += gridDim.x * blockDim.x) B.cell_count[c] = 0;
+    if (t >= B.n) return;
+    B.unsorted[t] = -1;
+    const_cast<uint16_t *>(B.inst_of)[t] = 0;
+    scatter_slot(B, I, G, t, x, v, p, nullptr, xw, vw);
+}
+
+// The rates of order B in caller order, and (status not null) the device-side
+// error bits as a status code.
+__global__ void __launch_bounds__(kBlock) k_rates_out(Buffers B, double *__restrict__ ap, double *__restrict__ F,
+                                                      int32_t *status)
+{
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s == 0 && status) {
+        const uint32_t e = *B.err;
+        *status = (e & kErrCapacity) ? DTSPH_E_CAPACITY : (e & kErrDomain) ? DTSPH_E_DOMAIN : DTSPH_OK;
+    }
+    if (s >= B.n) return;
+    const uint32_t g = B.gid_b[s];
+    if (g >= (uint32_t)B.nf) return;
+    ap[g] = B.ap_b[s];
+    for (int a = 0; a < B.dim; ++a) F[(size_t)g * B.dim + a] = B.f_b[(size_t)a * B.n + s];
+}
+
 // Slot order -> caller order (AoS), fluid particles only.
 __global__ void __launch_bounds__(kBlock) k_unpermute(int n, int nf, int comps, const uint32_t *__restrict__ gid,
                                                       const double *__restrict__ src, double *__restrict__ out)
@@ -398,23 +466,16 @@ __global__ void __launch_bounds__(kBlock) k_unpermute(int n, int nf, int comps, 
     for (int a = 0; a < comps; ++a) out[(size_t)g * comps + a] = src[(size_t)a * n + s];
 }
 
-__global__ void k_fill_instance(Inst *inst, Geom *geo, Phys *phys, int i, Inst I, Geom G, Phys P)
-{
-    inst[i] = I;
-    geo[i] = G;
-    phys[i] = P;
-}
-
 inline int blocks(int n) { return (n + kBlock - 1) / kBlock; }
 
 }  // namespace
 
-int launch_binning(const Buffers &B, const double *x_keys, const uint32_t *gid_src, cudaStream_t st)
+// From the keys to the slots: the scan of the cell counts, the scatter.
+static int launch_sort(const Buffers &B, cudaStream_t st)
 {
-    k_bin_keys<<<blocks(B.n), kBlock, 0, st>>>(B, x_keys, gid_src);
     // up to kScanCells1 cells one block scans them all; more take the block
     // totals, their scan, and the block scans with their carries
-    int k = 3;
+    int k = 2;
     if (B.ncell <= kScanCells1) {
         k_scan_final<kScanPerThread1, false><<<1, kScanThreads, 0, st>>>(B);
     } else {
@@ -425,19 +486,40 @@ int launch_binning(const Buffers &B, const double *x_keys, const uint32_t *gid_s
         k += 2;
     }
     k_scatter<<<blocks(B.n), kBlock, 0, st>>>(B);
-    k_cell_rank<<<blocks(B.n), kBlock, 0, st>>>(B, gid_src);
-    return k + 1;
+    return k;
 }
 
-int launch_permute_a_to_b(const Buffers &B, cudaStream_t st)
+int launch_bin_a_to_b(const Buffers &B, cudaStream_t st)
 {
-    k_permute_a_to_b<false><<<blocks(B.n), kBlock, 0, st>>>(B);
-    return 1;
+    k_bin_keys<<<blocks(B.n), kBlock, 0, st>>>(B, B.x_a, B.gid_a);
+    const int k = launch_sort(B, st);
+    k_rank_move<false><<<blocks(B.n), kBlock, 0, st>>>(B);
+    return k + 2;
+}
+
+int launch_bin_b_to_a(const Buffers &B, cudaStream_t st)
+{
+    const int k = launch_sort(B, st);                    // (the predictor counted the keys)
+    k_rank_move<true><<<blocks(B.n), kBlock, 0, st>>>(B);
+    return k + 1;
 }
 
 int launch_same_order_a_to_b(const Buffers &B, cudaStream_t st)
 {
-    k_permute_a_to_b<true><<<blocks(B.n), kBlock, 0, st>>>(B);
+    k_same_a_to_b<<<blocks(B.n), kBlock, 0, st>>>(B);
+    return 1;
+}
+
+int launch_begin_one(const Buffers &B, const Inst &I, const Geom &G, const Phys &P, const double *x, const double *v,
+                     const double *p, const double *xw, const double *vw, cudaStream_t st)
+{
+    k_begin_one<<<blocks(B.n), kBlock, 0, st>>>(B, I, G, P, x, v, p, xw, vw);
+    return 1;
+}
+
+int launch_rates_out(const Buffers &B, double *ap, double *F, int32_t *status, cudaStream_t st)
+{
+    k_rates_out<<<blocks(B.n), kBlock, 0, st>>>(B, ap, F, status);
     return 1;
 }
 
@@ -514,12 +596,6 @@ int launch_scatter_same(const Buffers &B, const double *x, const double *v, cons
     return 1;
 }
 
-int launch_permute_b_to_a(const Buffers &B, cudaStream_t st)
-{
-    k_permute_b_to_a<<<blocks(B.n), kBlock, 0, st>>>(B);
-    return 1;
-}
-
 int launch_scatter_in(const Buffers &B, const double *x, const double *v, const double *p, const double *vprev,
                       const double *xw, const double *vw, cudaStream_t st)
 {
@@ -548,13 +624,6 @@ int launch_copy(const double *src, double *dst, size_t count, cudaStream_t st)
 int launch_unpermute(const Buffers &B, const uint32_t *gid, const double *src, double *out, int comps, cudaStream_t st)
 {
     k_unpermute<<<blocks(B.n), kBlock, 0, st>>>(B.n, B.nf, comps, gid, src, out);
-    return 1;
-}
-
-int launch_fill_instance(Inst *inst, Geom *geo, Phys *phys, int i, const Inst &I, const Geom &G, const Phys &P,
-                         cudaStream_t st)
-{
-    k_fill_instance<<<1, 1, 0, st>>>(inst, geo, phys, i, I, G, P);
     return 1;
 }
 

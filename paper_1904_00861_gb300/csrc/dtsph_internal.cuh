@@ -283,9 +283,10 @@ __device__ __forceinline__ int block_instance(const Buffers &B, int first)
 // ------------------------------------------------------------ launchers
 // Every launcher enqueues on `st` and returns the number of kernels launched.
 
-int launch_binning(const Buffers &B, const double *x_keys, const uint32_t *gid_src, cudaStream_t st);
-int launch_permute_a_to_b(const Buffers &B, cudaStream_t st);
-int launch_permute_b_to_a(const Buffers &B, cudaStream_t st);
+// Bins at r^n (x_a) and moves the state into order B; bins at r^0 (keys counted by
+// the predictor) and moves it into order A, resetting the loop.
+int launch_bin_a_to_b(const Buffers &B, cudaStream_t st);
+int launch_bin_b_to_a(const Buffers &B, cudaStream_t st);
 #ifdef __CUDACC__
 // True in a launch of the step graph guarded on relisting (see Buffers::relist)
 // whose condition does not hold. Block-uniform.
@@ -349,10 +350,11 @@ int launch_unpermute(const Buffers &B, const uint32_t *gid, const double *src, d
 int launch_copy(const double *src, double *dst, size_t count, cudaStream_t st);
 int launch_scatter_in(const Buffers &B, const double *x, const double *v, const double *p, const double *vprev,
                       const double *xw, const double *vw, cudaStream_t st);
-// Writes one instance's tables (inst/geo/phys entry i) from values, for callers
-// whose tables live in device memory they cannot copy into from the host.
-int launch_fill_instance(Inst *inst, Geom *geo, Phys *phys, int i, const Inst &I, const Geom &G, const Phys &P,
-                         cudaStream_t st);
+// The allocation-free rate evaluation's first and last launches: tables, cleared
+// scratch and the input of one instance; the rates in caller order with the status.
+int launch_begin_one(const Buffers &B, const Inst &I, const Geom &G, const Phys &P, const double *x, const double *v,
+                     const double *p, const double *xw, const double *vw, cudaStream_t st);
+int launch_rates_out(const Buffers &B, double *ap, double *F, int32_t *status, cudaStream_t st);
 
 int iterate_tiles(const Buffers &B);   // tiles of the iterate kernel (one block each)
 // The loop kernels without the pair cache (iterate_fa.cu; contexts without walls).

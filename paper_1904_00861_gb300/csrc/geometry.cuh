@@ -116,6 +116,34 @@ __device__ __forceinline__ void grad_coef(const Phys &P, const T *d, T r2, T *g,
     }
 }
 
+// The cell of a position along one axis; outside a closed axis: flagged, clamped.
+__device__ __forceinline__ int cell_coord(double xa, double lo, double hi, double inv_s, int nc, int periodic,
+                                          uint32_t *err)
+{
+    int k = (int)floor((xa - lo) * inv_s);
+    if (k < 0) {
+        if (!periodic && xa < lo) atomicOr(err, kErrDomain);
+        k = 0;
+    }
+    if (k >= nc) {
+        if (!periodic && xa > hi) atomicOr(err, kErrDomain);
+        k = nc - 1;
+    }
+    return k;
+}
+
+// Counts particle i of the source order, at x, into its cell (global index).
+__device__ __forceinline__ void count_key(const Buffers &B, const Geom &G, int cell_off, int i, const double *x)
+{
+    int c = cell_off, mult = 1;
+    for (int a = 0; a < G.dim; ++a) {
+        c += cell_coord(x[a], G.lo[a], G.hi[a], G.inv_s[a], G.nc[a], G.periodic[a], B.err) * mult;
+        mult *= G.nc[a];
+    }
+    B.key[i] = c;
+    B.slot[i] = atomicAdd(&B.cell_count[c], 1);
+}
+
 template <typename T> struct Packed;
 template <> struct Packed<double> { using type = double4_32a; };
 template <> struct Packed<float> { using type = float4; };

@@ -1208,51 +1208,7 @@ __global__ void __launch_bounds__(kBlock) k_outer(Buffers B)
         atomicMax((unsigned long long *)&rec->vmax, bits);
 }
 
-// The pair-term form of the step (form = 0, in the step graph): without the
-// cache when the latest finished step's iterations, averaged over the
-// instances with their fluid counts as weights, are at most kstar (an
-// instance with no finished step since the allocation counts one iteration).
-// Sums in a fixed order; one block.
-__device__ void select_form(const Buffers &B)
-{
-    __shared__ double kw[kBlock], w[kBlock];
-    double a = 0.0, b = 0.0;
-    for (int i = threadIdx.x; i < B.ninst; i += blockDim.x) {
-        const double nf = (double)B.inst[i].nf;
-        const int k = B.ls[i].last_iters;
-        a = __fma_rn(nf, (double)(k > 0 ? k : 1), a);
-        b = __dadd_rn(b, nf);
-    }
-    kw[threadIdx.x] = a;
-    w[threadIdx.x] = b;
-    __syncthreads();
-    for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-        if (threadIdx.x < h) {
-            kw[threadIdx.x] = __dadd_rn(kw[threadIdx.x], kw[threadIdx.x + h]);
-            w[threadIdx.x] = __dadd_rn(w[threadIdx.x], w[threadIdx.x + h]);
-        }
-        __syncthreads();
-    }
-    __shared__ int f_sh;
-    if (threadIdx.x == 0) {
-        const int f = kw[0] <= B.kstar * w[0] ? 1 : 0;
-        *B.form_sel = f;
-        B.form_count[f] += 1ull;
-        f_sh = f;
-    }
-    __syncthreads();
-    // without the cache the loop pauses after floor(kstar) iterations, where the
-    // cache would have paid for itself; the step then builds it and goes on, so
-    // a wrong guess costs about one cache pass
-    const int m = f_sh && B.kstar >= 1.0 && B.kstar < 1e6 ? (int)B.kstar : 0;
-    for (int i = threadIdx.x; i < B.ninst; i += blockDim.x) B.ls[i].pause_at = m;
-}
-
-__global__ void __launch_bounds__(kBlock) k_loop_reset(Buffers B)
-{
-    if (B.form_sel) select_form(B);
-    reset_loops(B);
-}
+__global__ void __launch_bounds__(kBlock) k_loop_reset(Buffers B) { reset_loops(B); }
 
 // A new particle state: every instance's step log starts again at step 0.
 __global__ void __launch_bounds__(kBlock) k_restart_steps(Buffers B)

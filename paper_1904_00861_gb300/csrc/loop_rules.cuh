@@ -144,6 +144,46 @@ __device__ __forceinline__ void reset_loops(const Buffers &B)
     }
 }
 
+// The pair-term form of the step (form = 0, in the step graph): without the
+// cache when the latest finished step's iterations, averaged over the
+// instances with their fluid counts as weights, are at most kstar (an
+// instance with no finished step since the allocation counts one iteration).
+// Sums in a fixed order; one block.
+__device__ inline void select_form(const Buffers &B)
+{
+    __shared__ double kw[kBlock], w[kBlock];
+    double a = 0.0, b = 0.0;
+    for (int i = threadIdx.x; i < B.ninst; i += blockDim.x) {
+        const double nf = (double)B.inst[i].nf;
+        const int k = B.ls[i].last_iters;
+        a = __fma_rn(nf, (double)(k > 0 ? k : 1), a);
+        b = __dadd_rn(b, nf);
+    }
+    kw[threadIdx.x] = a;
+    w[threadIdx.x] = b;
+    __syncthreads();
+    for (int h = blockDim.x / 2; h > 0; h >>= 1) {
+        if (threadIdx.x < h) {
+            kw[threadIdx.x] = __dadd_rn(kw[threadIdx.x], kw[threadIdx.x + h]);
+            w[threadIdx.x] = __dadd_rn(w[threadIdx.x], w[threadIdx.x + h]);
+        }
+        __syncthreads();
+    }
+    __shared__ int f_sh;
+    if (threadIdx.x == 0) {
+        const int f = kw[0] <= B.kstar * w[0] ? 1 : 0;
+        *B.form_sel = f;
+        B.form_count[f] += 1ull;
+        f_sh = f;
+    }
+    __syncthreads();
+    // without the cache the loop pauses after floor(kstar) iterations, where the
+    // cache would have paid for itself; the step then builds it and goes on, so
+    // a wrong guess costs about one cache pass
+    const int m = f_sh && B.kstar >= 1.0 && B.kstar < 1e6 ? (int)B.kstar : 0;
+    for (int i = threadIdx.x; i < B.ninst; i += blockDim.x) B.ls[i].pause_at = m;
+}
+
 // In a step graph that holds both pair-term forms (form = 0): true in a launch
 // whose form_run is not the step's current form. Block-uniform, so a kernel
 // may return before any barrier.

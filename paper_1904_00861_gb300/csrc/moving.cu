@@ -32,14 +32,10 @@ namespace {
 
 inline int blocks(int n) { return (n + kBlock - 1) / kBlock; }
 
-// r^{1/2} = r^0 (V~^0 = 0) in both position buffers, V~ = 0, and the loop state
-// reset. Walls keep r^0 in both buffers for the whole loop.
+// r^{1/2} = r^0 (V~^0 = 0) in both position buffers, V~ = 0. Walls keep r^0 in both buffers for the whole loop.
 template <bool F32>
 __global__ void __launch_bounds__(kBlock) k_move_init(Buffers B)
 {
-    if (blockIdx.x == 0) {
-        reset_loops(B);
-    }
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= B.n || B.gid_a[s] == kNoParticle) return;
     for (int a = 0; a < B.dim; ++a) {

@@ -38,7 +38,7 @@ constexpr size_t round256(size_t b) { return (b + 255) / 256 * 256; }
 
 // The arrays carve() takes, in its order, for n slots, ncell cells and K list
 // entries per slot: each size in bytes before its 256-byte rounding.
-constexpr int kCarveArrays = 30;
+constexpr int kCarveArrays = 29;
 struct Carve {
     size_t bytes[kCarveArrays];
     int count;
@@ -50,7 +50,7 @@ constexpr Carve carve_sizes(size_t n, size_t ncell, size_t K)
              4 * n, 4 * n, 4 * n, 4 * n,                          // key, slot, unsorted, perm
              4 * n, 8 * nd, 8 * nd, 8 * nd, 8 * n, 4 * n,         // gid_b, x_b, vn_b, vnm1_b, pn_b, cell_b
              16 * n, 32 * n, 8 * n, 8 * nd, 4 * n,                // off, packed (V, p), ap_b, f_b, pcount
-             4 * n * K, 4 * n * ((K + 7) / 8 * 8),                // pj, pjt (rows rounded up to 8)
+             4 * n * ((K + 7) / 8 * 8),                           // pjt (rows rounded up to 8)
              4 * (ncell + 1), 4 * (ncell + 1), 4 * (ncell / 4096 + 2),   // cell_count, cell_start, scan_tmp
              256, 2 * n, sizeof(Inst), sizeof(Geom), sizeof(Phys)},     // err, inst_of, tables
             kCarveArrays};
@@ -131,7 +131,6 @@ size_t carve(unsigned char *base, int n, int ncell, Buffers &B)
     B.ap_b = (double *)take();
     B.f_b = (double *)take();
     B.pcount = (int *)take();
-    B.pj = (uint32_t *)take();
     B.pjt = (uint32_t *)take();
     B.cell_count = (int *)take();
     B.cell_start = (int *)take();
@@ -142,13 +141,6 @@ size_t carve(unsigned char *base, int n, int ncell, Buffers &B)
     B.geo = (Geom *)take();
     B.phys = (Phys *)take();
     return at == sz.count ? off : (size_t)-1;
-}
-
-// The device-side error bits of the call as a status code for the caller.
-__global__ void k_noalloc_status(const uint32_t *err, int32_t *status)
-{
-    const uint32_t e = *err;
-    *status = (e & kErrCapacity) ? DTSPH_E_CAPACITY : (e & kErrDomain) ? DTSPH_E_DOMAIN : DTSPH_OK;
 }
 
 }  // namespace
@@ -201,26 +193,16 @@ extern "C" int dtsph_eval_rates_noalloc(const dtsph_params *p, int64_t nf, const
     I.nf = (int)nf;
     I.nw = (int)nw;
 
-    // the counting sort needs zeroed cell counters and -1 in the permutation
-    // slots it never writes, and padding slots need empty neighbour lists; the
-    // last call may have left any state there
-    if (cudaMemsetAsync(B.cell_count, 0, sizeof(int) * (size_t)B.ncell, st) != cudaSuccess ||
-        cudaMemsetAsync(B.err, 0, sizeof(uint32_t), st) != cudaSuccess ||
-        cudaMemsetAsync(B.pcount, 0, sizeof(int) * (size_t)B.n, st) != cudaSuccess ||
-        cudaMemsetAsync(B.unsorted, 0xff, sizeof(int) * (size_t)B.n, st) != cudaSuccess ||
-        cudaMemsetAsync(B.perm, 0xff, sizeof(int) * (size_t)B.n, st) != cudaSuccess ||
-        cudaMemsetAsync((void *)B.inst_of, 0, sizeof(uint16_t) * (size_t)B.n, st) != cudaSuccess) {
+    if (cudaMemsetAsync(B.err, 0, sizeof(uint32_t), st) != cudaSuccess) {
         cudaGetLastError();
         return DTSPH_E_CUDA;
     }
-    launch_fill_instance((Inst *)B.inst, (Geom *)B.geo, (Phys *)B.phys, 0, I, G, P, st);
-    launch_scatter_in(B, x, v, pr, nullptr, xw, vw, st);
-    launch_binning(B, B.x_a, B.gid_a, st);
-    launch_permute_a_to_b(B, st);
+    // (a small input's time is its launches: what the last call may have left in the
+    // array is cleared, and the tables are written, by the launch that reads the input)
+    launch_begin_one(B, I, G, P, x, v, pr, xw, vw, st);
+    launch_bin_a_to_b(B, st);
     launch_state_n(B, false, st);
-    launch_unpermute(B, B.gid_b, B.ap_b, ap, 1, st);
-    launch_unpermute(B, B.gid_b, B.f_b, F, B.dim, st);
-    if (status) k_noalloc_status<<<1, 1, 0, st>>>(B.err, status);
+    launch_rates_out(B, ap, F, status, st);
     if (cudaGetLastError() != cudaSuccess) return DTSPH_E_CUDA;
     return DTSPH_OK;
 }

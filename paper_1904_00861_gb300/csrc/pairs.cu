@@ -170,10 +170,16 @@ __global__ void __launch_bounds__(kBlock, F32 ? (D == 2 ? 4 : 3) : 1) k_state_n(
         }
         rates64<D, L>(P, k, A, apT, FT);
     }
-    if (gs == kNoParticle || lane_in != 0) return;
+    if (lane_in != 0) return;
+    if (gs == kNoParticle) {
+        if (PRED && s < n) B.key[s] = -1;
+        return;
+    }
+    double xp[3] = {0, 0, 0};                        // r^0
     if (!fluid) {
         if (PRED) {
-            for (int a = 0; a < D; ++a) B.xp_b[(size_t)a * n + s] = B.x_b[(size_t)a * n + s];
+            for (int a = 0; a < D; ++a) B.xp_b[(size_t)a * n + s] = xp[a] = B.x_b[(size_t)a * n + s];
+            count_key(B, G, B.inst[inst].cell_off, s, xp);
         }
         return;
     }
@@ -187,7 +193,7 @@ __global__ void __launch_bounds__(kBlock, F32 ? (D == 2 ? 4 : 3) : 1) k_state_n(
         // stay, and the source is -g (the loop forms F + g - 0)
         for (int a = 0; a < D; ++a) {
             const size_t q = (size_t)a * n + s;
-            B.xp_b[q] = B.x_b[q];
+            B.xp_b[q] = xp[a] = B.x_b[q];
             B.v0_b[q] = B.vn_b[q];
             B.s_b[q] = -P.g[a];
         }
@@ -197,17 +203,18 @@ __global__ void __launch_bounds__(kBlock, F32 ? (D == 2 ? 4 : 3) : 1) k_state_n(
             const size_t q = (size_t)a * n + s;
             // explicit roundings: the same bits in every kernel variant
             const double V = B.vn_b[q];
-            double xp = __fma_rn(0.5 * P.dt * P.dt, Fv[a], __fma_rn(P.dt, V, B.x_b[q]));
+            xp[a] = __fma_rn(0.5 * P.dt * P.dt, Fv[a], __fma_rn(P.dt, V, B.x_b[q]));
             if (G.periodic[a]) {
-                if (xp >= G.hi[a]) xp = __dsub_rn(xp, G.L[a]);
-                else if (xp < G.lo[a]) xp = __dadd_rn(xp, G.L[a]);
+                if (xp[a] >= G.hi[a]) xp[a] = __dsub_rn(xp[a], G.L[a]);
+                else if (xp[a] < G.lo[a]) xp[a] = __dadd_rn(xp[a], G.L[a]);
             }
-            B.xp_b[q] = xp;
+            B.xp_b[q] = xp[a];
             B.v0_b[q] = __fma_rn(P.dt, Fv[a], V);
             B.s_b[q] = __dmul_rn(P.kappa, __fma_rn(__fma_rn(-4.0, V, B.vnm1_b[q]), P.inv_2dt, -P.g[a]));
         }
         B.ph0_b[s] = __fma_rn(0.5 * P.dtau, apv, B.pn_b[s]);
     }
+    if (PRED) count_key(B, G, B.inst[inst].cell_off, s, xp);     // for the binning at r^0
 }
 
 // --------------------------------------------------------------- pair cache
@@ -324,7 +331,7 @@ __device__ __forceinline__ void pair_cache_slot64(const Buffers &B, const Geom &
 // The pair coefficients of every list entry (order of the latest binning):
 // gradW_ij and F_ij for a fluid slot, W_wf and rho0 (g . r_wf) W_wf for a wall
 // slot, at the entry's place in the sliced layout. Entries are independent, so
-// L only sets the parallelism. Block 0 also resets the pseudo-time loop state.
+// L only sets the parallelism.
 template <int D, bool F32, int L>
 __global__ void __launch_bounds__(kBlock) k_pair_cache(Buffers B, const double *__restrict__ xpos,
                                                        const uint32_t *__restrict__ gid)
@@ -334,9 +341,6 @@ __global__ void __launch_bounds__(kBlock) k_pair_cache(Buffers B, const double *
     __shared__ Phys P;
     __shared__ float4 sh[kCodes];
     if (skip_form(B)) return;            // the step runs the other pair-term form
-    if (blockIdx.x == 0 && B.form_run != 2) {    // (2: a paused loop goes on with the cache)
-        reset_loops(B);
-    }
     // tiles of SPB slots, grid-stride (a launch with one block per tile takes
     // one each; a launch in a graph that may skip it takes one wave of blocks,
     // so that skipping costs little)
@@ -510,8 +514,7 @@ int launch_pair_cache_pass(const Buffers &B, const double *xpos, const uint32_t 
 
 int launch_shift(const Buffers &B, cudaStream_t st)
 {
-    int k = launch_binning(B, B.x_a, B.gid_a, st);            // cells at r^{n+1}
-    k += launch_permute_a_to_b(B, st);
+    const int k = launch_bin_a_to_b(B, st);                   // cells at r^{n+1}
     launch_nlist(B, B.x_b, st);
     DTSPH_DISPATCH(B.dim, B.fp32c, (k_shift<D, F32><<<(B.n + kBlock - 1) / kBlock, kBlock, 0, st>>>(B)));
     return k + 2;
