@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(kResThreads<F32> + kDecide, 1) k_loop_res(Buff
             }
             __syncthreads();
             if (stop) break;
-            if (!grid_barrier(&B.ctrl->bar, ++epoch, B.err, ok_sh, B.barrier_ns)) break;
+            if (!grid_barrier<true>(&B.ctrl->bar, ++epoch, B.err, ok_sh, B.barrier_ns)) break;
         }
         T apT = T(0), FT[3] = {T(0), T(0), T(0)};
         if (worker) {
@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(kResThreads<F32> + kDecide, 1) k_loop_res(Buff
                 g[1] = w_av;
             }
         }
-        if (!grid_barrier(&B.ctrl->bar, ++epoch, B.err, ok_sh, B.barrier_ns)) break;
+        if (!grid_barrier<true>(&B.ctrl->bar, ++epoch, B.err, ok_sh, B.barrier_ns)) break;
     }
     // `it` iterations are done (a barrier that gave up: the step is reported)
     if (fl)

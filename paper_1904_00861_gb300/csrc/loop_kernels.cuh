@@ -230,7 +230,7 @@ using Real = typename std::conditional<F32, float, double>::type;
 // The shift table of the uncached FP32C form and the geometry of the uncached
 // FP64 form, per block.
 struct FormGeom {
-    float4 sh[kCodes];
+    ShiftTable sh;
     Geom G;
 };
 
@@ -239,7 +239,7 @@ template <bool F32, bool FA>
 __device__ __forceinline__ void load_form_geom(const Buffers &B, int inst, FormGeom &fg)
 {
     if constexpr (FA && F32) {
-        if (threadIdx.x < kCodes) fg.sh[threadIdx.x] = code_shift(B.geo[inst], threadIdx.x);
+        load_shifts(fg.sh, B.geo[inst]);
     } else if constexpr (FA) {
         for (int w = threadIdx.x; w < (int)(sizeof(Geom) / 4); w += blockDim.x)
             reinterpret_cast<int *>(&fg.G)[w] = reinterpret_cast<const int *>(B.geo + inst)[w];
@@ -672,7 +672,7 @@ __device__ __forceinline__ void tile_iteration(const Buffers &B, const Phys &P, 
 // applies its stop rules; the last block of all sets the while-node condition
 // (some instance still iterating).
 template <int D, bool F32, bool WALLS, int L, bool FA = false>
-__global__ void __launch_bounds__(kBlock, F32 ? (L == 1 && !FA && D == 3 ? 2 : 3) : 1)
+__global__ void __launch_bounds__(kBlock, F32 ? (D == 3 && (L == 1 || FA) ? 2 : 3) : 1)
     k_iterate(Buffers B, unsigned long long cond, int use_cond)
 {
     using T = typename std::conditional<F32, float, double>::type;
@@ -743,11 +743,14 @@ __device__ __forceinline__ unsigned long long global_ns()
 
 // Grid barrier for a cooperative launch (all blocks resident): arrival counter
 // `bar`, reset to 0 before the launch; the epoch-th barrier waits for
-// epoch * gridDim.x arrivals: a release arrival of the block's writes, acquire
-// polls. The wait gives up after limit_ns (one second unless a test shortens it),
+// epoch * gridDim.x arrivals: a release arrival of the block's writes, then polls.
+// ALONE (one block per SM): acquire polls, the shortest way. Else relaxed polls and
+// one acquire fence, since every acquire would empty the L1 under the SM's other
+// blocks. The wait gives up after limit_ns (one second unless a test shortens it),
 // raises kErrBarrier and returns false (the caller then stops iterating).
-__device__ bool grid_barrier(unsigned int *bar, unsigned int epoch, uint32_t *err, int &ok_sh,
-                             unsigned long long limit_ns)
+template <bool ALONE>
+__device__ __forceinline__ bool grid_barrier(unsigned int *bar, unsigned int epoch, uint32_t *err, int &ok_sh,
+                                             unsigned long long limit_ns)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -757,7 +760,8 @@ __device__ bool grid_barrier(unsigned int *bar, unsigned int epoch, uint32_t *er
         unsigned long long t0 = 0;
         for (;;) {
             unsigned int v;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            if (ALONE) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            else asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
             if (v >= target) break;
             // (the clock every 64 polls: reading it costs more than a poll)
             if (limit_ns == 0 || (++polls & 63) == 0) {
@@ -770,6 +774,7 @@ __device__ bool grid_barrier(unsigned int *bar, unsigned int epoch, uint32_t *er
                 }
             }
         }
+        if (!ALONE) asm volatile("fence.acq_rel.gpu;" ::: "memory");
         ok_sh = ok;
     }
     __syncthreads();
@@ -846,7 +851,7 @@ __device__ __forceinline__ int dealt_instance(const int *pre, int ni, int k)
 // decisions; tiles of finished instances are skipped. Walls get their own phase
 // and barrier before the fluid phase.
 template <int D, bool F32, bool WALLS, int L, bool FA = false>
-__global__ void __launch_bounds__(kBlock, F32 ? (L == 1 && !FA && D == 3 ? 2 : 3) : L == 1 && !FA ? 3 : 2)
+__global__ void __launch_bounds__(kBlock, F32 ? (D == 3 && (L == 1 || FA) ? 2 : 3) : L == 1 && !FA ? 3 : 2)
     k_loop(Buffers B)
 {
     using T = typename std::conditional<F32, float, double>::type;
@@ -889,7 +894,7 @@ __global__ void __launch_bounds__(kBlock, F32 ? (L == 1 && !FA && D == 3 ? 2 : 3
                 // (one instance: it is iterating, no need to look)
                 if (single || !B.ls[B.inst_of[s]].done) wall_slot<D, F32>(B, s, cur, sub, gmask);
             }
-            if (!grid_barrier(&B.ctrl->bar, ++epoch, B.err, ok_sh, B.barrier_ns)) break;
+            if (!grid_barrier<false>(&B.ctrl->bar, ++epoch, B.err, ok_sh, B.barrier_ns)) break;
         }
         double *blk = B.blk + (size_t)(it & 1) * 2 * ntiles;
         int nwork = ntiles;
@@ -924,7 +929,7 @@ __global__ void __launch_bounds__(kBlock, F32 ? (L == 1 && !FA && D == 3 ? 2 : 3
                 blk[2 * t + 1] = b;
             }
         }
-        if (!grid_barrier(&B.ctrl->bar, ++epoch, B.err, ok_sh, B.barrier_ns)) break;
+        if (!grid_barrier<false>(&B.ctrl->bar, ++epoch, B.err, ok_sh, B.barrier_ns)) break;
         if (single) {
             double sa = 0, sb = 0;
             int tlo, thi;
@@ -953,7 +958,7 @@ __global__ void __launch_bounds__(kBlock, F32 ? (L == 1 && !FA && D == 3 ? 2 : 3
                 }
                 __syncthreads();
             }
-            if (!grid_barrier(&B.ctrl->bar, ++epoch, B.err, ok_sh, B.barrier_ns)) break;
+            if (!grid_barrier<false>(&B.ctrl->bar, ++epoch, B.err, ok_sh, B.barrier_ns)) break;
             if (threadIdx.x == 0) stop = *(volatile int *)&B.ctrl->active == 0;
             __syncthreads();
             if (stop) break;
@@ -1008,7 +1013,7 @@ __device__ __forceinline__ int block_min(int v, int *scratch)
 // tile and every decision is computed as in k_loop, so the results are the
 // same bits.
 template <int D, bool F32, int L, bool FA = false>
-__global__ void __launch_bounds__(kBlock, F32 ? (L == 1 && !FA && D == 3 ? 2 : 3) : L == 1 && !FA ? 3 : 2)
+__global__ void __launch_bounds__(kBlock, F32 ? (D == 3 && (L == 1 || FA) ? 2 : 3) : L == 1 && !FA ? 3 : 2)
     k_loop_async(Buffers B)
 {
     using T = typename std::conditional<F32, float, double>::type;

@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(kBlock) k_move_iter(Buffers B, unsigned long l
     using T = typename std::conditional<F32, float, double>::type;
     __shared__ Geom G;
     __shared__ Phys P;
-    __shared__ float4 sh[kCodes];
+    __shared__ ShiftTable sh;
     __shared__ double red[2][kBlock / kWarp];
     __shared__ int last, tlo_sh;
     if (!use_cond && B.ctrl->active == 0) return;   // whole grid agrees: nothing to do
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(kBlock) k_move_iter(Buffers B, unsigned long l
     const int it = ls->iter;
     const bool work = mine && !ls->done;
     if (work) {
-        if (F32 && threadIdx.x < kCodes) sh[threadIdx.x] = code_shift(B.geo[inst], threadIdx.x);
+        if (F32) load_shifts(sh, B.geo[inst]);
         block_copy(G, B.geo[inst]);
         block_copy(P, B.phys[inst]);
         const int cur = it & 1, nxt = cur ^ 1;

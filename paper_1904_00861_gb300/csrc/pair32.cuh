@@ -74,18 +74,15 @@ struct Sums32 {
 };
 
 // g = w r_ij / r and F = w r / (r^2 + eta h^2) of two neighbours, w the quintic
-// spline's dW/dq without sigma (0 from q = 3 on). r^2 is kept above 0, so that
-// r = 0 gives d = 0 times a finite factor and w(0) = 0: zeros.
+// spline's dW/dq without sigma (0 from q = 3 on). 1e-37 beside r^2 leaves it as it
+// is but for r = 0, where d = 0 times a finite factor and w(0) = 0 give zeros.
 template <int D>
 __device__ __forceinline__ void grad2(const PairK32 &k, const F2 *d, F2 *g, F2 &F)
 {
-    F2 r2 = fma2(d[1], d[1], mul2(d[0], d[0]));
+    F2 r2 = fma2(d[1], d[1], fma2(d[0], d[0], both(1e-37f)));
     if (D == 3) r2 = fma2(d[2], d[2], r2);
     float ra, rb;
     unpack2(r2, ra, rb);
-    ra = fmaxf(ra, 1e-37f);
-    rb = fmaxf(rb, 1e-37f);
-    r2 = pack2(ra, rb);
     const F2 rinv = pack2(rsqrt_fast(ra), rsqrt_fast(rb));
     const F2 r = mul2(r2, rinv);
     const F2 q = mul2(r, both(k.inv_h));
@@ -206,29 +203,39 @@ __device__ __forceinline__ void rates32(const PairK32 &k, const Sums32<D> &A, fl
     for (int a = 0; a < D; ++a) F[a] = __fmul_rn(k.s_F, merged32<L>(A.F[a]));
 }
 
-// Displacement of the home offset for every shift code: o_i moves by minus the
-// cell shift (a particle's own code, 13, by zero).
-__device__ __forceinline__ float4 code_shift(const Geom &G, int code)
+// Displacement of the home offset for every shift code, by component, in shared
+// memory: o_i moves by minus the cell shift (a particle's own code, 13, by zero). The
+// codes of a warp's entries differ, and 32 words by component lie in 32 banks: one
+// wavefront a component (records of 16 bytes: the 128^3 loop without the cache 1.23
+// ms an iteration, so 1.20 ms).
+constexpr int kCodes = 32;
+struct ShiftTable {
+    float c[3][kCodes];
+};
+__device__ __forceinline__ void load_shifts(ShiftTable &sh, const Geom &G)     // (whole block; sync after)
 {
+    const int code = threadIdx.x;
+    if (code >= kCodes) return;
     int dx, dy, dz;
-    decode_shift(code, dx, dy, dz);
-    return make_float4(-(float)dx * G.s_f[0], -(float)dy * G.s_f[1], -(float)dz * G.s_f[2], 0.f);
+    decode_shift(code < 27 ? code : 13, dx, dy, dz);
+    sh.c[0][code] = -(float)dx * G.s_f[0];
+    sh.c[1][code] = -(float)dy * G.s_f[1];
+    sh.c[2][code] = -(float)dz * G.s_f[2];
 }
-constexpr int kCodes = 27;
 
 // r_ij of list entry e: (o_i - shift) - o_j.
 template <int D>
-__device__ __forceinline__ void entry_sep(const float4 *sh, float4 oi, float4 oj, uint32_t e, float *d)
+__device__ __forceinline__ void entry_sep(const ShiftTable &sh, float4 oi, float4 oj, uint32_t e, float *d)
 {
-    const float4 t = sh[entry_code(e)];
-    d[0] = __fsub_rn(__fadd_rn(oi.x, t.x), oj.x);
-    d[1] = __fsub_rn(__fadd_rn(oi.y, t.y), oj.y);
-    if (D == 3) d[2] = __fsub_rn(__fadd_rn(oi.z, t.z), oj.z);
+    const int t = entry_code(e);
+    d[0] = __fsub_rn(__fadd_rn(oi.x, sh.c[0][t]), oj.x);
+    d[1] = __fsub_rn(__fadd_rn(oi.y, sh.c[1][t]), oj.y);
+    if (D == 3) d[2] = __fsub_rn(__fadd_rn(oi.z, sh.c[2][t]), oj.z);
 }
 
 // g and F of list entries ea, eb with the neighbours' offsets oa, ob.
 template <int D>
-__device__ __forceinline__ void entry_grad2(const PairK32 &k, const float4 *sh, float4 oi, float4 oa, float4 ob,
+__device__ __forceinline__ void entry_grad2(const PairK32 &k, const ShiftTable &sh, float4 oi, float4 oa, float4 ob,
                                             uint32_t ea, uint32_t eb, F2 *g, F2 &F)
 {
     float da[3], db[3];
@@ -247,7 +254,7 @@ __host__ __device__ __forceinline__ int list_pairs(int cnt) { return (cnt + 3) /
 // lane_in, lane_in + L, ..., two in flight): offsets off, states nb, geometry
 // recomputed. wall(entry, w) gives a neighbour's divergence-term velocity (WALLS).
 template <int D, bool WALLS, int L, typename WV, typename M>
-__device__ __forceinline__ void list_sums32(const PairK32 &k, const float4 *sh, const uint32_t *__restrict__ lst,
+__device__ __forceinline__ void list_sums32(const PairK32 &k, const ShiftTable &sh, const uint32_t *__restrict__ lst,
                                             int cnt, int lane_in, float4 oi, const float *vi, float pi,
                                             const float4 *off, const float4 *nb, WV wall, Sums32<D> &A, M &mv)
 {
@@ -278,6 +285,42 @@ __device__ __forceinline__ void list_sums32(const PairK32 &k, const float4 *sh, 
             F2 g[D], F;
             entry_grad2<D>(k, sh, oi, o[r], o[r + 1], e[r], e[r + 1], g, F);
             pair2_accumulate<D, WALLS>(k, g, F, vi, pi, q[r], q[r + 1], w[r], w[r + 1], A, mv);
+        }
+    }
+}
+
+// The rates of a warp's 32 slots (s: the lane's own, cnt its list's length, 0 if it
+// has no rates to form), G lanes to a slot: the warp takes 32 / G slots at a time,
+// so that a gather's 32 entries are G neighbours in a row of each of them and fall
+// on fewer lines: the L1 looks up one line a cycle, and one lane per slot puts
+// the entries of a 3D gather on 17 lines, eight lanes on 10 (2D: 8.5, four lanes
+// 5). A slot's sums then come back to its own lane. sums(slot, lane of the slot,
+// count, V_i, p_i, A) adds the pairs.
+template <int D, int G, typename SUMS>
+__device__ __forceinline__ void warp_rates32(const PairK32 &k, int s, int cnt, const float4 *nb, SUMS sums, float &ap,
+                                             float *F)
+{
+    constexpr int P = kWarp / G;                         // slots at a time
+    const int lane = threadIdx.x & (kWarp - 1), s0 = s - lane;
+    ap = 0.f;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) F[a] = 0.f;
+#pragma unroll 1
+    for (int g = 0; g < G; ++g) {
+        const int from = g * P + lane / G;               // the slot this lane works on
+        const int c = __shfl_sync(0xffffffffu, cnt, from), sg = s0 + from;
+        const float4 qi = c > 0 ? nb[sg] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float vi[3] = {qi.x, qi.y, qi.z};
+        Sums32<D> A;
+        sums(sg, lane % G, c, vi, qi.w, A);
+        float r[D + 1];
+        rates32<D, G>(k, A, r[0], r + 1);
+        const int src = (lane - g * P) * G & (kWarp - 1);
+        const bool mine = lane / P == g;
+#pragma unroll
+        for (int a = 0; a <= D; ++a) {
+            const float v = __shfl_sync(0xffffffffu, r[a], src);
+            if (mine) (a == 0 ? ap : F[a - 1]) = v;
         }
     }
 }

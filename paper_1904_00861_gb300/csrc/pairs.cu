@@ -20,14 +20,21 @@ namespace {
 // takes the list entries (FP32C: pairs of entries) l, l + L, ... Summing kernels
 // merge the lanes' partial sums by shuffles, so their summation order depends on L
 // alone: they use a fixed L per path, which keeps every context (solo or batched,
-// any size) on the same order. FP32C: one lane per slot measured fastest on large
-// problems and costs little on small ones. FP64: eight, a small problem's chain of
+// any size) on the same order. FP32C: one lane per slot, the warp sharing the slots'
+// lists inside (kStateLanes). FP64: eight, a small problem's chain of
 // pairs being what its pass takes (1,024 2D particles: 139 us with one lane, 14 us
 // now, the factored sums included), at no cost to large ones, which the FP64
 // pipe bounds. Block b covers slots b * (kBlock / L) ...
 
 template <bool F32>
 constexpr int kSumLanes = F32 ? 1 : 8;
+// Lanes a slot within the warp in the FP32C state-n pass (warp_rates32). 128^3: one
+// lane 1.1 ms a pass, eight 0.78 ms; in 2D four take 1% off a step of the 64-vortex
+// batch and of the 200 x 200 vortex. (In the loops, whose iterations find the
+// states in no L1, lanes sharing a warp's slots measured slower: 128^3 without the
+// cache 1.23 ms an iteration at one lane, 1.48 at eight.)
+template <int D>
+constexpr int kStateLanes = D == 3 ? 8 : 4;
 
 // Adami et al. wall values at state n in order B: p_w = (sum_f p_f W + rho0 g .
 // sum_f r_wf W) / sum_f W, ghost velocity 2 v_w - sum_f V_f W / sum_f W; written
@@ -103,9 +110,9 @@ __global__ void __launch_bounds__(kBlock, F32 ? (D == 2 ? 4 : 3) : 1) k_state_n(
     constexpr int SPB = kBlock / L;
     __shared__ Geom G;
     __shared__ Phys P;
-    __shared__ float4 sh[kCodes];
+    __shared__ ShiftTable sh;
     const int inst = block_instance(B, blockIdx.x * SPB);
-    if (F32 && threadIdx.x < kCodes) sh[threadIdx.x] = code_shift(B.geo[inst], threadIdx.x);
+    if (F32) load_shifts(sh, B.geo[inst]);
     block_copy(G, B.geo[inst]);
     block_copy(P, B.phys[inst]);
     const int n = B.n;
@@ -117,20 +124,23 @@ __global__ void __launch_bounds__(kBlock, F32 ? (D == 2 ? 4 : 3) : 1) k_state_n(
     const int cnt = fluid ? B.pcount[s] : 0;
     const uint32_t *lst = slot_list(B, s);
     if constexpr (F32) {
+        static_assert(L == 1, "a warp's lanes and slots one to one");
         const PairK32 k = P.k32;
         const float4 *nb = B.nb32[1];
-        const float4 qi = fluid ? nb[s] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float4 oi = fluid ? B.off[s] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float vi[3] = {qi.x, qi.y, qi.z};
         auto wall = [&](uint32_t e, const float4 &q, float *w) {
             w[0] = q.x; w[1] = q.y; w[2] = q.z;
             if (e & kWallBit)
                 for (int a = 0; a < D; ++a) w[a] = (float)B.vn_b[(size_t)a * n + entry_slot(e)];
         };
-        Sums32<D> A;
-        NoMove mv;
-        list_sums32<D, WALLS, L>(k, sh, lst, cnt, lane_in, oi, vi, qi.w, B.off, nb, wall, A, mv);
-        rates32<D, L>(k, A, apT, FT);
+        constexpr int G = kStateLanes<D>;
+        warp_rates32<D, G>(
+            k, s, cnt, nb,
+            [&](int sg, int sub, int c, const float *vi, float pi, Sums32<D> &A) {
+                const float4 oi = c > 0 ? B.off[sg] : make_float4(0.f, 0.f, 0.f, 0.f);
+                NoMove mv;
+                list_sums32<D, WALLS, G>(k, sh, slot_list(B, sg), c, sub, oi, vi, pi, B.off, nb, wall, A, mv);
+            },
+            apT, FT);
     } else {
         const double4_32a *nb = B.nb64[1];
         const PairConst<double> k = pair_const<double>(P);
@@ -223,7 +233,7 @@ __global__ void __launch_bounds__(kBlock, F32 ? (D == 2 ? 4 : 3) : 1) k_state_n(
 // threadIdx.x % L of the slot's group takes the pairs of entries lane, lane + L, ...,
 // two in flight.
 template <int D, int L>
-__device__ __forceinline__ void pair_cache_slot32(const Buffers &B, const Phys &P, const float4 *sh,
+__device__ __forceinline__ void pair_cache_slot32(const Buffers &B, const Phys &P, const ShiftTable &sh,
                                                   const uint32_t *__restrict__ gid, int s)
 {
     const PairK32 k = P.k32;
@@ -339,7 +349,7 @@ __global__ void __launch_bounds__(kBlock) k_pair_cache(Buffers B, const double *
     constexpr int SPB = kBlock / L;
     __shared__ Geom G;
     __shared__ Phys P;
-    __shared__ float4 sh[kCodes];
+    __shared__ ShiftTable sh;
     if (skip_form(B)) return;            // the step runs the other pair-term form
     // tiles of SPB slots, grid-stride (a launch with one block per tile takes
     // one each; a launch in a graph that may skip it takes one wave of blocks,
@@ -350,7 +360,7 @@ __global__ void __launch_bounds__(kBlock) k_pair_cache(Buffers B, const double *
         const int inst = block_instance(B, bt * SPB);
         if (inst != p_inst) {
             __syncthreads();                 // the previous tile is done with G and P
-            if (F32 && threadIdx.x < kCodes) sh[threadIdx.x] = code_shift(B.geo[inst], threadIdx.x);
+            if (F32) load_shifts(sh, B.geo[inst]);
             block_copy(G, B.geo[inst]);
             block_copy(P, B.phys[inst]);
             p_inst = inst;
