@@ -134,8 +134,8 @@ typedef struct {
                                  1: over the neighbour lists of r^0; 2: neighbours updated at
                                  every pass (lists with the cutoff 3h + skin; a particle that
                                  moves farther than skin/2 from r^0 ends the step with
-                                 DTSPH_E_SKIN). Not with steady. With graph = 2 the loop runs
-                                 as in graph = 1. Instances of a batch share it. */
+                                 DTSPH_E_SKIN). Not with steady. With graph = 2 a batch runs the
+                                 loop as in graph = 1. Instances of a batch share it. */
     int32_t form;             /* the pair terms of the pseudo-time loop. 1: from the pair-
                                  coefficient cache, written once per real step by a pass over
                                  the lists at r^0 (gradW_ij and F_ij per pair). 2: recomputed

@@ -584,9 +584,12 @@ int allocate(dtsph_ctx *c, const int64_t *nf)
     }
     if (c->prm[0].moving && !c->prm[0].steady) {
         // the moving pass: the lanes asked for, else one lane per particle on
-        // the FP32C path (measured fastest: more lanes add blocks beyond the
-        // resident set and redundant per-lane state loads) and up to four on the
-        // FP64 path (FP64-pipe-bound: more threads help while there are few)
+        // the FP32C path, whatever the size, so that an instance of a batch has the
+        // bits of its solo run (iteration of 151 x 151 particles 16.8 / 17.0 / 21.4
+        // us at 1 / 2 / 4 lanes, of 250 x 250 25 / 30 / 40 us; small problems gain
+        // from more, 90 x 90 16.6 / 12.6 / 10.9 us, and can ask for them), and up
+        // to four on the FP64 path (FP64-pipe-bound: more threads help while there
+        // are few; 90 x 90 152 / 82 / 48 us, 151 x 151 152 / 159 / 137 us)
         int L = c->prm[0].lanes;
         if (L == 0) {
             L = 1;
@@ -859,9 +862,8 @@ bool auto_form(const dtsph_ctx *c)
 // Graph of one real step: pre-loop kernels -> while node (walls, iterate) -> outer.
 int build_graph(dtsph_ctx *c)
 {
-    // the persistent loop kernel runs the frozen pass only; moving runs take the
-    // while node
-    if (c->prm[0].graph == 2 && !c->B.xk[0]) {
+    // batches of moving particles take the while node
+    if (c->prm[0].graph == 2 && (!c->B.xk[0] || c->ninst == 1)) {
         // the kernels take Buffers by value: the words of the per-step form
         // choice are set in the graph's copies only
         c->form_graph = auto_form(c) && c->kstar >= 0.0;

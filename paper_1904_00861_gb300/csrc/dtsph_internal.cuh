@@ -324,6 +324,8 @@ int launch_move_prepare(const Buffers &B, cudaStream_t st);
 // pair pass with the advective terms, the update of V, V~, r and p-hat, and the
 // stop rules (sets the while-node condition when use_cond).
 int launch_move_iteration(const Buffers &B, unsigned long long cond_handle, int use_cond, cudaStream_t st);
+// The persistent loop kernel of one instance with moving particles.
+const void *move_loop_function(const Buffers &B);
 // Particle shifting of the fluid after the real step: bins at r^{n+1}, gathers
 // the state into order B, builds the lists, and shifts (results written back to
 // order A).

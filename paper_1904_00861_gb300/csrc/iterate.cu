@@ -66,7 +66,7 @@ static const void *loop_lanes(int lanes)
 // Dynamic shared memory of the iterate and loop kernels of this shape.
 static size_t iterate_smem(const Buffers &B)
 {
-    if (B.lanes != 1 || B.form_a) return 0;              // the ring holds cache rows only
+    if (B.lanes != 1 || B.form_a || B.xk[0]) return 0;              // the ring holds cache rows only
     return B.fp32c ? ring_bytes<true>(B.stages) : ring_bytes<false>(B.stages);
 }
 
@@ -97,6 +97,7 @@ static const void *async_lanes(int lanes)
 
 static const void *loop_function(const Buffers &B)
 {
+    if (B.xk[0]) return move_loop_function(B);
     if (B.form_a) return loop_function_fa(B);
     if (B.async_loop) {
         if (B.dim == 2) return B.fp32c ? async_lanes<2, true>(B.lanes) : async_lanes<2, false>(B.lanes);

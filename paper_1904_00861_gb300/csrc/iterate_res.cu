@@ -392,7 +392,7 @@ constexpr size_t kResSmem = 232448 - 10 * 1024;
 
 bool resident_shape(const Buffers &B, ResShape *S)
 {
-    if (B.ninst != 1 || B.form_a || B.nsm < 1) return false;
+    if (B.ninst != 1 || B.form_a || B.xk[0] || B.nsm < 1) return false;
     const int groups = B.n / kWarp;
     const int q = (groups + B.nsm - 1) / B.nsm * kWarp;
     if (q * B.lanes > (B.fp32c ? kResThreads<true> : kResThreads<false>) || B.n / (kBlock / B.lanes) > kResTiles) return false;

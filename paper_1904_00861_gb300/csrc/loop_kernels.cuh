@@ -33,6 +33,7 @@
 
 #include "bulk.cuh"
 #include "geometry.cuh"
+#include "grid_barrier.cuh"
 #include "loop_rules.cuh"
 #include "pair32.cuh"
 #include "pair64.cuh"
@@ -734,53 +735,6 @@ __global__ void __launch_bounds__(kBlock, F32 ? (D == 3 && (L == 1 || FA) ? 2 : 
     }
 }
 
-__device__ __forceinline__ unsigned long long global_ns()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// Grid barrier for a cooperative launch (all blocks resident): arrival counter
-// `bar`, reset to 0 before the launch; the epoch-th barrier waits for
-// epoch * gridDim.x arrivals: a release arrival of the block's writes, then polls.
-// ALONE (one block per SM): acquire polls, the shortest way. Else relaxed polls and
-// one acquire fence, since every acquire would empty the L1 under the SM's other
-// blocks. The wait gives up after limit_ns (one second unless a test shortens it),
-// raises kErrBarrier and returns false (the caller then stops iterating).
-template <bool ALONE>
-__device__ __forceinline__ bool grid_barrier(unsigned int *bar, unsigned int epoch, uint32_t *err, int &ok_sh,
-                                             unsigned long long limit_ns)
-{
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const unsigned int target = epoch * gridDim.x;
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-        int ok = 1, polls = 0;
-        unsigned long long t0 = 0;
-        for (;;) {
-            unsigned int v;
-            if (ALONE) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-            else asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-            if (v >= target) break;
-            // (the clock every 64 polls: reading it costs more than a poll)
-            if (limit_ns == 0 || (++polls & 63) == 0) {
-                const unsigned long long now = global_ns();
-                if (t0 == 0) t0 = now;
-                if (limit_ns == 0 || now - t0 > limit_ns) {
-                    atomicOr(err, kErrBarrier);
-                    ok = 0;
-                    break;
-                }
-            }
-        }
-        if (!ALONE) asm volatile("fence.acq_rel.gpu;" ::: "memory");
-        ok_sh = ok;
-    }
-    __syncthreads();
-    return ok_sh != 0;
-}
-
 // Exclusive prefix of the active (not yet converged) tiles of every instance,
 // by the whole block: pre[i] = active tiles of instances 0 .. i-1, pre[ninst] =
 // all of them. Reads the instances' done flags, so call it after the barrier
@@ -1071,7 +1025,7 @@ __global__ void __launch_bounds__(kBlock, F32 ? (D == 3 && (L == 1 || FA) ? 2 : 
             if (w_inst >= 0) {
                 waiting = false;
             } else if (!quit) {
-                const unsigned long long now = global_ns();
+                const unsigned long long now = globaltimer_ns();
                 if (!waiting) {
                     waiting = true;
                     wait_from = now;
