@@ -17,9 +17,9 @@ namespace {
 
 // Cell (global index) of every particle of the source order; -1 for padding. (The
 // keys at r^0 are counted by the state-n pass that predicts the positions.)
-__global__ void __launch_bounds__(kBlock) k_bin_keys(Buffers B, const double *__restrict__ x,
-                                                     const uint32_t *__restrict__ gid)
+__global__ void __launch_bounds__(kBlock) k_bin_keys(Buffers B, const double *x, const uint32_t *gid)
 {
+    grid_start<true>();
     if (skip_relist(B)) return;   // (the step graph: relisting or not)
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= B.n) return;
@@ -75,6 +75,7 @@ __device__ __forceinline__ int block_exclusive_scan(int v)
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_partial(Buffers B)
 {
+    grid_start<true>();
     if (skip_relist(B)) return;   // (the step graph: relisting or not)
     const int base = blockIdx.x * kScanCells + threadIdx.x * kScanPerThread;
     int s = 0;
@@ -96,6 +97,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_partial(Buffers B)
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_top(Buffers B, int nblocks)
 {
+    grid_start<true>();
     if (skip_relist(B)) return;   // (the step graph: relisting or not)
     // exclusive prefix of the block totals, in chunks of the block width
     int carry = 0;
@@ -133,6 +135,7 @@ __device__ __forceinline__ int cell_instance(const Buffers &B, int c)
 template <int PER, bool MULTI>
 __global__ void __launch_bounds__(kScanThreads) k_scan_final(Buffers B)
 {
+    grid_start<true>();
     if (skip_relist(B)) return;   // (the step graph: relisting or not)
     static_assert(PER % 4 == 0, "whole pieces");
     const int base = (blockIdx.x * kScanThreads + threadIdx.x) * PER;
@@ -187,6 +190,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_final(Buffers B)
 
 __global__ void __launch_bounds__(kBlock) k_scatter(Buffers B)
 {
+    grid_start<true>();
     if (skip_relist(B)) return;   // (the step graph: relisting or not)
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= B.n) return;
@@ -322,6 +326,7 @@ __device__ __forceinline__ void move_b_to_a(const Buffers &B, int o, int s, int 
 template <bool TO_A>
 __global__ void __launch_bounds__(kBlock) k_rank_move(Buffers B)
 {
+    grid_start<true>();
     if (skip_relist(B)) return;   // (the step graph: relisting or not)
     if constexpr (TO_A) {
         if (blockIdx.x == 0) {
@@ -425,6 +430,7 @@ __global__ void __launch_bounds__(kBlock) k_begin_one(Buffers B, Inst I, Geom G,
                                                       const double *__restrict__ v, const double *__restrict__ p,
                                                       const double *__restrict__ xw, const double *__restrict__ vw)
 {
+    grid_start<true>();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t == 0) {
         *const_cast<Inst *>(B.inst) = I;
@@ -443,6 +449,7 @@ __global__ void __launch_bounds__(kBlock) k_begin_one(Buffers B, Inst I, Geom G,
 __global__ void __launch_bounds__(kBlock) k_rates_out(Buffers B, double *__restrict__ ap, double *__restrict__ F,
                                                       int32_t *status)
 {
+    grid_start<false>();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s == 0 && status) {
         const uint32_t e = *B.err;
@@ -477,30 +484,30 @@ static int launch_sort(const Buffers &B, cudaStream_t st)
     // totals, their scan, and the block scans with their carries
     int k = 2;
     if (B.ncell <= kScanCells1) {
-        k_scan_final<kScanPerThread1, false><<<1, kScanThreads, 0, st>>>(B);
+        launch_next(B, st, 1, kScanThreads, k_scan_final<kScanPerThread1, false>, B);
     } else {
         const int nsb = (B.ncell + kScanCells - 1) / kScanCells;
-        k_scan_partial<<<nsb, kScanThreads, 0, st>>>(B);
-        k_scan_top<<<1, kScanThreads, 0, st>>>(B, nsb);
-        k_scan_final<kScanPerThread, true><<<nsb, kScanThreads, 0, st>>>(B);
+        launch_next(B, st, nsb, kScanThreads, k_scan_partial, B);
+        launch_next(B, st, 1, kScanThreads, k_scan_top, B, nsb);
+        launch_next(B, st, nsb, kScanThreads, k_scan_final<kScanPerThread, true>, B);
         k += 2;
     }
-    k_scatter<<<blocks(B.n), kBlock, 0, st>>>(B);
+    launch_next(B, st, blocks(B.n), kBlock, k_scatter, B);
     return k;
 }
 
 int launch_bin_a_to_b(const Buffers &B, cudaStream_t st)
 {
-    k_bin_keys<<<blocks(B.n), kBlock, 0, st>>>(B, B.x_a, B.gid_a);
+    launch_next(B, st, blocks(B.n), kBlock, k_bin_keys, B, B.x_a, B.gid_a);
     const int k = launch_sort(B, st);
-    k_rank_move<false><<<blocks(B.n), kBlock, 0, st>>>(B);
+    launch_next(B, st, blocks(B.n), kBlock, k_rank_move<false>, B);
     return k + 2;
 }
 
 int launch_bin_b_to_a(const Buffers &B, cudaStream_t st)
 {
     const int k = launch_sort(B, st);                    // (the predictor counted the keys)
-    k_rank_move<true><<<blocks(B.n), kBlock, 0, st>>>(B);
+    launch_next(B, st, blocks(B.n), kBlock, k_rank_move<true>, B);
     return k + 1;
 }
 
@@ -519,7 +526,7 @@ int launch_begin_one(const Buffers &B, const Inst &I, const Geom &G, const Phys 
 
 int launch_rates_out(const Buffers &B, double *ap, double *F, int32_t *status, cudaStream_t st)
 {
-    k_rates_out<<<blocks(B.n), kBlock, 0, st>>>(B, ap, F, status);
+    launch_next(B, st, blocks(B.n), kBlock, k_rates_out, B, ap, F, status);
     return 1;
 }
 

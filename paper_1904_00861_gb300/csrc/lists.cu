@@ -59,6 +59,7 @@ __device__ __forceinline__ int cell_instance(const Buffers &B, int c)
 __global__ void __launch_bounds__(kBlock) k_nlist_cells2(Buffers B, const double *__restrict__ xpos,
                                                          uint32_t *__restrict__ lists, int Ks)
 {
+    grid_start<false>();
     if (skip_relist(B)) return;   // (the step graph: relisting or not)
     constexpr int NC = 9;                               // surrounding cells
     constexpr int CH = 256;                             // staged candidates per round
@@ -271,6 +272,7 @@ template <int D>
 __global__ void __launch_bounds__(kListWarps * kWarp) k_nlist_home(Buffers B, const double *__restrict__ xpos,
                                                                    uint32_t *__restrict__ lists, int Ks)
 {
+    grid_start<false>();
     if (skip_relist(B)) return;   // (the step graph: relisting or not)
     constexpr int SEG = D == 2 ? kSeg2 : 1;
     constexpr int NCOL = SEG + 2;                       // candidate columns
@@ -517,14 +519,14 @@ void launch_nlist(const Buffers &B, const double *xpos, cudaStream_t st)
     const int Ks = list_stride(B.K);
     if (B.dim == 2 && B.nseg2 < kRowsMinSegments) {
         const int nb = (B.ncell + kWarpsPerBlock - 1) / kWarpsPerBlock;
-        k_nlist_cells2<<<nb, kBlock, 0, st>>>(B, xpos, B.pjt, Ks);
+        launch_next(B, st, nb, kBlock, k_nlist_cells2, B, xpos, B.pjt, Ks);
     } else
     if (B.dim == 2) {
         const int nb = (B.nseg2 + kListWarps - 1) / kListWarps;
-        k_nlist_home<2><<<nb, kListWarps * kWarp, 0, st>>>(B, xpos, B.pjt, Ks);
+        launch_next(B, st, nb, kListWarps * kWarp, k_nlist_home<2>, B, xpos, B.pjt, Ks);
     } else {
         const int nb = (B.ncell + kListWarps - 1) / kListWarps;
-        k_nlist_home<3><<<nb, kListWarps * kWarp, 0, st>>>(B, xpos, B.pjt, Ks);
+        launch_next(B, st, nb, kListWarps * kWarp, k_nlist_home<3>, B, xpos, B.pjt, Ks);
     }
 }
 

@@ -38,7 +38,7 @@ __device__ inline int stop_rule(const LoopState &L, int k1)
             // (hi - lo) / hi < stag_tol: by hi - lo against stag_tol hi, 4096 units in
             // the last place apart; nearer, by the quotient
             const double top = __longlong_as_double(hi), d = __dsub_rn(top, __longlong_as_double(lo));
-            const long long gap = __double_as_longlong(d) - __double_as_longlong(__dmul_rn(L.stag_tol, top));
+            const long long gap = __double_as_longlong(d) - __double_as_longlong(__dmul_rn(fabs(L.stag_tol), top));
             stag = gap < -4096 || (gap <= 4096 && d / top < L.stag_tol);
         }
         if (stag) return 1;

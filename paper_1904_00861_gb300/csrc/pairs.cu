@@ -42,6 +42,7 @@ constexpr int kStateLanes = D == 3 ? 8 : 4;
 template <int D, bool F32, int L>
 __global__ void __launch_bounds__(kBlock) k_walls_state_n(Buffers B)
 {
+    grid_start<false>();
     using T = typename std::conditional<F32, float, double>::type;
     constexpr int SPB = kBlock / L;
     __shared__ Geom G;
@@ -106,6 +107,7 @@ __global__ void __launch_bounds__(kBlock) k_walls_state_n(Buffers B)
 template <int D, bool F32, bool PRED, bool WALLS, int L>
 __global__ void __launch_bounds__(kBlock, F32 ? (D == 2 ? 4 : 3) : 1) k_state_n(Buffers B)
 {
+    grid_start<false>();
     using T = typename std::conditional<F32, float, double>::type;
     constexpr int SPB = kBlock / L;
     __shared__ Geom G;
@@ -488,14 +490,14 @@ int launch_state_n(const Buffers &B, bool predictor, cudaStream_t st, bool build
         constexpr int L = kSumLanes<F32>;
         const int nb = (int)(((long long)B.n * L + kBlock - 1) / kBlock);
         if (B.nw > 0) {
-            k_walls_state_n<D, F32, L><<<nb, kBlock, 0, st>>>(B);
+            launch_next(B, st, nb, kBlock, k_walls_state_n<D, F32, L>, B);
             ++k;
-            if (predictor) k_state_n<D, F32, true, true, L><<<nb, kBlock, 0, st>>>(B);
-            else k_state_n<D, F32, false, true, L><<<nb, kBlock, 0, st>>>(B);
+            if (predictor) launch_next(B, st, nb, kBlock, k_state_n<D, F32, true, true, L>, B);
+            else launch_next(B, st, nb, kBlock, k_state_n<D, F32, false, true, L>, B);
         } else if (predictor) {
-            k_state_n<D, F32, true, false, L><<<nb, kBlock, 0, st>>>(B);
+            launch_next(B, st, nb, kBlock, k_state_n<D, F32, true, false, L>, B);
         } else {
-            k_state_n<D, F32, false, false, L><<<nb, kBlock, 0, st>>>(B);
+            launch_next(B, st, nb, kBlock, k_state_n<D, F32, false, false, L>, B);
         }
     });
     return k + 1;
