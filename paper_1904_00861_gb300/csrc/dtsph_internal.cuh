@@ -262,6 +262,7 @@ struct Buffers {
     double kstar;          // the uncached form runs when the latest step took at most kstar iterations
     StatRec *stats;        // [kStatRing][ninst]
     uint32_t *err;
+    int claim_tiles;       // tiles a block of k_loop_async claims at a time
     int chain;             // host: the launches of launch_next overlap (see there)
 };
 

@@ -128,6 +128,10 @@ int loop_grid(const Buffers &B, int *grid)
 cudaError_t launch_loop(const Buffers &B, int grid, cudaStream_t st)
 {
     Buffers b = B;
+    // tiles a claim of k_loop_async takes: two halve its claims and postings, but leave
+    // blocks idle where few tiles are open. Three steps in ms at one and at two (456
+    // blocks): 5,760 tiles 11.4, 10.7; 2,816 4.87, 4.57; 1,440 3.36, 3.68; 960 3.76, 3.82
+    b.claim_tiles = iterate_tiles(B) >= 6 * grid ? 2 : 1;
     const void *fn = nullptr;
     cudaLaunchConfig_t cfg = {};
     ResShape R;

@@ -965,7 +965,10 @@ __device__ __forceinline__ int block_min(int v, int *scratch)
 // from the smallest instances up (they take the most iterations) and waits,
 // bounded by the barrier give-up time, while every open tile is taken. Every
 // tile and every decision is computed as in k_loop, so the results are the
-// same bits.
+// same bits. Claiming and posting are chains of atomics, a quarter of a tile's time
+// (6,200 of 25,800 cycles), so a claim takes two tiles where many are open (64
+// vortices, 5,888 tiles: three steps 13.3 -> 12.8 ms). What is not kept: one warp
+// alone claiming ahead and deciding (15.5 ms; its work stands at the next barrier).
 template <int D, bool F32, int L, bool FA = false>
 __global__ void __launch_bounds__(kBlock, F32 ? (D == 3 && (L == 1 || FA) ? 2 : 3) : L == 1 && !FA ? 3 : 2)
     k_loop_async(Buffers B)
@@ -975,12 +978,15 @@ __global__ void __launch_bounds__(kBlock, F32 ? (D == 3 && (L == 1 || FA) ? 2 : 
     __shared__ TileShared<T, D, L> sh;
     __shared__ Phys P;
     __shared__ FormGeom fg;
-    __shared__ int p_inst, w_inst, w_tile, w_it, last_sh, quit;
+    __shared__ int p_inst, w_inst, w_tile, w_end, w_it, last_sh, more, quit;
     __shared__ int mins[kBlock / kWarp];
     if (skip_form(B)) return;         // the step runs the other pair-term form
     const int ntiles = (B.n + PPB - 1) / PPB;
     const int ni = B.ninst;
-    if (threadIdx.x == 0) p_inst = -1;
+    if (threadIdx.x == 0) {
+        p_inst = -1;
+        more = 0;
+    }
     // (ends with the barrier that publishes thread 0's set-up of the block's
     // shared state, ring or not)
     ring_init<!F32 && L == 1 && !FA>(B.stages);
@@ -988,68 +994,71 @@ __global__ void __launch_bounds__(kBlock, F32 ? (D == 3 && (L == 1 || FA) ? 2 : 
     unsigned long long wait_from = 0;
     bool waiting = false;
     for (;;) {
-        // the first instance in search order with a tile left to hand out
-        int cand = 0x7fffffff;
-        for (int q = threadIdx.x; q < ni; q += kBlock) {
-            const int i = B.sched[q];
-            if (*(volatile int *)&B.ls[i].done) continue;
-            const unsigned long long cl = *(volatile unsigned long long *)&B.il[i].claim;
-            int tlo, thi;
-            instance_tiles(B.inst[i], PPB, tlo, thi);
-            if ((int)(cl & 0xffffffffull) < thi - tlo) {
-                cand = q;
-                break;
-            }
-        }
-        cand = block_min(cand, mins);
-        if (threadIdx.x == 0) {
-            w_inst = -1;
-            quit = 0;
-            if (cand != 0x7fffffff) {
-                const int i = B.sched[cand];
+        if (!more) {   // (else the next of the tiles claimed together)
+            // the first instance in search order with a tile left to hand out
+            int cand = 0x7fffffff;
+            for (int q = threadIdx.x; q < ni; q += kBlock) {
+                const int i = B.sched[q];
+                if (*(volatile int *)&B.ls[i].done) continue;
+                const unsigned long long cl = *(volatile unsigned long long *)&B.il[i].claim;
                 int tlo, thi;
                 instance_tiles(B.inst[i], PPB, tlo, thi);
-                const unsigned long long old = atomicAdd(&B.il[i].claim, 1ull);
-                const int t = (int)(old & 0xffffffffull);
-                if (t < thi - tlo) {
-                    w_inst = i;
-                    w_tile = tlo + t;
-                    w_it = (int)(old >> 32);
-                    __threadfence();
+                if ((int)(cl & 0xffffffffull) < thi - tlo) {
+                    cand = q;
+                    break;
                 }
-            } else if (*(volatile int *)&B.ctrl->active == 0) {
-                quit = 1;
             }
-            // every open tile is taken: wait, bounded, for an iteration to open
-            // (thread 0 alone keeps the clock, so the block decides as one)
-            if (w_inst >= 0) {
-                waiting = false;
-            } else if (!quit) {
-                const unsigned long long now = globaltimer_ns();
-                if (!waiting) {
-                    waiting = true;
-                    wait_from = now;
-                } else if (now - wait_from > B.barrier_ns) {
-                    atomicOr(B.err, kErrBarrier);
+            cand = block_min(cand, mins);
+            if (threadIdx.x == 0) {
+                w_inst = -1;
+                quit = 0;
+                if (cand != 0x7fffffff) {
+                    const int i = B.sched[cand];
+                    int tlo, thi;
+                    instance_tiles(B.inst[i], PPB, tlo, thi);
+                    const unsigned long long old = atomicAdd(&B.il[i].claim, (unsigned long long)B.claim_tiles);
+                    const int t = (int)(old & 0xffffffffull);
+                    if (t < thi - tlo) {
+                        w_inst = i;
+                        w_tile = tlo + t;
+                        w_end = tlo + min(t + B.claim_tiles, thi - tlo);
+                        w_it = (int)(old >> 32);
+                        __threadfence();
+                    }
+                } else if (*(volatile int *)&B.ctrl->active == 0) {
                     quit = 1;
                 }
+                // every open tile is taken: wait, bounded, for an iteration to open
+                // (thread 0 alone keeps the clock, so the block decides as one)
+                if (w_inst >= 0) {
+                    waiting = false;
+                } else if (!quit) {
+                    const unsigned long long now = globaltimer_ns();
+                    if (!waiting) {
+                        waiting = true;
+                        wait_from = now;
+                    } else if (now - wait_from > B.barrier_ns) {
+                        atomicOr(B.err, kErrBarrier);
+                        quit = 1;
+                    }
+                }
+            }
+            __syncthreads();
+            if (quit) break;
+            const int inst = w_inst;
+            if (inst < 0) {
+                __nanosleep(128);
+                continue;
+            }
+            if (inst != p_inst) {
+                for (int w = threadIdx.x; w < (int)(sizeof(Phys) / 4); w += blockDim.x)
+                    reinterpret_cast<int *>(&P)[w] = reinterpret_cast<const int *>(B.phys + inst)[w];
+                load_form_geom<F32, FA>(B, inst, fg);
+                __syncthreads();
+                if (threadIdx.x == 0) p_inst = inst;
             }
         }
-        __syncthreads();
-        if (quit) break;
-        const int inst = w_inst;
-        if (inst < 0) {
-            __nanosleep(128);
-            continue;
-        }
-        const int t = w_tile, it = w_it;
-        if (inst != p_inst) {
-            for (int w = threadIdx.x; w < (int)(sizeof(Phys) / 4); w += blockDim.x)
-                reinterpret_cast<int *>(&P)[w] = reinterpret_cast<const int *>(B.phys + inst)[w];
-            load_form_geom<F32, FA>(B, inst, fg);
-            __syncthreads();
-            if (threadIdx.x == 0) p_inst = inst;
-        }
+        const int inst = w_inst, t = w_tile, it = w_it;
         double a = 0, b = 0;
         tile_iteration<D, F32, false, L, FA>(B, P, fg, it & 1, t, sh, rp, a, b);
         int tlo, thi;
@@ -1058,8 +1067,16 @@ __global__ void __launch_bounds__(kBlock, F32 ? (D == 3 && (L == 1 || FA) ? 2 : 
         if (threadIdx.x == 0) {
             blk[2 * t] = a;
             blk[2 * t + 1] = b;
-            __threadfence();
-            last_sh = atomicAdd(&B.il[inst].done_tiles, 1u) == (unsigned int)(thi - tlo - 1);
+            more = t + 1 < w_end;
+            last_sh = 0;
+            if (more) {
+                w_tile = t + 1;
+            } else {
+                // (the claim's tiles: from a multiple of claim_tiles of the instance's)
+                const unsigned int k = (t - tlo) % B.claim_tiles + 1;
+                __threadfence();
+                last_sh = atomicAdd(&B.il[inst].done_tiles, k) + k == (unsigned int)(thi - tlo);
+            }
         }
         __syncthreads();
         if (last_sh) {
