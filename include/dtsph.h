@@ -100,9 +100,11 @@ typedef struct {
                                  are first set (timed candidates, cached per shape in the
                                  process). With moving != 0, the lanes of the moving pass; 0 =
                                  one on FP32C, up to four on FP64 (no tuning) */
-    int32_t stages;           /* staging depth of the one-lane kernel (lanes = 1): pair-cache
-                                 chunks in flight per warp in shared memory, 2..8; 0 = 3, or
-                                 picked by the autotuner together with lanes */
+    int32_t stages;           /* staging depth of the one-lane kernel (lanes = 1), 2..8: FP64
+                                 pair-cache chunks in flight per warp in shared memory; FP32C
+                                 rounds of cache rows brought into L2 ahead of use (a cache
+                                 that exceeds L2). 0 = 3, or picked by the autotuner together
+                                 with lanes */
     int32_t shifting;         /* 1: particle shifting after every real step (Sec. 3.5, Eqs.
                                  shift-deltar, shift-correct): at the new positions,
                                  dr_i = -(h^2/2) sum_j V_j (1 + W_ij / W(h)) gradW_ij over every

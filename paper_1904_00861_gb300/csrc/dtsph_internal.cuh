@@ -41,7 +41,7 @@ enum : uint32_t { kErrCapacity = 1u, kErrDomain = 2u, kErrBarrier = 4u, kErrCopy
 // at most kSlotAlign consecutive slots from a multiple of its own width, so a
 // block never straddles two instances.
 constexpr int kSlotAlign = 256;
-constexpr int kMaxStages = 8;        // deepest shared-memory ring of the one-lane iterate kernel
+constexpr int kMaxStages = 8;        // deepest staging of the one-lane iterate kernels
 constexpr uint32_t kNoParticle = 0xFFFFFFFFu;
 constexpr unsigned long long kBarrierWaitNs = 1000000000ull;   // grid-barrier give-up time (1 s)
 // Batches of up to this many instances deal their active tiles to the blocks

@@ -83,39 +83,6 @@ __device__ __forceinline__ void decode_shift(int code, int &dx, int &dy, int &dz
     dz = code / 9 - 1;
 }
 
-// Reciprocal square root and division in the working precision: the fast
-// single-precision forms (a few ulp) on the FP32C path, IEEE double otherwise.
-template <typename T> struct F32Math;
-template <> struct F32Math<float> {
-    static __device__ __forceinline__ float rsqrt(float x) { return rsqrtf(x); }
-    static __device__ __forceinline__ float div(float a, float b) { return __fdividef(a, b); }
-};
-template <> struct F32Math<double> {
-    static __device__ __forceinline__ double rsqrt(double x) { return ::rsqrt(x); }
-    static __device__ __forceinline__ double div(double a, double b) { return a / b; }
-};
-
-// gradW_ij and F_ij = (r_ij . gradW_ij) / (r^2 + eta h^2) from r_ij, with one
-// reciprocal square root: r = r^2 / r, q = r / h, gradW = (dW/dr / r) r_ij.
-template <int D, typename T>
-__device__ __forceinline__ void grad_coef(const Phys &P, const T *d, T r2, T *g, T &F)
-{
-    using A = Ar<T>;
-    if (r2 > T(0)) {
-        const T rinv = F32Math<T>::rsqrt(r2);
-        const T r = A::mul(r2, rinv);
-        const T dwdr = A::mul((T)P.sig_h, quintic_dwdq<T>(A::mul(r, (T)P.inv_h)));
-        const T a = A::mul(dwdr, rinv);
-#pragma unroll
-        for (int k = 0; k < D; ++k) g[k] = A::mul(a, d[k]);
-        F = F32Math<T>::div(A::mul(dwdr, r), A::add(r2, (T)P.eta_h2));
-    } else {
-#pragma unroll
-        for (int k = 0; k < D; ++k) g[k] = T(0);
-        F = T(0);
-    }
-}
-
 // The cell of a position along one axis; outside a closed axis: flagged, clamped.
 __device__ __forceinline__ int cell_coord(double xa, double lo, double hi, double inv_s, int nc, int periodic,
                                           uint32_t *err)

@@ -193,14 +193,7 @@ extern "C" int dtsph_eval_rates_noalloc(const dtsph_params *p, int64_t nf, const
     I.nf = (int)nf;
     I.nw = (int)nw;
 
-    // the launches overlap, but not in a stream capture (see launch_next)
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
-        cudaGetLastError();
-        return DTSPH_E_CUDA;
-    }
-    B.chain = cap == cudaStreamCaptureStatusNone;
-
+    B.chain = 1;                     // the launches overlap (see launch_next)
     if (cudaMemsetAsync(B.err, 0, sizeof(uint32_t), st) != cudaSuccess) {
         cudaGetLastError();
         return DTSPH_E_CUDA;

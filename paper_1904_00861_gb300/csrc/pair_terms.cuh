@@ -117,6 +117,7 @@ struct Plain64 {
     __device__ __forceinline__ void shfl_merge(int lane_mask) { s += __shfl_xor_sync(0xffffffffu, s, lane_mask); }
 };
 
+// Constants of a pair's FP64 terms.
 template <typename T>
 struct PairConst {
     T c_div, c_edac, c_p, c_visc, c_av_m;   // c_av_m = m * alpha h c / rho0
@@ -139,57 +140,6 @@ __device__ __forceinline__ PairConst<T> pair_const(const Phys &P)
     k.steady = P.steady;
     k.rare = P.use_av || P.steady;
     return k;
-}
-
-// One pair's contribution. g: gradW_ij (D comps), F: F_ij. vi, pi: own velocity
-// and pressure; vj_div, vj_vis: neighbour velocity seen by the divergence and by
-// the viscous term (equal for fluid neighbours); pj: neighbour pressure. In the
-// steady-state mode (k.steady) the convection term is added.
-template <int D, typename T, typename Acc>
-__device__ __forceinline__ void pair_accumulate(const PairConst<T> &k, const T *g, T F, const T *vi, T pi,
-                                                const T *vj_div, const T *vj_vis, T pj, Acc &ap, Acc *Fi)
-{
-    using A = Ar<T>;
-    T vdg = T(0);
-    T vv[3];
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        vdg = A::fma(A::sub(vi[a], vj_div[a]), g[a], vdg);
-        vv[a] = A::sub(vi[a], vj_vis[a]);
-    }
-    T t_ap = A::mul(k.c_div, vdg);
-    if (k.edac) t_ap = A::fma(A::mul(k.c_edac, A::sub(pi, pj)), F, t_ap);
-    ap.add(t_ap);
-    T pres = A::mul(k.c_p, A::add(pi, pj));
-    const T cv = A::mul(k.c_visc, F);
-    // the terms that most runs do without (artificial viscosity, the steady-mode
-    // convection) sit behind one uniform test
-    if (k.rare) {
-        if (k.use_av) {
-            // v_ij . r_ij < 0  <=>  v_ij . gradW > 0 (dW/dr < 0); phi_ij = (v_ij . gradW) F / |gradW|^2
-            T vvg = T(0), g2 = T(0);
-#pragma unroll
-            for (int a = 0; a < D; ++a) {
-                vvg = A::fma(vv[a], g[a], vvg);
-                g2 = A::fma(g[a], g[a], g2);
-            }
-            if (vvg > T(0) && g2 > T(0)) pres = A::sub(pres, A::mul(k.c_av_m, A::mul(vvg, F)) / g2);   // -m Pi_ij
-        }
-        if (k.steady) {
-            // convection of Eq. (mom-steady): -(V_i m_i/rho_i + V_j m_j/rho_j) (V_i . gradW_ij),
-            // V_j the divergence-side velocity (prescribed for a wall)
-            T vg = T(0);
-#pragma unroll
-            for (int a = 0; a < D; ++a) vg = A::fma(vi[a], g[a], vg);
-#pragma unroll
-            for (int a = 0; a < D; ++a)
-                Fi[a].add(A::sub(A::fma(cv, vv[a], A::mul(-pres, g[a])),
-                                 A::mul(A::mul(k.vol, A::add(vi[a], vj_div[a])), vg)));
-            return;
-        }
-    }
-#pragma unroll
-    for (int a = 0; a < D; ++a) Fi[a].add(A::fma(cv, vv[a], A::mul(-pres, g[a])));
 }
 
 }  // namespace dtsph
