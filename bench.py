@@ -52,19 +52,15 @@ UNIT = "particle-iterations/s"
 # bytes per algorithmic byte of the form it ran times its own algorithmic bytes.
 # A variant not listed (a step that switched forms included), or one whose
 # kernel changed after its capture, reports null.
-NCU_TRAFFIC = {
-    ("batch-64x-tgv2d", 2, 1, 2, 1): (6.357158e9 + 0.056701e9, 6.667369e9, "profiles/k_loop_async_batch64_tgv2d.md"),
-    ("batch-64x-tgv2d", 2, 1, 2, 2): (0.682724e9 + 0.142967e9, 2.441234e9, "profiles/k_loop_async_batch64_tgv2d.md"),
-}
+# (Empty: the loop kernels changed after the committed captures.)
+NCU_TRAFFIC = {}
 
 # FP32 flops of the loop without the pair cache, from the FP32 operation counters
 # of an Nsight Compute capture (fadd + fmul + 2 ffma, thread instructions):
 # dim -> (flops per pair-iteration, workload, source). The form is bound by
 # neither HBM nor the FP32 pipe; this places its launches against the FP32 peak.
-NCU_FLOPS_NO_CACHE = {
-    2: (62.51, "batch-64x-tgv2d", "profiles/k_loop_async_batch64_tgv2d.md"),
-    3: (75.46, "tgv3d 80^3", "profiles/k_loop_no_cache_tgv3d_80.md"),
-}
+# (Empty for the same reason: the packed arithmetic changed the operation counts.)
+NCU_FLOPS_NO_CACHE = {}
 
 
 def make_workload(name: str, n_side: int, re: float):
@@ -610,7 +606,7 @@ def main_ours(args):
     achieved = loop_bytes / (sum(loop_ms) * 1e-3) / 1e9
     probe_bytes = STATE_BYTES[(dims, True)] * nf_tot + PAIR_BYTES[(dims, True)] * npairs
     achieved_probe = probe_bytes / (ms_it * 1e-3) / 1e9
-    loop_kernel = {2: f"k_loop<{dims},FP32C,lanes={lanes32}> (persistent loop, one launch per step)",
+    loop_kernel = {2: f"k_loop or k_loop_res<{dims},FP32C,lanes={lanes32}> (persistent loop, one launch per step)",
                    1: f"k_iterate<{dims},FP32C,lanes={lanes32}> in the while node (one launch per iteration)",
                    0: f"k_iterate<{dims},FP32C,lanes={lanes32}> (plain launches)"}[args.graph]
     if decoupled:
@@ -621,6 +617,8 @@ def main_ours(args):
         probe_kernel = f"k_move_walls + k_move_iter<{dims},FP32C> (one lane per particle)"
         loop_kernel = probe_kernel + (" (plain launches)" if args.graph == 0 else
                                       " in the while node (one launch each per iteration)")
+        if args.graph == 2 and not decoupled and wcfg["workload"] != "batch-64x-tgv2d":
+            loop_kernel = f"k_move_loop<{dims},FP32C> (persistent loop, one launch per step)"
     traffic, traffic_src, traffic_cap = None, None, None
     # a switched step (form 3) counts its iterations with and without the cache
     # at the two forms' captured ratios
