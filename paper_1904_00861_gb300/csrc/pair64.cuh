@@ -20,12 +20,13 @@ namespace dtsph {
 // 1/sqrt(x) for a normal positive x: from an approximation y with e = 1 - x y^2,
 // the third-order step y (1 + e/2 + 3 e^2/8) of the binomial series of (1 -
 // e)^(-1/2). The approximation's relative error is below 2^-19 (e < 2^-18), the
-// step's truncation below 5/16 e^3 < 2^-55.
+// step's truncation below 5/16 e^3 < 2^-55. The approximation has few digits, so y^2
+// loses none (x y would, as much as the step's last bit).
 __device__ __forceinline__ double rsqrt_step(double x)
 {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = __fma_rn(-__dmul_rn(x, y), y, 1.0);
+    const double e = __fma_rn(-x, __dmul_rn(y, y), 1.0);
     return __fma_rn(__dmul_rn(y, e), __fma_rn(0.375, e, 0.5), y);
 }
 
