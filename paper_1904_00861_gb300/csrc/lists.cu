@@ -352,8 +352,7 @@ __global__ void __launch_bounds__(kListWarps * kWarp) k_nlist_home(Buffers B, co
         const bool act = s < he;
         const int nh = min(kWarp, he - h0);
         const int kh = D == 2 ? (s >= b1) + (s >= b2) : 0;      // the lane's cell in the segment
-        // an idle lane tests from far away: it fails every distance test
-        float4 oi = make_float4(3e18f, 3e18f, 3e18f, 0.f);
+        float4 oi = make_float4(0.f, 0.f, 0.f, 0.f);    // (an idle lane's hits are dropped)
         if (act) {
             oi = B.off[s];
             if (D == 2) oi.x = __fadd_rn(oi.x, (float)kh * sx);
@@ -409,14 +408,15 @@ __global__ void __launch_bounds__(kListWarps * kWarp) k_nlist_home(Buffers B, co
                 p0 += kWarp;
             }
             const bool end = p0 >= total;
+            const int real = take;                      // (beyond: the fill of the last chunk)
             if (end && (take & (kWarp - 1))) {
-                // the last chunk is filled up with candidates that fail every test
+                // the last chunk is filled up; hits beyond the candidates are dropped
                 const int at = take + lane;
                 take = (take + kWarp - 1) / kWarp * kWarp;
                 if (at < take) {
-                    cx[w][0][at] = -3e18f;
-                    cx[w][1][at] = -3e18f;
-                    if constexpr (D == 3) cx[w][2][at] = -3e18f;
+                    cx[w][0][at] = 0.f;
+                    cx[w][1][at] = 0.f;
+                    if constexpr (D == 3) cx[w][2][at] = 0.f;
                     ent[w][at] = 0u;
                 }
             }
@@ -441,8 +441,10 @@ __global__ void __launch_bounds__(kListWarps * kWarp) k_nlist_home(Buffers B, co
                     }
                 }
                 // the FP64 decision inside the band (rare)
-                if (__any_sync(full, near < band) && near < band) {
-                    for (int q = 0; q < kWarp; ++q) {
+                const int nv = min(kWarp, real - c * kWarp);
+                const bool at_cutoff = act && near < band;
+                if (__any_sync(full, at_cutoff) && at_cutoff) {
+                    for (int q = 0; q < nv; ++q) {
                         const int at = c * kWarp + q;
                         const float d2 = near_test<D>(oi, cx[w][0][at], cx[w][1][at], cx[w][D - 1][at], neg_lo);
                         if (__float_as_uint(d2) >= band) continue;
@@ -450,6 +452,9 @@ __global__ void __launch_bounds__(kListWarps * kWarp) k_nlist_home(Buffers B, co
                         if (sep64<D>(G, xpos, n, s, entry_slot(ent[w][at]), d64) < G.rc2) hits |= 0x80000000u >> q;
                     }
                 }
+                // real candidates of a lane with a particle only (by their number: whatever
+                // the scale of the coordinates, nothing else is listed)
+                hits &= act ? ~(uint32_t)(0xffffffffull >> nv) : 0u;
                 if (mine >> 5 == c) hits &= ~(0x80000000u >> (mine & 31));    // not itself
                 const int nhit = __popc(hits);
                 // (a list longer than its row is cut there and raises the error below)
