@@ -193,6 +193,7 @@ int dtsph::make_geometry(const dtsph_params &p, Geom &G, char *msg, size_t cap)
     // (pairs beyond 3h add exact zeros)
     const double rc = 3.0 * p.h + (p.moving == 2 ? p.skin : 0.0) + p.list_skin;
     G.ncell = 1;
+    G.off_scale = p.precision == DTSPH_FP64 ? std::ldexp(1.0, -std::ilogb(rc)) : 1.0;
     for (int a = 0; a < 3; ++a) {
         G.periodic[a] = a < p.dim ? p.periodic[a] : 0;
         G.lo[a] = p.lo[a];
@@ -220,7 +221,7 @@ int dtsph::make_geometry(const dtsph_params &p, Geom &G, char *msg, size_t cap)
         G.nc[a] = (int)k;
         G.s[a] = L / (double)k;
         G.inv_s[a] = 1.0 / G.s[a];
-        G.s_f[a] = (float)G.s[a];
+        G.s_f[a] = (float)(G.s[a] * G.off_scale);
         G.L[a] = L;
         G.halfL[a] = 0.5 * L;
         G.ncell *= (int)k;
@@ -229,8 +230,9 @@ int dtsph::make_geometry(const dtsph_params &p, Geom &G, char *msg, size_t cap)
     G.rc2 = rc * rc;
     // FP32 band around the cutoff: the FP32 separation from cell offsets is accurate
     // to a few 1e-7 h, so outside +-2e-5 relative the FP32 test decides
-    G.rc2_lo = (float)(G.rc2 * (1.0 - 2e-5));
-    G.rc2_hi = (float)(G.rc2 * (1.0 + 2e-5));
+    const double rs2 = (rc * G.off_scale) * (rc * G.off_scale);
+    G.rc2_lo = (float)(rs2 * (1.0 - 2e-5));
+    G.rc2_hi = (float)(rs2 * (1.0 + 2e-5));
     return DTSPH_OK;
 }
 

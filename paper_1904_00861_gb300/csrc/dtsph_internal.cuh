@@ -72,9 +72,15 @@ struct Geom {
     double lo[3], hi[3];
     double L[3], halfL[3];
     double s[3], inv_s[3];
+    // FP32 offsets, cell sides and the pre-test band (below lo is in, above hi is out)
+    // are in units of 1 / off_scale: FP32C 1; FP64, whose offsets the list builders
+    // alone read, the power of two next to the cutoff, so that the pre-test holds at
+    // every scale that FP64 does
+    double off_scale;
     float s_f[3];
+    float rc2_lo, rc2_hi;
+    float pad_f;
     double rc2;           // (3h + skin)^2, the FP64 neighbour test (skin: moving = 2 only)
-    float rc2_lo, rc2_hi; // FP32 pre-test band: below lo is in, above hi is out
 };
 
 // Constants of the FP32C path's packed pair sums (pair32.cuh), rounded from Phys.

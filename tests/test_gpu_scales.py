@@ -1,7 +1,9 @@
 """Length scales at which squares of coordinates leave single precision.
 
 The list builders decide most pairs on FP32 offsets. On the FP32C path such a scale
-has no meaning for the sums, but a list must hold nothing except particles.
+has no meaning for the sums, but a list must hold nothing except particles. The FP64
+path computes at every scale: a change of the unit of length by a power of two is
+exact, so its lists stay the same.
 """
 import numpy as np
 import pytest
@@ -47,3 +49,16 @@ def test_only_particles_are_listed_beyond_single_precision(dim, ncell, n):
     cfg, x = scattered(dim, ncell, n, 2.0 ** 70)
     for i, a in enumerate(lists(cfg, x, F32)):
         assert len(np.unique(a)) == len(a) and i not in a and (len(a) == 0 or (a.min() >= 0 and a.max() < n)), i
+
+
+# the builder of few 2D cells, the one of many segments, 3D; (3h)^2 overflows FP32 from
+# h = 2^62 on and is subnormal below h = 2^-64; at 2^61 an FP32 offset is finite still
+@pytest.mark.parametrize("exponent", [-200, -80, -66, 61, 70, 200])
+@pytest.mark.parametrize("dim,ncell,n", [(2, 12, 700), (2, 224, 300), (3, 9, 400)])
+def test_fp64_lists_do_not_depend_on_the_unit_of_length(dim, ncell, n, exponent):
+    cfg, x = scattered(dim, ncell, n, 1.0)
+    want = lists(cfg, x, F64)
+    assert max(len(a) for a in want) > 8
+    cfg, x = scattered(dim, ncell, n, 2.0 ** exponent)
+    for i, (a, b) in enumerate(zip(want, lists(cfg, x, F64))):
+        assert np.array_equal(a, b), i
