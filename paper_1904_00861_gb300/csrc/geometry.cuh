@@ -10,7 +10,7 @@ namespace dtsph {
 
 // r_ij in FP64 with the minimum image; returns |r_ij|^2 (no FMA contraction).
 template <int D>
-__device__ __forceinline__ double sep64(const Geom &G, const double *__restrict__ x, int n, int i, int j, double *d)
+__device__ __forceinline__ double sep64(const Geom &G, const double *x, int n, int i, int j, double *d)
 {
 #pragma unroll
     for (int a = 0; a < D; ++a) {

@@ -56,7 +56,7 @@ __device__ __forceinline__ int cell_instance(const Buffers &B, int c)
 
 // 2D lists of small problems, one warp per cell with the candidates in the lanes
 // (see the top of the file).
-__global__ void __launch_bounds__(kBlock) k_nlist_cells2(Buffers B, const double *__restrict__ xpos,
+__global__ void __launch_bounds__(kBlock) k_nlist_cells2(Buffers B, const double *xpos,
                                                          uint32_t *__restrict__ lists, int Ks)
 {
     grid_start<false>();
@@ -269,7 +269,7 @@ __device__ __forceinline__ void near_test2(const F2 *oi, F2 x, F2 y, F2 z, F2 ne
 }
 
 template <int D>
-__global__ void __launch_bounds__(kListWarps * kWarp) k_nlist_home(Buffers B, const double *__restrict__ xpos,
+__global__ void __launch_bounds__(kListWarps * kWarp) k_nlist_home(Buffers B, const double *xpos,
                                                                    uint32_t *__restrict__ lists, int Ks)
 {
     grid_start<false>();
