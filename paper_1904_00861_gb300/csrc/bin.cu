@@ -201,10 +201,9 @@ __global__ void __launch_bounds__(kBlock) k_scatter(Buffers B)
 
 // FP32 offset of slot s from the origin of its cell (in units of 1 / off_scale: 1 on
 // the FP32C path); .w is 1 for a wall particle.
-template <bool F32>
 __device__ __forceinline__ float4 cell_offset(const Geom &G, int local_cell, const double *x, int n, int s, bool wall)
 {
-    const double u = F32 ? 1.0 : G.off_scale;
+    const double u = G.off_scale;
     const int c0 = local_cell % G.nc[0];
     const int c1 = (local_cell / G.nc[0]) % G.nc[1];
     const int c2 = local_cell / (G.nc[0] * G.nc[1]);
@@ -267,14 +266,12 @@ __device__ __forceinline__ void move_a_to_b(const Buffers &B, int o, int s, int 
     const double p = B.pn_a[o];
     B.pn_b[s] = p;
     // (the FP64 path reads the offsets in the list builders only)
-    const int inst = B.inst_of[s], lc = cell - B.inst[inst].cell_off;
-    const bool wall = g >= (uint32_t)B.nf;
+    const int inst = B.inst_of[s];
+    B.off[s] = SAME ? cell_offset_near(B.geo[inst], cell - B.inst[inst].cell_off, B.x_b, n, s, g >= (uint32_t)B.nf)
+                    : cell_offset(B.geo[inst], cell - B.inst[inst].cell_off, B.x_b, n, s, g >= (uint32_t)B.nf);
     if (B.fp32c) {
-        B.off[s] = SAME ? cell_offset_near(B.geo[inst], lc, B.x_b, n, s, wall)
-                        : cell_offset<true>(B.geo[inst], lc, B.x_b, n, s, wall);
         B.nb32[1][s] = make_float4((float)v[0], (float)v[1], (float)v[2], (float)p);
     } else {
-        if (!SAME) B.off[s] = cell_offset<false>(B.geo[inst], lc, B.x_b, n, s, wall);
         B.nb64[1][s] = make_double4_32a(v[0], v[1], v[2], p);
     }
 }
@@ -312,12 +309,11 @@ __device__ __forceinline__ void move_b_to_a(const Buffers &B, int o, int s, int 
     }
     if (wall) store_wall_velocity(B, s, u);
     const double ph = B.ph0_b[o];
-    const int inst = B.inst_of[s], lc = cell - B.inst[inst].cell_off;
+    const int inst = B.inst_of[s];
+    B.off[s] = cell_offset(B.geo[inst], cell - B.inst[inst].cell_off, B.xp_a, n, s, g >= (uint32_t)B.nf);
     if (B.fp32c) {
-        B.off[s] = cell_offset<true>(B.geo[inst], lc, B.xp_a, n, s, wall);
         B.nb32[0][s] = make_float4((float)v[0], (float)v[1], (float)v[2], (float)ph);
     } else {
-        B.off[s] = cell_offset<false>(B.geo[inst], lc, B.xp_a, n, s, wall);
         B.nb64[0][s] = make_double4_32a(v[0], v[1], v[2], ph);
     }
 }

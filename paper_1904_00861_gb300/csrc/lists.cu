@@ -352,7 +352,11 @@ __global__ void __launch_bounds__(kListWarps * kWarp) k_nlist_home(Buffers B, co
         const bool act = s < he;
         const int nh = min(kWarp, he - h0);
         const int kh = D == 2 ? (s >= b1) + (s >= b2) : 0;      // the lane's cell in the segment
-        float4 oi = make_float4(0.f, 0.f, 0.f, 0.f);    // (an idle lane's hits are dropped)
+        // NaN fails every test whatever the scale of the coordinates (its bits are those
+        // of a large positive number: arithmetic gives 0x7fffffff): an idle lane's place,
+        // and below the fill of the last chunk
+        const float nan = __int_as_float(0x7fffffff);
+        float4 oi = make_float4(nan, nan, nan, 0.f);
         if (act) {
             oi = B.off[s];
             if (D == 2) oi.x = __fadd_rn(oi.x, (float)kh * sx);
@@ -408,15 +412,14 @@ __global__ void __launch_bounds__(kListWarps * kWarp) k_nlist_home(Buffers B, co
                 p0 += kWarp;
             }
             const bool end = p0 >= total;
-            const int real = take;                      // (beyond: the fill of the last chunk)
             if (end && (take & (kWarp - 1))) {
-                // the last chunk is filled up; hits beyond the candidates are dropped
+                // the last chunk is filled up with candidates that fail every test
                 const int at = take + lane;
                 take = (take + kWarp - 1) / kWarp * kWarp;
                 if (at < take) {
-                    cx[w][0][at] = 0.f;
-                    cx[w][1][at] = 0.f;
-                    if constexpr (D == 3) cx[w][2][at] = 0.f;
+                    cx[w][0][at] = nan;
+                    cx[w][1][at] = nan;
+                    if constexpr (D == 3) cx[w][2][at] = nan;
                     ent[w][at] = 0u;
                 }
             }
@@ -441,10 +444,8 @@ __global__ void __launch_bounds__(kListWarps * kWarp) k_nlist_home(Buffers B, co
                     }
                 }
                 // the FP64 decision inside the band (rare)
-                const int nv = min(kWarp, real - c * kWarp);
-                const bool at_cutoff = act && near < band;
-                if (__any_sync(full, at_cutoff) && at_cutoff) {
-                    for (int q = 0; q < nv; ++q) {
+                if (__any_sync(full, near < band) && near < band) {
+                    for (int q = 0; q < kWarp; ++q) {
                         const int at = c * kWarp + q;
                         const float d2 = near_test<D>(oi, cx[w][0][at], cx[w][1][at], cx[w][D - 1][at], neg_lo);
                         if (__float_as_uint(d2) >= band) continue;
@@ -452,9 +453,6 @@ __global__ void __launch_bounds__(kListWarps * kWarp) k_nlist_home(Buffers B, co
                         if (sep64<D>(G, xpos, n, s, entry_slot(ent[w][at]), d64) < G.rc2) hits |= 0x80000000u >> q;
                     }
                 }
-                // real candidates of a lane with a particle only (by their number: whatever
-                // the scale of the coordinates, nothing else is listed)
-                hits &= act ? ~(uint32_t)(0xffffffffull >> nv) : 0u;
                 if (mine >> 5 == c) hits &= ~(0x80000000u >> (mine & 31));    // not itself
                 const int nhit = __popc(hits);
                 // (a list longer than its row is cut there and raises the error below)
