@@ -9,35 +9,13 @@
 // which takes 4 d + 3 instructions a pair (11 in 2D, 15 in 3D; with the constants
 // inside the sums 18 and 23), every one of them on a difference or sum formed
 // first as before. The geometry takes comparisons of high words instead of FP64
-// comparisons, and the reciprocal and its square root from one third-order step
-// on the hardware's approximations.
+// comparisons; its square root and its division are CUDA's (a reciprocal in the place of
+// the division was 1 to 2.5% faster, with a rounding more).
 #pragma once
 
 #include "geometry.cuh"
 
 namespace dtsph {
-
-// 1/sqrt(x) for a normal positive x: from an approximation y with e = 1 - x y^2,
-// the third-order step y (1 + e/2 + 3 e^2/8) of the binomial series of (1 -
-// e)^(-1/2). The approximation's relative error is below 2^-19 (e < 2^-18), the
-// step's truncation below 5/16 e^3 < 2^-55. The approximation has few digits, so y^2
-// loses none (x y would, as much as the step's last bit).
-__device__ __forceinline__ double rsqrt_step(double x)
-{
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = __fma_rn(-x, __dmul_rn(y, y), 1.0);
-    return __fma_rn(__dmul_rn(y, e), __fma_rn(0.375, e, 0.5), y);
-}
-
-// 1/x for a normal x: y (1 + e + e^2), e = 1 - x y, truncation e^3 < 2^-57.
-__device__ __forceinline__ double rcp_step(double x)
-{
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = __fma_rn(-x, y, 1.0);
-    return __fma_rn(y, __fma_rn(e, e, e), y);
-}
 
 // r_ij of a listed neighbour with the minimum image, and |r_ij|^2: sep64's
 // operations, the image chosen by comparing high words (a listed pair lies within
@@ -66,7 +44,7 @@ __device__ __forceinline__ void grad64(const Phys &P, const double *d, double r2
     for (int a = 0; a < D; ++a) g[a] = 0.0;
     F = 0.0;
     if (__double2hiint(r2) < 0x00100000) return;        // r = 0 (or r^2 subnormal)
-    const double rinv = rsqrt_step(r2);
+    const double rinv = rsqrt(r2);
     const double r = __dmul_rn(r2, rinv);
     const double q = __dmul_rn(r, P.inv_h);
     const int qh = __double2hiint(q);                   // 1, 2 and 3 have zero low words
@@ -84,7 +62,7 @@ __device__ __forceinline__ void grad64(const Phys &P, const double *d, double r2
     const double wr = __dmul_rn(w, rinv);
 #pragma unroll
     for (int e = 0; e < D; ++e) g[e] = __dmul_rn(wr, d[e]);
-    F = __dmul_rn(__dmul_rn(w, r), rcp_step(__dadd_rn(r2, P.eta_h2)));
+    F = __ddiv_rn(__dmul_rn(w, r), __dadd_rn(r2, P.eta_h2));
 }
 
 template <int D>
