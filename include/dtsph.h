@@ -26,8 +26,9 @@
  *    persistent loop's grid barrier (default one second); a step whose barrier
  *    gave up is reported by dtsph_sync as DTSPH_E_TIMEOUT.
  *  - DTSPH_TUNE_CACHE (a file name, optional): the autotuner's choices persist
- *    there across processes, keyed by device, dim, precision, slots, instances
- *    and loop driver; a shape found in the file is not timed again.
+ *    there across processes, keyed by device, the library's kernels, list capacity,
+ *    walls or not, dim, precision, slots, instances and loop driver; a shape found in
+ *    the file is not timed again.
  */
 #ifndef DTSPH_H
 #define DTSPH_H

@@ -345,14 +345,14 @@ int validate(dtsph_ctx *c, const dtsph_params *p)
 }
 
 // Autotuner results: lanes per particle of the iterate kernel and, with one
-// lane, its staging depth, keyed by (device, dim, precision, slots, instances,
-// persistent loop or not), shared by every context of the process. With
-// DTSPH_TUNE_CACHE set to a file name they also persist across processes: the
-// file is read once per process, and every new choice is appended to it as one
-// line "dtsph-tune-v1 <device> <dim> <precision> <slots> <instances> <loop>
-// <lanes> <stages>" (the last line of a key wins).
+// lane, its staging depth, keyed by (device, kernels, list capacity, walls or not,
+// dim, precision, slots, instances, persistent loop or not), shared by every context
+// of the process. With DTSPH_TUNE_CACHE set to a file name they also persist across
+// processes: the file is read once per process, and every new choice is appended to
+// it as one line "dtsph-tune-v1 <key> <dim> <precision> <slots> <instances> <loop>
+// <lanes> <stages>" (the last line of a key wins), <key> the first four in one word.
 struct TuneKey {
-    std::string dev;   // device name and SM count, spaces replaced
+    std::string dev;   // device name and SM count, spaces replaced, then /kernels/K[/walls]
     int dim, prec;
     int64_t n;
     int ninst, loop;
@@ -391,8 +391,8 @@ std::map<FormKey, FormCosts> &form_cache()
 }
 
 // Reads the persisted choices once (tune_mu held): one record per line,
-// "dtsph-tune-v1 <device> dim precision slots instances loop lanes stages" and
-// "dtsph-form-v1 <device> dim precision slots instances loop lanes stages kstar
+// "dtsph-tune-v1 <key> dim precision slots instances loop lanes stages" and
+// "dtsph-form-v1 <key> dim precision slots instances loop lanes stages kstar
 // cache_ms cached_ms uncached_ms"; other lines are skipped.
 void load_tune_file()
 {
@@ -469,9 +469,19 @@ std::string device_tag(int dev)
     return name + "/" + std::to_string(prop.multiProcessorCount) + "sm";
 }
 
+// The generation of the kernels that the times belong to: a choice or a break-even
+// count that an older build left in the file was timed on other kernels. To be
+// raised when the loop, the cache pass or the uncached form change.
+constexpr const char *kTunedKernels = "resident2";
+
+// Part of the key with the slots: the list capacity, which sets how many cache rows the
+// resident loop keeps in shared memory, and whether there are walls, whose loop is
+// another kernel with a phase and a barrier more.
 TuneKey tune_key(const dtsph_ctx *c, int64_t n)
 {
-    return TuneKey{device_tag(c->device), c->prm[0].dim, c->prm[0].precision, n, c->ninst, c->prm[0].graph == 2};
+    const std::string dev = device_tag(c->device) + "/" + kTunedKernels + "/K" + std::to_string(c->B.K) +
+                            (c->B.nw > 0 ? "/walls" : "");
+    return TuneKey{dev, c->prm[0].dim, c->prm[0].precision, n, c->ninst, c->prm[0].graph == 2};
 }
 
 // Lanes and stages for n slots: the parameters' when fixed, else the process

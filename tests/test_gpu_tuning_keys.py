@@ -1,0 +1,63 @@
+"""What a tuned choice is kept under: the kernels it was timed on, the list capacity and
+whether there are walls, besides the shape. Contexts that differ in one of them are
+timed on their own, and a file written for other kernels is passed over."""
+import json
+import os
+import subprocess
+import sys
+
+import pytest
+
+import paper_1904_00861_gb300 as dt
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_1904_00861_gb300 import build
+    build.build()
+
+
+def timed(d, **over):
+    """The number of candidates that a context of this state times."""
+    sim = dt.Simulation(d["cfg"], precision=dt.DTSPH_FP32C, lanes=0, graph=2, form=1, **over)
+    nf = d["nf"]
+    sim.set_state(d["x"][:nf], d["v"], d["p"], d["v_prev"], walls=None if d["vw"] is None else (d["x"][nf:], d["vw"]))
+    out = len(dt.dtsph_tuning_candidates(sim.ctx)[1])
+    sim.close()
+    return out
+
+
+def test_walls_and_capacity_are_timed_on_their_own():
+    # 44^2 = 1936 fluid particles; 38^2 with three rings of walls the same number of all
+    plain, walled = synth.tgv2d(44, seed=9), synth.cavity2d(38)
+    assert len(plain["x"]) == len(walled["x"])
+    assert timed(plain) == 7 and timed(plain) == 0
+    assert timed(walled) == 7 and timed(walled) == 0
+    assert timed(plain, max_neighbors=77) == 7 and timed(plain, max_neighbors=77) == 0
+
+
+def test_a_file_of_other_kernels_is_passed_over(tmp_path):
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    code = ("import json, synth, paper_1904_00861_gb300 as dt\n"
+            "d = synth.tgv2d(46, seed=2)\n"
+            "s = dt.Simulation(d['cfg'], precision=dt.DTSPH_FP32C, lanes=0, graph=2)\n"
+            "s.set_state(d['x'], d['v'], d['p'], d['v_prev'])\n"
+            "print(json.dumps([len(dt.dtsph_tuning_candidates(s.ctx)[1]), s.form_stats()['kstar']]))\n")
+    path = tmp_path / "tune.txt"
+    env = dict(os.environ, DTSPH_TUNE_CACHE=str(path))
+    run = lambda: json.loads(subprocess.run([sys.executable, "-c", code], cwd=root, env=env, check=True,
+                                            capture_output=True, text=True).stdout.strip().splitlines()[-1])
+    assert run()[0] == 7
+    lines = [ln.split() for ln in path.read_text().splitlines()]
+    # the lines as builds with other kernels wrote them: the device alone; a kstar of note
+    old = [[ln[0], "/".join(ln[1].split("/")[:2])] + ln[2:] for ln in lines]
+    for ln in old:
+        if ln[0] == "dtsph-form-v1":
+            ln[9] = "12345.0"
+    path.write_text("".join(" ".join(ln) + "\n" for ln in old))
+    n, kstar = run()
+    assert n == 7 and kstar != 12345.0
+    assert run()[0] == 0                                  # its own lines are taken
