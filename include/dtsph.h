@@ -348,8 +348,8 @@ int dtsph_tuning(const dtsph_ctx *ctx, int32_t *lanes, float *ms_by_lanes);
 /* Every candidate the autotuner timed when this context tuned, in the order
  * timed: lanes per particle, staging depth (0 for lanes > 1) and mean ms per
  * launch of the pseudo-iteration kernel (graph = 0, 1) or per iteration of the
- * persistent loop kernel over four fixed iterations (graph = 2). Writes min(cap, count) entries of
- * the three arrays (each may be NULL when cap is 0); *count = candidates timed
+ * persistent loop kernel over four fixed iterations, 16 where the problem fits the
+ * resident loop (graph = 2). Writes min(cap, count) entries of the three arrays (each may be NULL when cap is 0); *count = candidates timed
  * (0 when the shape's choice came from the process cache or lanes was fixed);
  * *stages = staging depth in use (0 when lanes > 1). */
 int dtsph_tuning_candidates(const dtsph_ctx *ctx, int32_t cap, int32_t *lanes, int32_t *stages, float *ms,
@@ -359,8 +359,9 @@ int dtsph_tuning_candidates(const dtsph_ctx *ctx, int32_t cap, int32_t *lanes, i
  * persistent loop (one instance, or a batch's decoupled loop), no walls and
  * particles fixed in pseudo-time, the context measured at dtsph_set_particles
  * (or took from the process cache or the DTSPH_TUNE_CACHE file) the costs
- * ms[0] = one pair-cache pass, ms[1] = one pseudo-iteration with the cache,
- * ms[2] = one without it (milliseconds, at the lanes and staging depth in use),
+ * ms[0] = one pair-cache pass (with what the cached loop does once a step beyond
+ * the uncached one), ms[1] = one pseudo-iteration with the cache, ms[2] = one
+ * without it (milliseconds, at the lanes and staging depth in use),
  * and *kstar = ms[0] / (ms[2] - ms[1]) (1e9 when the uncached iteration is not
  * slower). The step graph then holds both forms and picks one per step on the
  * device, in stream order: without the cache when the previous step took at

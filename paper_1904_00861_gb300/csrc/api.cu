@@ -1004,9 +1004,9 @@ int probe_ms(dtsph_ctx *c, const Buffers &B, int launches, float *out)
     return DTSPH_OK;
 }
 
-// Mean device time per pseudo-iteration of the persistent loop kernel over
-// `iters` iterations of every instance (fixed_iters forced on the loop state for
-// the probe, then restored), `reps` launches after one untimed launch.
+// Mean device time of a launch of the persistent loop kernel with `iters` iterations
+// of every instance (fixed_iters forced on the loop state for the probe, then
+// restored), `reps` launches after one untimed launch.
 int probe_loop_ms(dtsph_ctx *c, int iters, int reps, float *out)
 {
     const Buffers &B = c->B;
@@ -1035,8 +1035,34 @@ int probe_loop_ms(dtsph_ctx *c, int iters, int reps, float *out)
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     CK(cudaMemcpy(B.ls, saved.data(), sizeof(LoopState) * c->ninst, cudaMemcpyHostToDevice));
-    *out = tot / (float)(reps * iters);
+    *out = tot / (float)reps;
     return DTSPH_OK;
+}
+
+// The loop's time per iteration, and what a launch takes beside its iterations. The
+// resident loop copies its cache rows to shared memory once a launch (2 to 25 us
+// beside a launch's own 8), which four iterations do not spread as the 7 to 50 of a
+// step do: 100 x 100 FP32C 8.1 us an iteration over four, 5.5 by the slope. `slope`:
+// from launches of 4 and of 16 iterations; else four, and nothing beside them.
+int probe_iteration_ms(dtsph_ctx *c, bool slope, int reps, float *per_iter, float *beside)
+{
+    float t4 = 0, t16 = 0;
+    int r = probe_loop_ms(c, 4, reps, &t4);
+    if (!r && slope) r = probe_loop_ms(c, 16, reps, &t16);
+    if (r) return r;
+    *per_iter = slope && t16 > t4 ? (t16 - t4) / 12.f : t4 / 4.f;
+    *beside = std::max(0.f, t4 - 4.f * *per_iter);
+    return DTSPH_OK;
+}
+
+// True where the problem fits the resident loop with one lane per particle.
+bool fits_resident(const Buffers &B)
+{
+    Buffers b = B;
+    b.lanes = 1;
+    b.form_a = 0;
+    ResShape S;
+    return resident_shape(b, &S);
 }
 
 // Times the candidates of the iterate kernel (one lane per particle at
@@ -1072,6 +1098,8 @@ int autotune(dtsph_ctx *c)
     for (int L : {2, 4, 8}) cand.push_back({L, kDefaultStages});
     TuneChoice best{c->B.lanes, c->B.stages};
     float best_ms = 1e30f;
+    // (over as many iterations as a step takes where a launch has a cost of its own)
+    const int iters = fits_resident(B) ? 16 : 4;
     c->tune_log.clear();
     for (const TuneChoice &ch : cand) {
         c->B.lanes = ch.lanes;
@@ -1079,7 +1107,8 @@ int autotune(dtsph_ctx *c)
         float ms = 0;
         int r;
         if (c->prm[0].graph == 2) {
-            r = probe_loop_ms(c, 4, 5, &ms);
+            r = probe_loop_ms(c, iters, 5, &ms);
+            ms /= (float)iters;
         } else {
             probe_ms(c, c->B, 3, &ms);         // warm-up
             r = probe_ms(c, c->B, 10, &ms);
@@ -1109,7 +1138,9 @@ int autotune(dtsph_ctx *c)
 // uncached form leaves out (both build the lists), and one pseudo-iteration of
 // the persistent loop in each form at the context's lanes and staging depth. A
 // step of k iterations costs cache + k * cached against k * uncached, so the
-// uncached form pays up to kstar = cache / (uncached - cached) iterations.
+// uncached form pays up to kstar = cache / (uncached - cached) iterations. What the
+// cached loop's launch takes beside its iterations, beyond the uncached one's, counts
+// with the cache pass.
 // Cached per shape in the process and in the persisted file.
 int measure_form_costs(dtsph_ctx *c)
 {
@@ -1149,16 +1180,18 @@ int measure_form_costs(dtsph_ctx *c)
         if (rep > 0) t_cache += a;
     }
     for (auto &ev : e) cudaEventDestroy(ev);
-    const float ms_cache = t_cache / kReps;
-    float ms_b = 0, ms_a = 0;
+    float ms_cache = t_cache / kReps;
+    float ms_b = 0, ms_a = 0, beside_b = 0, beside_a = 0;
     B.form_a = 0;
-    int r = probe_loop_ms(c, 4, 5, &ms_b);
+    const bool slope = fits_resident(B);
+    int r = probe_iteration_ms(c, slope, 5, &ms_b, &beside_b);
     if (!r) {
         B.form_a = 1;
-        r = probe_loop_ms(c, 4, 5, &ms_a);
+        r = probe_iteration_ms(c, slope, 5, &ms_a, &beside_a);
         B.form_a = 0;
     }
     if (r) return r;
+    ms_cache += std::max(0.f, beside_b - beside_a);
     FormCosts fc;
     fc.ms[0] = ms_cache;
     fc.ms[1] = ms_b;

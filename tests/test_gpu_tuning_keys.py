@@ -61,3 +61,29 @@ def test_a_file_of_other_kernels_is_passed_over(tmp_path):
     n, kstar = run()
     assert n == 7 and kstar != 12345.0
     assert run()[0] == 0                                  # its own lines are taken
+
+
+# the iteration times behind the choice of the pair-term form are those of a step's
+# iterations: what a launch does once (the resident loop copies its cache rows) is not
+# in them. Two sizes that the resident loop holds, where four iterations with it came
+# out at 1.5 times the time of one; 25% for the clocks of two measurements.
+@pytest.mark.parametrize("n,lanes", [(50, 4), (100, 4)])
+def test_form_costs_are_those_of_an_iteration(n, lanes):
+    import numpy as np
+    d = synth.tgv2d(n, seed=3)
+    make = lambda **over: dt.Simulation(d["cfg"], precision=dt.DTSPH_FP32C, graph=2, lanes=lanes, **over)
+    sim = make()
+    sim.set_state(d["x"], d["v"], d["p"], d["v_prev"])
+    ms = sim.form_stats()["ms"]
+    sim.close()
+    for form in (1, 2):
+        t = {}
+        for k in (8, 48):
+            sim = make(form=form, fixed_iters=k)
+            sim.set_state(d["x"], d["v"], d["p"], d["v_prev"])
+            sim.step(8)
+            sim.sync()
+            t[k] = float(np.median(dt.dtsph_loop_times(sim.ctx, 1, 7)))
+            sim.close()
+        slope = (t[48] - t[8]) / 40
+        assert abs(ms[form] - slope) < 0.25 * slope, (form, ms, slope)
