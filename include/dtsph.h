@@ -320,6 +320,12 @@ int dtsph_get_neighbors(dtsph_ctx *ctx, int64_t i, int64_t *out, int64_t cap, in
 int dtsph_probe_iterate(dtsph_ctx *ctx, int32_t launches, float *ms_per_launch, double *bytes_per_launch,
                         int64_t *pairs);
 
+/* Test entry: the kernels of the context's steps whose choice depends on its size, by
+ * name: the list builder, then the pseudo-time loop (with the pair cache, where
+ * the form is chosen per step); empty before the particles are set. Valid until the
+ * next call or dtsph_destroy. */
+const char *dtsph_step_kernels(const dtsph_ctx *ctx);
+
 /* Device time (ms) of the pseudo-time loop of real steps first .. first+count-1
  * (steps are numbered from 0 since dtsph_set_particles; each must be among the
  * last 256 taken), from CUDA events recorded just before and after the loop of

@@ -79,6 +79,7 @@ _SIGS = [
     ("dtsph_build_neighbors", C.c_int, [_VP]),
     ("dtsph_get_neighbors", C.c_int, [_VP, C.c_int64, _I64P, C.c_int64, _I64P]),
     ("dtsph_probe_iterate", C.c_int, [_VP, C.c_int32, C.POINTER(C.c_float), _DP, _I64P]),
+    ("dtsph_step_kernels", C.c_char_p, [_VP]),
     ("dtsph_tuning", C.c_int, [_VP, C.POINTER(C.c_int32), C.POINTER(C.c_float)]),
     ("dtsph_form_stats", C.c_int, [_VP, C.POINTER(C.c_double), C.POINTER(C.c_float), C.POINTER(C.c_int64),
                                    C.POINTER(C.c_int64), C.POINTER(C.c_int64)]),
@@ -339,6 +340,11 @@ def dtsph_form_stats(ctx):
     _check(ctx, lib().dtsph_form_stats(ctx, C.byref(k), ms, C.byref(a), C.byref(b), C.byref(sw)))
     return {"kstar": k.value, "ms": [float(m) for m in ms], "steps_cache": a.value, "steps_nocache": b.value,
             "steps_switched": sw.value}
+
+
+def dtsph_step_kernels(ctx):
+    """[list builder, pseudo-time loop kernel] of the context's steps."""
+    return lib().dtsph_step_kernels(ctx).decode().split()
 
 
 def dtsph_tuning(ctx):

@@ -76,6 +76,7 @@ struct dtsph_ctx {
     int64_t steps_cache = 0, steps_nocache = 0;   // steps of the other paths
     struct TuneRec { int lanes, stages; float ms; };
     std::vector<TuneRec> tune_log;      // candidates timed by the last tuning
+    std::string kernels;                // dtsph_step_kernels
 };
 
 namespace {
@@ -1750,6 +1751,20 @@ int dtsph_probe_iterate(dtsph_ctx *c, int32_t launches, float *ms_per_launch, do
     if (bytes_per_launch) *bytes_per_launch = bytes;
     if (pairs) *pairs = np;
     return DTSPH_OK;
+}
+
+const char *dtsph_step_kernels(const dtsph_ctx *c_)
+{
+    dtsph_ctx *c = const_cast<dtsph_ctx *>(c_);
+    if (!c || !c->have_particles) return "";
+    const Buffers &B = c->B;
+    ResShape S;
+    c->kernels = nlist_few_cells(B) ? "k_nlist_cells2 " : "k_nlist_home ";
+    if (c->prm[0].graph != 2 || (B.xk[0] && c->ninst > 1)) c->kernels += B.xk[0] ? "k_move_iter" : "k_iterate";
+    else if (B.xk[0]) c->kernels += "k_move_loop";
+    else if (resident_shape(B, &S)) c->kernels += "k_loop_res";
+    else c->kernels += B.async_loop ? "k_loop_async" : "k_loop";
+    return c->kernels.c_str();
 }
 
 int dtsph_form_stats(const dtsph_ctx *c, double *kstar, float *ms, int64_t *steps_cache, int64_t *steps_nocache,

@@ -354,6 +354,7 @@ int launch_scatter_same(const Buffers &B, const double *x, const double *v, cons
 // Neighbour lists of every slot at positions xpos (order of the latest binning);
 // one launch.
 void launch_nlist(const Buffers &B, const double *xpos, cudaStream_t st);
+bool nlist_few_cells(const Buffers &B);   // k_nlist_cells2 builds them, else k_nlist_home
 // The state-n pass at r^n in order B: its lists built first, or (build_lists
 // false) the r^0 lists of the previous step, built with list_skin, as they are.
 int launch_state_n(const Buffers &B, bool predictor, cudaStream_t st, bool build_lists = true);

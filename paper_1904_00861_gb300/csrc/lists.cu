@@ -516,15 +516,16 @@ __global__ void __launch_bounds__(kListWarps * kWarp) k_nlist_home(Buffers B, co
 
 static_assert(list_stride(1) % 4 == 0, "a list row holds whole 16-byte stores");
 
+bool nlist_few_cells(const Buffers &B) { return B.dim == 2 && B.nseg2 < kRowsMinSegments; }
+
 // The lists of every slot at xpos (order of the latest binning); one launch.
 void launch_nlist(const Buffers &B, const double *xpos, cudaStream_t st)
 {
     const int Ks = list_stride(B.K);
-    if (B.dim == 2 && B.nseg2 < kRowsMinSegments) {
+    if (nlist_few_cells(B)) {
         const int nb = (B.ncell + kWarpsPerBlock - 1) / kWarpsPerBlock;
         launch_next(B, st, nb, kBlock, k_nlist_cells2, B, xpos, B.pjt, Ks);
-    } else
-    if (B.dim == 2) {
+    } else if (B.dim == 2) {
         const int nb = (B.nseg2 + kListWarps - 1) / kListWarps;
         launch_next(B, st, nb, kListWarps * kWarp, k_nlist_home<2>, B, xpos, B.pjt, Ks);
     } else {
