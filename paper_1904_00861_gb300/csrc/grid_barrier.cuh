@@ -6,6 +6,13 @@
 
 namespace dtsph {
 
+// True when the arrival counter has reached target. Both wrap at 2^32 (steps of several
+// million iterations) and lie less than 2^31 apart.
+__host__ __device__ __forceinline__ bool barrier_reached(unsigned int arrivals, unsigned int target)
+{
+    return (int)(arrivals - target) >= 0;
+}
+
 // Grid barrier for a cooperative launch (all blocks resident): arrival counter
 // `bar`, reset to 0 before the launch; the epoch-th barrier waits for
 // epoch * gridDim.x arrivals: a release arrival of the block's writes, then polls.
@@ -27,7 +34,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned int *bar, unsigned int epo
             unsigned int v;
             if (ALONE) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
             else asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-            if (v >= target) break;
+            if (barrier_reached(v, target)) break;
             // (the clock every 64 polls: reading it costs more than a poll)
             if (limit_ns == 0 || (++polls & 63) == 0) {
                 const unsigned long long now = globaltimer_ns();
