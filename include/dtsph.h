@@ -137,7 +137,9 @@ typedef struct {
                                  1: over the neighbour lists of r^0; 2: neighbours updated at
                                  every pass (lists with the cutoff 3h + skin; a particle that
                                  moves farther than skin/2 from r^0 ends the step with
-                                 DTSPH_E_SKIN). Not with steady. With graph = 2 a batch runs the
+                                 DTSPH_E_SKIN). Not with steady. With graph = 2 one instance
+                                 runs the persistent kernel (so its step can end with
+                                 DTSPH_E_TIMEOUT, as other steps with graph = 2), a batch the
                                  loop as in graph = 1. Instances of a batch share it. */
     int32_t form;             /* the pair terms of the pseudo-time loop. 1: from the pair-
                                  coefficient cache, written once per real step by a pass over

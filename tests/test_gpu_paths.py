@@ -2,7 +2,8 @@
 loop at the largest square that fits one block per SM and at the next one, for every
 number of lanes, with walls and in 3D (bits against the launch-per-iteration graph);
 the list builder of many segments with closed axes, walls, crowded cells and several
-instances (sets against the oracle), and its rows cut at the capacity.
+instances (sets against the oracle), and its rows cut at the capacity; the barrier of
+every persistent loop giving up.
 """
 import numpy as np
 import pytest
@@ -145,3 +146,30 @@ def test_a_cut_list_is_reported(nx, kernel, prec):
     sim.set_state(d["x"], d["v"], d["p"])
     check_lists(sim.ctx, [d], 300)
     sim.close()
+
+
+@pytest.mark.parametrize("prec", [F64, F32])
+@pytest.mark.parametrize("case,over,kernel", [
+    ("tgv2d", dict(moving=1), "k_move_loop"), ("cavity2d", dict(moving=2), "k_move_loop"),
+    ("tgv2d", dict(form=1), "k_loop_res"), ("cavity2d", dict(), "k_loop_res")])
+def test_a_barrier_that_gives_up_ends_the_step_with_a_status(monkeypatch, case, over, kernel, prec):
+    """A give-up time of zero: every persistent loop ends its step early and dtsph_sync says
+    DTSPH_E_TIMEOUT; a context without the setting runs the same state to its end."""
+    d = getattr(synth, case)(60)
+    nf = d["nf"]
+    walls = None if d["vw"] is None else (d["x"][nf:], d["vw"])
+    monkeypatch.setenv("DTSPH_TEST_BARRIER_WAIT_NS", "0")
+    for give_up in (True, False):
+        sim = dt.Simulation(d["cfg"], precision=prec, graph=2, lanes=2, max_iter=60, **over)
+        sim.set_state(d["x"][:nf], d["v"], d["p"], d["v_prev"], walls=walls)
+        assert dt.dtsph_step_kernels(sim.ctx)[1] == kernel
+        sim.step(1)
+        if give_up:
+            with pytest.raises(dt.DtsphError) as e:
+                sim.sync()
+            assert e.value.code == dt.DTSPH_E_TIMEOUT
+        else:
+            sim.sync()
+            assert sim.stats()[0]["reason"] in (0, 1, 2)
+        sim.close()
+        monkeypatch.delenv("DTSPH_TEST_BARRIER_WAIT_NS", raising=False)
