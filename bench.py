@@ -498,12 +498,21 @@ def loop_launch_bytes(dims, fp32c, form, pairs_per_particle, nfs, iters, kstar):
 
 
 def fp64_flops(dim):
-    """FP64 flops (FMA = 2) of the FP64 pseudo-iteration, counted from the pair
+    """FP64 flops (FMA = 2) of the FP64 pseudo-iteration as the equations state the pair
     terms (EDAC on, no artificial viscosity): per cached pair the divergence
     and EDAC terms of dp/dtau and the pressure and viscous terms of F,
     8 dim + 9; per fluid particle the BDF2 pseudo-acceleration, the update and
     the residual terms, 8 dim + 3."""
     return 8.0 * dim + 3.0, 8.0 * dim + 9.0
+
+
+def fp64_flops_done(dim):
+    """The same as the kernels evaluate it, with the constants outside the sums: per
+    cached pair dim velocity differences, the pressures' difference and sum, an
+    FMA for each component of three sums and one for the EDAC sum: 7 dim + 4 in 4 dim
+    + 3 instructions (so a full pipe shows as (7 dim + 4) / (8 dim + 6) of the FMA
+    peak)."""
+    return fp64_flops(dim)[0], 7.0 * dim + 4.0
 
 
 def measure_peaks(dt):
@@ -576,9 +585,10 @@ def main_ours(args):
         v64 = sim64.velocities()
         ms_it64, bytes_it64, npairs64 = dt.dtsph_probe_iterate(sim64.ctx, 20)
         lanes64, _ = dt.dtsph_tuning(sim64.ctx)
+        loop_name64 = dt.dtsph_step_kernels(sim64.ctx)[1]
         # the FP64 loop is bound by the FP64 pipe: algorithmic FP64 flops of the
         # timed loops over their device time, against the measured FP64 FMA peak
-        f_part, f_pair = fp64_flops(dims)
+        f_part, f_pair = fp64_flops_done(dims)
         w64, lms64, _, _ = loop64
         flops64 = float(np.sum(w64)) * (f_part + f_pair * npairs64 / nf_tot)
         ach64 = flops64 / (sum(lms64) * 1e-3) / 1e12
@@ -586,11 +596,13 @@ def main_ours(args):
                 "iterate_kernel_ms": ms_it64, "speedup_fp32c_over_fp64": value / (rate64 * world),
                 "roofline": {"bound": "alu", "pipe": "fp64", "achieved": ach64, "peak": fma["fp64_fma_tflops"],
                              "unit": "TFLOP/s", "frac": ach64 / fma["fp64_fma_tflops"],
-                             "kernel": f"{'k_loop_async' if decoupled else 'k_loop'}<{dims},FP64,lanes={lanes64}>",
+                             "kernel": f"{loop_name64}<{dims},FP64,lanes={lanes64}>",
                              "flops_per_launch": flops64 / len(lms64), "launch_ms": sum(lms64) / len(lms64),
                              "flops_counted": f"{f_part:.0f} per particle-iteration + {f_pair:.0f} per pair-iteration "
                                               f"(FMA = 2; the pair terms as the cached form evaluates them, "
-                                              f"whichever form ran), {npairs64 / nf_tot:.2f} pairs per particle",
+                                              f"{4 * dims + 3} instructions a pair, whichever form ran; as the "
+                                              f"equations state them {fp64_flops(dims)[1]:.0f}), "
+                                              f"{npairs64 / nf_tot:.2f} pairs per particle",
                              "peak_source": "dtsph_fma_peak(FP64), measured in this run"}}
         sim64.close()
     # the dominant kernel of the timed steps is the pseudo-time loop: its
@@ -606,7 +618,8 @@ def main_ours(args):
     achieved = loop_bytes / (sum(loop_ms) * 1e-3) / 1e9
     probe_bytes = STATE_BYTES[(dims, True)] * nf_tot + PAIR_BYTES[(dims, True)] * npairs
     achieved_probe = probe_bytes / (ms_it * 1e-3) / 1e9
-    loop_kernel = {2: f"k_loop or k_loop_res<{dims},FP32C,lanes={lanes32}> (persistent loop, one launch per step)",
+    loop_name = dt.dtsph_step_kernels(sim32.ctx)[1]
+    loop_kernel = {2: f"{loop_name}<{dims},FP32C,lanes={lanes32}> (persistent loop, one launch per step)",
                    1: f"k_iterate<{dims},FP32C,lanes={lanes32}> in the while node (one launch per iteration)",
                    0: f"k_iterate<{dims},FP32C,lanes={lanes32}> (plain launches)"}[args.graph]
     if decoupled:
