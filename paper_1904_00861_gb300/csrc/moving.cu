@@ -463,7 +463,10 @@ __global__ void __launch_bounds__(kBlock, F32 ? 2 : 1) k_move_loop(Buffers B)
     for (;; ++it) {
         const int cur = it & 1;
         if constexpr (WALLS) {
-            for (int w = blockIdx.x * kBlock + threadIdx.x; w < B.nw; w += gridDim.x * kBlock)
+            // the wall list's warps dealt to the blocks in turn (eight to a block, the FP64
+            // sums of 3,000 walls kept 12 SMs busy: @@)
+            for (int w = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * kWarp + (threadIdx.x & 31); w < B.nw;
+                 w += (kBlock / kWarp) * gridDim.x * kWarp)
                 move_wall<D, F32>(B, G, P, cur, B.wslot_a[w]);
             if (!grid_barrier<false>(&B.ctrl->bar, ++epoch, B.err, ok_sh, B.barrier_ns)) break;
         }
