@@ -102,14 +102,14 @@ __device__ __forceinline__ void wall_slot(const Buffers &B, int s, int cur, int 
         for (int t = 0; t < D + 2; ++t) acc[t] += __shfl_xor_sync(gmask, acc[t], o);
     // FP64 instructions are what this phase takes, and every lane has the sums: lane 0
     // divides for p_w, lanes 1 to D for a component of the ghost velocity, so the warp
-    // issues one division (five steps of a dam break of 20,402 particles 3.98 ms, 4.26 ms
-    // with lane 0 dividing for all)
+    // issues one division (five steps of a dam break of 20,402 particles 3.93 ms; 3.98 ms with
+    // CUDA's division, 4.26 with lane 0 dividing for all by it)
     if (sub > 3) return;
     double num = acc[1];
 #pragma unroll
     for (int a = 0; a < D; ++a)
         if (sub == 1 + a) num = acc[2 + a];
-    double v = acc[0] > 0 ? num / acc[0] : 0.0;
+    double v = acc[0] > 0 ? quotient(num, acc[0]) : 0.0;
     if (sub == 0) {
         if (v < 0.0 && B.phys[B.inst_of[s]].free_surface) v = 0.0;   // free-surface runs (Sec. 3.2)
     } else {
