@@ -52,14 +52,22 @@ UNIT = "particle-iterations/s"
 # bytes per algorithmic byte of the form it ran times its own algorithmic bytes.
 # A variant not listed (a step that switched forms included), or one whose
 # kernel changed after its capture, reports null.
-# (Empty: the loop kernels changed after the committed captures.)
-NCU_TRAFFIC = {}
+_BATCH_TRAFFIC = "profiles/traffic_batch64_tgv2d.md"
+NCU_TRAFFIC = {
+    ("batch-64x-tgv2d", 2, 1, 2, 1): (6.077598e9 + 0.203470e9, 6.985625e9, _BATCH_TRAFFIC),
+    ("batch-64x-tgv2d", 2, 1, 3, 1): (6.170196e9 + 0.211839e9, 6.985625e9, _BATCH_TRAFFIC),
+    ("batch-64x-tgv2d", 2, 1, 4, 1): (6.191082e9 + 0.214370e9, 6.985625e9, _BATCH_TRAFFIC),
+    ("batch-64x-tgv2d", 2, 1, 6, 1): (6.247166e9 + 0.221759e9, 6.985625e9, _BATCH_TRAFFIC),
+    # (without the cache the staging depth has no part)
+    **{("batch-64x-tgv2d", 2, 1, stages, 2): (1.937722e9 + 0.341515e9, 2.520798e9, _BATCH_TRAFFIC)
+       for stages in (2, 3, 4, 6)},
+}
 
 # FP32 flops of the loop without the pair cache, from the FP32 operation counters
 # of an Nsight Compute capture (fadd + fmul + 2 ffma, thread instructions):
 # dim -> (flops per pair-iteration, workload, source). The form is bound by
 # neither HBM nor the FP32 pipe; this places its launches against the FP32 peak.
-# (Empty for the same reason: the packed arithmetic changed the operation counts.)
+# (Empty: the packed arithmetic changed the operation counts after the committed captures.)
 NCU_FLOPS_NO_CACHE = {}
 
 

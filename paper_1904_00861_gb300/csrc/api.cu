@@ -252,7 +252,6 @@ void dtsph::make_phys(const dtsph_params &p, Phys &P)
     P.dtau_f = (float)P.dtau;
     P.sig_h = quintic_sigma(p.dim, p.h) / p.h;
     P.eta_h2 = p.eta * p.h * p.h;
-    P.edac_h2 = P.eta_h2;
     const double rho = p.rho0;
     P.c_div = p.m * (rho / rho) * P.c * P.c;
     P.c_edac = 4.0 * p.m / ((rho + rho) * rho) * P.nu_e;
@@ -261,8 +260,7 @@ void dtsph::make_phys(const dtsph_params &p, Phys &P)
     P.c_av = p.alpha * p.h * P.c / rho;
     for (int a = 0; a < 3; ++a) P.g[a] = a < p.dim ? p.g[a] : 0.0;
     P.kappa = 2.0 * p.dt / (2.0 * p.dt + 3.0 * P.dtau);
-    P.c3 = 3.0 / (2.0 * p.dt);
-    P.kc3 = P.kappa * P.c3;
+    P.kc3 = P.kappa * (3.0 / (2.0 * p.dt));
     P.inv_h = 1.0 / p.h;
     P.inv_2dt = 1.0 / (2.0 * p.dt);
     P.edac = p.edac;

@@ -50,15 +50,6 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t by
                  : "memory");
 }
 
-// Bulk copy of `bytes` from global src to shared dst, completion on bar.
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_addr(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_addr(bar))
-                 : "memory");
-}
-
 // L2 eviction-priority policies for the cache_hint forms below: data read once
 // per pass that should leave L2 first (the pair-cache stream), and data that
 // should stay (the neighbour states every pass gathers again).
@@ -83,7 +74,8 @@ __device__ __forceinline__ uint64_t l2_policy_evict_last()
     return p;
 }
 
-// bulk_g2s with an L2 eviction policy for the copied lines.
+// Bulk copy of `bytes` from global src to shared dst, completion on bar, with an L2
+// eviction policy for the copied lines.
 __device__ __forceinline__ void bulk_g2s_hint(void *dst, const void *src, uint32_t bytes, uint64_t *bar,
                                               uint64_t policy)
 {

@@ -50,7 +50,7 @@ constexpr unsigned long long kBarrierWaitNs = 1000000000ull;   // grid-barrier g
 constexpr int kDealMaxInst = 1024;
 
 constexpr int kPassWaveBlocksPerSm = 8;   // blocks per SM of a grid-stride pass that a graph may skip
-constexpr int kSeg2 = 3;   // cells along x in one row segment of the 2D FP32C list builder
+constexpr int kSeg2 = 3;   // cells along x in one row segment of the 2D list builder
 
 struct Inst {
     int slot_off;          // first slot
@@ -59,7 +59,7 @@ struct Inst {
     int cell_off;          // first cell; the instance owns ncell + 1 cells, the last one
                            // always empty so that its start marks the end of the range
     int shift;             // slot_off minus the particles of the instances before it
-    int seg_off;           // first row segment of the 2D FP32C list builder (kSeg2 cells along x)
+    int seg_off;           // first row segment of the 2D list builder (kSeg2 cells along x)
 };
 
 // Cell grid and neighbour-test constants of one binning. Cells have side
@@ -100,7 +100,6 @@ struct Phys {
     double h, m, rho0, c, nu, nu_e, dt, dtau;
     double sig_h;        // sigma / h: dW/dr = sig_h * dWdq(q)
     double eta_h2;       // eta h^2 (viscous and artificial-viscosity denominators)
-    double edac_h2;      // eta h^2, or h^2 for the literal reading
     double c_div;        // m (rho_i / rho_j) c^2                       divergence term
     double c_edac;       // 4 m nu_e / ((rho_i + rho_j) rho_j)           EDAC term
     double c_p;          // m / rho0^2                                  pressure term
@@ -108,7 +107,6 @@ struct Phys {
     double c_av;         // alpha h c / rho0                            artificial viscosity
     double g[3];
     double kappa;        // 2 dt / (2 dt + 3 dtau), Eq. (dv_dtau_exact)
-    double c3;           // 3 / (2 dt)
     double kc3;          // kappa * 3 / (2 dt)
     double inv_h;        // 1 / h
     double inv_2dt;      // 1 / (2 dt)
@@ -182,7 +180,7 @@ constexpr int kStatRing = 65536;   // real steps kept per instance
 struct Buffers {
     int n;                          // slots (all instances, padding included)
     int nf, nw;                     // fluid and wall particles of all instances
-    int nseg2;                      // row segments of the 2D FP32C list builder, all instances
+    int nseg2;                      // row segments of the 2D list builder, all instances
     int nsm;                        // streaming multiprocessors of the device
     int l2_stream;                  // 1: the pair cache exceeds half of L2 (its rows stream, evicting first)
     int reuse_lists;                // 1: the r^0 lists (with list_skin) serve the next step at r^n

@@ -227,15 +227,16 @@ constexpr int kRowsMinSegments = 16384;
 //    after the other. The particle's mask word says which lanes write, the bits
 //    before a lane's own where, so every hit costs the warp nothing beyond its
 //    particle's word and the hits of a chunk leave as one contiguous run. (Each
-//    lane walking the bits of its own words: 1.5 ms against 1.1 ms a build at
-//    128^3, the lanes out of step.)
+//    lane walking the bits of its own words: 1.4 times as long at 128^3, the
+//    lanes out of step.)
 // For every particle the candidates of its own 3^D cells come in the order of
 // k_nlist_cells2; the FP32 separation o_i - (o_j + shift s) decides outside the
 // band as the canonical form does, so sets and order are the same on every path.
 // The FP64 path takes the same pre-test (its offsets are kept for it): FP64 tests
 // of every candidate run at 1/64 of the rate (45^3: 3.7 ms a build, now 0.1 ms).
 // Against the builders with a per-hit append by the home particle's lane: 128^3
-// 2.04 ms a build, now 1.1 ms; the 64-vortex batch 0.37 ms, now 0.24 ms.
+// 2.04 ms a build, now 0.85 ms; the 64-vortex batch 0.37 ms, now 0.24 ms. 61^3: 0.14 ms,
+// 96 M warp instructions, 69% of the issue slots.
 constexpr int kListWarps = 4;                 // warps per block
 constexpr int kStage = 256;                   // staged candidates per warp
 

@@ -1,8 +1,9 @@
 // The pair terms of the FP32C path, two neighbours of a particle at a time.
 //
 // With one neighbour at a time the kernels that sum over neighbour lists were bound
-// by instruction issue (59-66% of the issue slots busy with no pipe near its
-// peak: 129 instructions a pair in the 3D state-n pass, 56 now), so the arithmetic of two
+// by instruction issue (59-66% of the issue slots busy with no pipe near its peak: 111 M
+// warp instructions in the state-n pass of 61^3 particles, 54 M so; 74 M and 48% of the
+// slots with the lanes shared, see warp_rates32), so the arithmetic of two
 // list entries runs in the packed single-precision instructions (add, sub, mul and
 // fma .f32x2: two IEEE-rounded results per issue). Entries 2m and 2m + 1 of a list
 // form pair m; the even and the odd entries have their own Kahan-compensated sums,
@@ -206,8 +207,8 @@ __device__ __forceinline__ void rates32(const PairK32 &k, const Sums32<D> &A, fl
 // Displacement of the home offset for every shift code, by component, in shared
 // memory: o_i moves by minus the cell shift (a particle's own code, 13, by zero). The
 // codes of a warp's entries differ, and 32 words by component lie in 32 banks: one
-// wavefront a component (records of 16 bytes: the 128^3 loop without the cache 1.23
-// ms an iteration, so 1.20 ms).
+// wavefront a component (records of 16 bytes: 2.5% more time in the 128^3 loop
+// without the cache).
 constexpr int kCodes = 32;
 struct ShiftTable {
     float c[3][kCodes];
@@ -292,9 +293,8 @@ __device__ __forceinline__ void list_sums32(const PairK32 &k, const ShiftTable &
 // The rates of a warp's 32 slots (s: the lane's own, cnt its list's length, 0 if it
 // has no rates to form), G lanes to a slot: the warp takes 32 / G slots at a time,
 // so that a gather's 32 entries are G neighbours in a row of each of them and fall
-// on fewer lines: the L1 looks up one line a cycle, and one lane per slot puts
-// the entries of a 3D gather on 17 lines, eight lanes on 10 (2D: 8.5, four lanes
-// 5). A slot's sums then come back to its own lane. sums(slot, lane of the slot,
+// on fewer lines: the L1 looks up one line a cycle. Tag lookups a load, by counter at
+// 61^3: 17.5 with one lane per slot (the loop without the cache), 8.3 with eight. A slot's sums then come back to its own lane. sums(slot, lane of the slot,
 // count, V_i, p_i, A) adds the pairs.
 template <int D, int G, typename SUMS>
 __device__ __forceinline__ void warp_rates32(const PairK32 &k, int s, int cnt, const float4 *nb, SUMS sums, float &ap,

@@ -114,7 +114,6 @@ struct Plain64 {
     __device__ __forceinline__ Plain64() : s(0.0) {}
     __device__ __forceinline__ void add(double v) { s += v; }
     __device__ __forceinline__ double value() const { return s; }
-    __device__ __forceinline__ void shfl_merge(int lane_mask) { s += __shfl_xor_sync(0xffffffffu, s, lane_mask); }
 };
 
 // Constants of a pair's FP64 terms.
