@@ -1041,15 +1041,16 @@ int probe_loop_ms(dtsph_ctx *c, int iters, int reps, float *out)
 // The loop's time per iteration, and what a launch takes beside its iterations. The
 // resident loop copies its cache rows to shared memory once a launch (2 to 25 us
 // beside a launch's own 8), which four iterations do not spread as the 7 to 50 of a
-// step do: 100 x 100 FP32C 8.1 us an iteration over four, 5.5 by the slope. `slope`:
-// from launches of 4 and of 16 iterations; else four, and nothing beside them.
-int probe_iteration_ms(dtsph_ctx *c, bool slope, int reps, float *per_iter, float *beside)
+// step do: 100 x 100 FP32C 8.1 us an iteration over four, 5.5 by the slope. From
+// launches of 4 and of `more` iterations; with more = 0 from four, and nothing beside.
+int probe_iteration_ms(dtsph_ctx *c, int more, float *per_iter, float *beside)
 {
-    float t4 = 0, t16 = 0;
+    const int reps = more ? 2 : 5;
+    float t4 = 0, tm = 0;
     int r = probe_loop_ms(c, 4, reps, &t4);
-    if (!r && slope) r = probe_loop_ms(c, 16, reps, &t16);
+    if (!r && more) r = probe_loop_ms(c, more, reps, &tm);
     if (r) return r;
-    *per_iter = slope && t16 > t4 ? (t16 - t4) / 12.f : t4 / 4.f;
+    *per_iter = more && tm > t4 ? (tm - t4) / (float)(more - 4) : t4 / 4.f;
     *beside = std::max(0.f, t4 - 4.f * *per_iter);
     return DTSPH_OK;
 }
@@ -1097,17 +1098,24 @@ int autotune(dtsph_ctx *c)
     for (int L : {2, 4, 8}) cand.push_back({L, kDefaultStages});
     TuneChoice best{c->B.lanes, c->B.stages};
     float best_ms = 1e30f;
-    // (over as many iterations as a step takes where a launch has a cost of its own)
-    const int iters = fits_resident(B) ? 16 : 4;
+    // where a launch has a cost of its own, over as many iterations as a step takes, and
+    // one lane once: the resident loop has no staging depth
+    const bool res = fits_resident(B);
+    const int iters = res ? 16 : 4, reps = res ? 2 : 5;
+    float one_lane = -1.f;
     c->tune_log.clear();
     for (const TuneChoice &ch : cand) {
         c->B.lanes = ch.lanes;
         c->B.stages = ch.stages;
         float ms = 0;
         int r;
-        if (c->prm[0].graph == 2) {
-            r = probe_loop_ms(c, iters, 5, &ms);
+        if (c->prm[0].graph == 2 && res && ch.lanes == 1 && one_lane >= 0.f) {
+            r = DTSPH_OK;
+            ms = one_lane;
+        } else if (c->prm[0].graph == 2) {
+            r = probe_loop_ms(c, iters, reps, &ms);
             ms /= (float)iters;
+            if (ch.lanes == 1) one_lane = ms;
         } else {
             probe_ms(c, c->B, 3, &ms);         // warm-up
             r = probe_ms(c, c->B, 10, &ms);
@@ -1183,10 +1191,10 @@ int measure_form_costs(dtsph_ctx *c)
     float ms_b = 0, ms_a = 0, beside_b = 0, beside_a = 0;
     B.form_a = 0;
     const bool slope = fits_resident(B);
-    int r = probe_iteration_ms(c, slope, 5, &ms_b, &beside_b);
+    int r = probe_iteration_ms(c, slope ? 16 : 0, &ms_b, &beside_b);
     if (!r) {
         B.form_a = 1;
-        r = probe_iteration_ms(c, slope, 5, &ms_a, &beside_a);
+        r = probe_iteration_ms(c, slope ? 8 : 0, &ms_a, &beside_a);   // (the slower one)
         B.form_a = 0;
     }
     if (r) return r;
