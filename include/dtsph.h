@@ -355,9 +355,9 @@ int dtsph_tuning(const dtsph_ctx *ctx, int32_t *lanes, float *ms_by_lanes);
 
 /* Every candidate the autotuner timed when this context tuned, in the order
  * timed: lanes per particle, staging depth (0 for lanes > 1) and mean ms per
- * launch of the pseudo-iteration kernel (graph = 0, 1) or per iteration of the
- * persistent loop kernel over four fixed iterations, 16 where the problem fits the
- * resident loop (graph = 2). Writes min(cap, count) entries of the three arrays (each may be NULL when cap is 0); *count = candidates timed
+ * launch of the pseudo-iteration kernel (graph = 0, 1) or ms per iteration of the
+ * fastest of a few launches of the persistent loop kernel over four fixed iterations,
+ * 16 where the problem fits the resident loop (graph = 2). Writes min(cap, count) entries of the three arrays (each may be NULL when cap is 0); *count = candidates timed
  * (0 when the shape's choice came from the process cache or lanes was fixed);
  * *stages = staging depth in use (0 when lanes > 1). */
 int dtsph_tuning_candidates(const dtsph_ctx *ctx, int32_t cap, int32_t *lanes, int32_t *stages, float *ms,

@@ -1003,9 +1003,10 @@ int probe_ms(dtsph_ctx *c, const Buffers &B, int launches, float *out)
     return DTSPH_OK;
 }
 
-// Mean device time of a launch of the persistent loop kernel with `iters` iterations
+// Least device time of a launch of the persistent loop kernel with `iters` iterations
 // of every instance (fixed_iters forced on the loop state for the probe, then
-// restored), `reps` launches after one untimed launch.
+// restored), of `reps` launches after one untimed launch (the least: a host that is held
+// up between the events shows as device time).
 int probe_loop_ms(dtsph_ctx *c, int iters, int reps, float *out)
 {
     const Buffers &B = c->B;
@@ -1019,7 +1020,7 @@ int probe_loop_ms(dtsph_ctx *c, int iters, int reps, float *out)
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
-    float tot = 0;
+    float least = 1e30f;
     for (int i = 0; i <= reps; ++i) {
         launch_loop_reset(B, c->stream);
         CK(cudaEventRecord(e0, c->stream));
@@ -1028,13 +1029,13 @@ int probe_loop_ms(dtsph_ctx *c, int iters, int reps, float *out)
         CK(cudaEventSynchronize(e1));
         float ms = 0;
         CK(cudaEventElapsedTime(&ms, e0, e1));
-        if (i > 0) tot += ms;
+        if (i > 0) least = std::min(least, ms);
     }
     c->launches += 2 * (reps + 1);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     CK(cudaMemcpy(B.ls, saved.data(), sizeof(LoopState) * c->ninst, cudaMemcpyHostToDevice));
-    *out = tot / (float)reps;
+    *out = least;
     return DTSPH_OK;
 }
 
