@@ -403,8 +403,8 @@ int dtsph_form_stats(const dtsph_ctx *ctx, double *kstar, float *ms, int64_t *st
  *              (nf x dim), in the caller's particle order
  *   status     optional device int32 (may be NULL): after the call's GPU work it
  *              holds DTSPH_OK, DTSPH_E_CAPACITY (a particle had more neighbours
- *              than the neighbour capacity; its list was cut there and its rates
- *              are wrong) or DTSPH_E_DOMAIN (a particle lay outside the box of a
+ *              than the neighbour capacity; its list was cut there, or left
+ *              empty, and its rates are wrong) or DTSPH_E_DOMAIN (a particle lay outside the box of a
  *              non-periodic axis)
  *   stream     cudaStream_t or NULL; it must belong to the current device. The
  *              call only enqueues work and returns.
