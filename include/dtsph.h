@@ -357,8 +357,9 @@ int dtsph_tuning(const dtsph_ctx *ctx, int32_t *lanes, float *ms_by_lanes);
  * timed: lanes per particle, staging depth (0 for lanes > 1) and mean ms per
  * launch of the pseudo-iteration kernel (graph = 0, 1) or ms per iteration of the
  * fastest of a few launches of the persistent loop kernel over four fixed iterations,
- * 16 where the problem fits the resident loop (graph = 2). Writes min(cap, count) entries of the three arrays (each may be NULL when cap is 0); *count = candidates timed
- * (0 when the shape's choice came from the process cache or lanes was fixed);
+ * 16 where the problem fits the resident loop (graph = 2). Writes min(cap, count)
+ * entries of the three arrays (each may be NULL when cap is 0); *count = candidates
+ * timed (0 when the shape's choice came from the process cache or lanes was fixed);
  * *stages = staging depth in use (0 when lanes > 1). */
 int dtsph_tuning_candidates(const dtsph_ctx *ctx, int32_t cap, int32_t *lanes, int32_t *stages, float *ms,
                             int32_t *count, int32_t *stages_in_use);
@@ -404,8 +405,8 @@ int dtsph_form_stats(const dtsph_ctx *ctx, double *kstar, float *ms, int64_t *st
  *   status     optional device int32 (may be NULL): after the call's GPU work it
  *              holds DTSPH_OK, DTSPH_E_CAPACITY (a particle had more neighbours
  *              than the neighbour capacity; its list was cut there, or left
- *              empty, and its rates are wrong) or DTSPH_E_DOMAIN (a particle lay outside the box of a
- *              non-periodic axis)
+ *              empty, and its rates are wrong) or DTSPH_E_DOMAIN (a particle lay
+ *              outside the box of a non-periodic axis)
  *   stream     cudaStream_t or NULL; it must belong to the current device. The
  *              call only enqueues work and returns.
  * All work happens in one fixed scratch array of about 18 MB that is part of the

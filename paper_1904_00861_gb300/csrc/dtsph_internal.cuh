@@ -305,11 +305,11 @@ __device__ __forceinline__ void grid_start()
 // parameter that points at what a launch before it in the chain writes: such a parameter
 // says that the data stays as it is from the kernel's start, and the kernel starts
 // while they run (its loads may move up past grid_start, or take the path that is not
-// coherent with other kernels' writes). With B.chain, whose launch before on the stream is such a kernel too, the
-// launches overlap: the 8 launches of the allocation-free rates of 1,024 FP64 particles
-// take 52 instead of 66 us, of 12,167 FP32C particles 142 instead of 147. The step
-// graph goes without: 10 steps of 200 x 200 particles took 2,417 us with such edges,
-// 2,284 us without.
+// coherent with other kernels' writes). With B.chain, whose launch before on the
+// stream is such a kernel too, the launches overlap: the 8 launches of the
+// allocation-free rates of 1,024 FP64 particles take 52 instead of 66 us, of 12,167
+// FP32C particles 142 instead of 147. The step graph goes without: 10 steps of 200 x
+// 200 particles took 2,417 us with such edges, 2,284 us without.
 template <typename... P, typename... A>
 inline void launch_next(const Buffers &B, cudaStream_t st, int grid, int block, void (*kernel)(P...), A... args)
 {
